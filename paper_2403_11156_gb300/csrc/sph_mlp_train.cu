@@ -1,18 +1,20 @@
 // sph_mlp_train.cu -- training of the warm-start network on the GPU: forward and backward
 // of the mean-squared error on tcgen05 tensor cores (BF16 operands, FP32 accumulation in
 // tensor memory), Adam updates of the FP32 master weights, and the feature / label
-// standardisation statistics.  Per CTA, 128 samples:
+// standardisation statistics.  Per tile of 128 samples:
 //   forward   D1 = F W1^T, a1 = gelu(z1);  D2 = a1 W2^T, a2 = gelu(z2);  y = a2 . W3 + b3
 //   backward  dy = 2 (y - t) / B;  delta2 = dy W3 gelu'(z2);  D3 = delta2 W2 (-> delta1)
-//             dW2 = delta2^T a1 and dW1 = delta1^T F as MMAs over the sample dimension
-//             (the 64 weight rows padded to the 128-row MMA shape)
-// Gradients are accumulated across CTAs with FP32 atomics (training does not need a
-// bit-reproducible order); the loss sum in FP64.
+//             [delta2 | delta1]^T [a1 | F] as one MMA over the sample dimension: rows 0-63 x
+//             columns 0-63 are dW2, rows 64-127 x columns 64-67 are dW1
+// A CTA walks its tiles with the weight gradients accumulating in tensor memory and the
+// vector gradients in registers, and adds them to the result once, with FP32 atomics
+// (training does not need a bit-reproducible order); the loss sum in FP64.
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
 #include "sph.h"
+#include "sph_gelu.cuh"
 #include "sph_internal.cuh"
 #include "sph_tc.cuh"
 
@@ -36,30 +38,31 @@ constexpr int kOffSdY = kOffMuY + 1;
 static_assert(kOffSdY + 1 == SPH_MLP_PARAMS, "parameter block layout");
 static_assert(kNW == SPH_MLP_WEIGHTS, "weight count");
 
-// shared-memory map (bytes); every operand tile starts on a 1 KB boundary
-constexpr uint32_t kA1 = 0;          // 128 x 16   features (samples x k)
-constexpr uint32_t kB1 = 4096;       // 64 x 16    W1
-constexpr uint32_t kA2 = 8192;       // 128 x 64   a1 (samples x k)
-constexpr uint32_t kB2 = 24576;      // 64 x 64    W2 (o x k)
-constexpr uint32_t kB2T = 32768;     // 64 x 64    W2^T (k x o)
-constexpr uint32_t kAD2 = 40960;     // 128 x 64   delta2 (samples x o)
-constexpr uint32_t kAD2T = 57344;    // 128 x 128  delta2^T (o x samples), rows 64.. zero
-constexpr uint32_t kBA1T = 90112;    // 64 x 128   a1^T (k x samples)
-constexpr uint32_t kAD1T = 106496;   // 128 x 128  delta1^T (k x samples), rows 64.. zero
-constexpr uint32_t kBFT = 139264;    // 16 x 128   F^T (k x samples), rows 4.. zero
-constexpr uint32_t kVec = 143360;    // b1, b2, w3 (float[64] each)
-constexpr uint32_t kRed = 144128;    // reductions: dW3[64], db2[64], db1[64], db3, loss
-constexpr uint32_t kBar = 145152;
-constexpr uint32_t kTmemSlot = 145160;
-constexpr uint32_t kSmem = 146 * 1024;
-constexpr uint32_t kCols = 256;
+// shared-memory map (bytes) of one CTA.  Both operand tiles keep a sample's row of columns
+// contiguous in core matrices of 8 samples x 8 columns, so the same bytes serve as a
+// K-major operand (K = columns: the layers) and as an M/N-major one (K = samples: the weight
+// gradients), without a transposed copy.
+constexpr int kThreads = 256;          // two threads a row, 32 columns each
+constexpr uint32_t kColsD = 128;       // delta tile: delta2 | delta1
+constexpr uint32_t kColsA = 80;        // activation tile: a1 | F (4 features, 12 zeros)
+constexpr uint32_t kSmD = 0;                               // 128 x 128
+constexpr uint32_t kSmA = kSmD + 128 * kColsD * 2;         // 128 x 80
+constexpr uint32_t kSmW1 = kSmA + 128 * kColsA * 2;        // 64 x 16  W1 (o x f)
+constexpr uint32_t kSmW2 = kSmW1 + 64 * 16 * 2;            // 64 x 64  W2 (o x k)
+constexpr uint32_t kSmVec = kSmW2 + 64 * 64 * 2;           // b1 / 2, b2 / 2, w3 (float[64] each)
+constexpr uint32_t kSmY = kSmVec + 3 * 64 * 4;             // two partial outputs a row
+constexpr uint32_t kSmRed = kSmY + 2 * 128 * 4;            // per warp: dW3, db2, db1 of its 32 columns
+constexpr uint32_t kSmSum = kSmRed + 8 * 3 * 32 * 4;       // per warp: db3, and the loss (FP64)
+constexpr uint32_t kSmBar = kSmSum + 8 * 16;
+constexpr uint32_t kSmTmem = kSmBar + 8;
+// requested: caps residency at two CTAs per SM, whose 256 tensor-memory columns each fill
+// the SM's 512
+constexpr uint32_t kSmem = 100 * 1024;
+static_assert(kSmTmem + 4 <= kSmem, "shared-memory map");
+constexpr int kCtasPerSm = 2;
+constexpr uint32_t kCols = 256;        // tensor memory: z1 | z2, later delta2 W2 | gradients
+constexpr uint32_t kColZ2 = 64, kColG = 128;
 constexpr uint32_t kWaitLimit = 1u << 20;
-
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_d(float z)
-{
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * __expf(-0.5f * z * z);
-}
 
 __device__ __forceinline__ uint32_t pack2(float a, float b)
 {
@@ -71,11 +74,6 @@ __device__ __forceinline__ void store8(unsigned char *tile, uint32_t r, uint32_t
     *reinterpret_cast<uint4 *>(tile + tc::tile_offset(r, k0, K)) =
         make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
 }
-__device__ __forceinline__ void store1(unsigned char *tile, uint32_t r, uint32_t k, uint32_t K, float v)
-{
-    *reinterpret_cast<__nv_bfloat16 *>(tile + tc::tile_offset(r, k, K)) = __float2bfloat16_rn(v);
-}
-
 __device__ __forceinline__ void sync_for_mma()
 {
     tc::fence_proxy_async();
@@ -90,196 +88,268 @@ __device__ __forceinline__ int64_t permute(int64_t p, int64_t n, uint64_t a, uin
     return (int64_t)(((uint64_t)p * a + c) % (uint64_t)n);
 }
 
-// Gradient of the batch's mean squared error (standardised features and labels).
-__global__ void __launch_bounds__(128) k_mlp_grad(const float *__restrict__ w, const float4 *__restrict__ F,
-                                                  const float *__restrict__ T, int64_t n, int64_t batch_begin,
-                                                  int64_t batch_size, uint64_t pa, uint64_t pc, float *grad,
-                                                  double *loss, int *err)
+// Sums of 32 columns over the warp's 32 rows: v[k] is this lane's value of column k; lane l
+// gets the sum of column l (recursive halving, 31 shuffles).
+__device__ __forceinline__ float column_sums(float (&v)[32])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float keep = up ? v[k + o] : v[k], give = up ? v[k] : v[k + o];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0];
+}
+
+// grad[0..3] += v (16-byte aligned, or element by element).
+__device__ __forceinline__ void add4(float *g, const float *v, bool vec)
+{
+    if (vec) {
+        asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(g), "f"(v[0]), "f"(v[1]),
+                     "f"(v[2]), "f"(v[3])
+                     : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) atomicAdd(g + k, v[k]);
+    }
+}
+
+// Gradient of the batch's mean squared error (standardised features and labels).  A
+// persistent grid of at most two CTAs per SM walks 128-sample tiles; warps w and w + 4 share
+// the rows of tensor-memory lanes 32 (w mod 4) and take 32 of the 64 columns each.  Bound by
+// the CUDA-core work of 64 x 4 GELU-like terms a sample; the column sums run as 31 shuffles
+// per 32 columns.  200,000 samples: 56 us (86 TFLOP/s), 6,950 us before, when every row added
+// its 192 terms to 192 shared words atomically, each tile added 4.5k weight gradients to
+// memory and the transposed copies of the operands held a CTA at 146 KB.
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+    k_mlp_grad(const float *__restrict__ w, const float4 *__restrict__ F, const float *__restrict__ T, int64_t n,
+               int64_t batch_begin, int64_t batch_size, uint64_t pa, uint64_t pc, float *grad, double *loss, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
-    const int t = threadIdx.x, warp = t >> 5;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kBar);
-    uint32_t *slot = reinterpret_cast<uint32_t *>(sm + kTmemSlot);
-    float *vb1 = reinterpret_cast<float *>(sm + kVec), *vb2 = vb1 + kH, *vw3 = vb2 + kH;
-    float *rw3 = reinterpret_cast<float *>(sm + kRed), *rb2 = rw3 + kH, *rb1 = rb2 + kH, *rb3 = rb1 + kH;
-    float *rloss = rb3 + 1;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int half = warp >> 2, row = t & 127, c0 = 32 * half;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kSmBar);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(sm + kSmTmem);
+    float *vb1 = reinterpret_cast<float *>(sm + kSmVec), *vb2 = vb1 + kH, *vw3 = vb2 + kH;
+    float *ypart = reinterpret_cast<float *>(sm + kSmY);
 
-    const int64_t pos = (int64_t)blockIdx.x * 128 + t;
-    const bool valid = pos < batch_size && batch_begin + pos < n;
-    float f[4] = {0.f, 0.f, 0.f, 0.f};
-    float target = 0.0f;
-    if (valid) {
-        const int64_t s = permute(batch_begin + pos, n, pa, pc);
-        const float4 q = F[s];
-        f[0] = q.x; f[1] = q.y; f[2] = q.z; f[3] = q.w;
-        target = T[s];
-    }
     if (warp == 0) tc::tmem_alloc(slot, kCols);
     if (t == 0) tc::mbar_init(bar, 1);
-    // zero the padded halves and stage the operands
-    for (uint32_t o = t * 16; o < 16384; o += 128 * 16) {
-        *reinterpret_cast<uint4 *>(sm + kAD2T + 16384 + o) = make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4 *>(sm + kAD1T + 16384 + o) = make_uint4(0, 0, 0, 0);
+    const float z8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (t < 128) store8(sm + kSmA, t, kH + 8, kColsA, z8);
+    if (t < kH) {
+        const float u[8] = {w[kOffW1 + 4 * t], w[kOffW1 + 4 * t + 1], w[kOffW1 + 4 * t + 2], w[kOffW1 + 4 * t + 3],
+                            0.f, 0.f, 0.f, 0.f};
+        store8(sm + kSmW1, t, 0, 16, u);
+        store8(sm + kSmW1, t, 8, 16, z8);
+        vb1[t] = 0.5f * w[kOffB1 + t];
+        vb2[t] = 0.5f * w[kOffB2 + t];
+        vw3[t] = w[kOffW3 + t];
     }
-    for (uint32_t o = t * 16; o < 4096; o += 128 * 16) *reinterpret_cast<uint4 *>(sm + kBFT + o) = make_uint4(0, 0, 0, 0);
-    for (int k = t; k < 3 * kH + 2; k += 128) rw3[k] = 0.0f;
-    __syncthreads();
-    {
-        const float z8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float v[8] = {f[0], f[1], f[2], f[3], 0.f, 0.f, 0.f, 0.f};
-        store8(sm + kA1, t, 0, 16, v);
-        store8(sm + kA1, t, 8, 16, z8);
-        for (int k = 0; k < 4; ++k) store1(sm + kBFT, k, t, 128, f[k]);
-        if (t < kH) {
-            float u[8] = {w[kOffW1 + 4 * t], w[kOffW1 + 4 * t + 1], w[kOffW1 + 4 * t + 2], w[kOffW1 + 4 * t + 3],
-                          0.f, 0.f, 0.f, 0.f};
-            store8(sm + kB1, t, 0, 16, u);
-            store8(sm + kB1, t, 8, 16, z8);
-            vb1[t] = w[kOffB1 + t];
-            vb2[t] = w[kOffB2 + t];
-            vw3[t] = w[kOffW3 + t];
-        }
-        for (int idx = t; idx < kH * 8; idx += 128) {
-            const int r = idx >> 3, kc = (idx & 7) * 8;
-            float u[8], ut[8];
+    for (int idx = t; idx < kH * 8; idx += kThreads) {
+        const int r = idx >> 3, kc = (idx & 7) * 8;
+        float u[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                u[q] = w[kOffW2 + r * kH + kc + q];          // W2[r][kc+q]
-                ut[q] = w[kOffW2 + (kc + q) * kH + r];       // W2^T[r][kc+q] = W2[kc+q][r]
-            }
-            store8(sm + kB2, r, kc, kH, u);
-            store8(sm + kB2T, r, kc, kH, ut);
-        }
+        for (int q = 0; q < 8; ++q) u[q] = w[kOffW2 + r * kH + kc + q];
+        store8(sm + kSmW2, r, kc, kH, u);
     }
-    sync_for_mma();
-    const uint32_t tmem = *slot;
+    // the tensor-memory address is read after the first barrier of the walk below
     const uint32_t sb = tc::smem_addr(sm);
-    const uint32_t id64 = tc::idesc_bf16_f32(128, 64), id16 = tc::idesc_bf16_f32(128, 16);
-    const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+    constexpr uint32_t id_layer = tc::idesc_bf16_f32(128, 64);
+    constexpr uint32_t id_layer_t = id_layer | tc::kIdescBMajorN;
+    constexpr uint32_t id_grad = tc::idesc_bf16_f32(128, kColsA) | tc::kIdescAMajorM | tc::kIdescBMajorN;
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    const float b3 = w[kOffB3], inv_b = 1.0f / (float)batch_size;
+    uint32_t tmem = 0, phase = 0;
     bool good = true;
-    uint32_t phase = 0;
     auto wait_mma = [&]() {
         good = tc::mbar_wait_bounded(bar, phase & 1u, kWaitLimit) && good;
         ++phase;
         tc::fence_after_sync();
     };
-    // layer 1 -> tensor-memory columns [0, 64)
-    if (t == 0) {
-        tc::mma_bf16(tmem, tc::smem_desc(sb + kA1, 128, 256), tc::smem_desc(sb + kB1, 128, 256), id64, 0);
-        tc::mma_commit(bar);
-    }
-    wait_mma();
-    for (int c = 0; c < 4; ++c) {
-        float v[16];
-        tc::tmem_ld16(tmem + lanes + c * 16, v);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            v[k] = gelu(v[k] + vb1[c * 16 + k]);
-            store1(sm + kBA1T, c * 16 + k, t, 128, v[k]);
+    float s_w3 = 0.0f, s_b2 = 0.0f, s_b1 = 0.0f, s_b3 = 0.0f;   // of column c0 + lane; s_b3 of this row
+    double s_loss = 0.0;
+    const int64_t ntiles = (batch_size + 127) / 128;
+    bool first = true;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t pos = tile * 128 + row;
+        const bool valid = pos < batch_size && batch_begin + pos < n;
+        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float target = 0.0f;
+        if (valid) {
+            const int64_t s = permute(batch_begin + pos, n, pa, pc);
+            if (half == 0) {
+                const float4 q = F[s];
+                f[0] = q.x; f[1] = q.y; f[2] = q.z; f[3] = q.w;
+            }
+            target = T[s];
         }
-        store8(sm + kA2, t, c * 16, kH, v);
-        store8(sm + kA2, t, c * 16 + 8, kH, v + 8);
-    }
-    sync_for_mma();
-    // layer 2 -> columns [64, 128)
-    if (t == 0) {
-        for (int k = 0; k < 4; ++k)
-            tc::mma_bf16(tmem + 64, tc::smem_desc(sb + kA2 + k * 256, 128, 1024),
-                         tc::smem_desc(sb + kB2 + k * 256, 128, 1024), id64, k > 0);
-        tc::mma_commit(bar);
-    }
-    wait_mma();
-    float y = w[kOffB3];
-    for (int c = 0; c < 4; ++c) {
-        float v[16];
-        tc::tmem_ld16(tmem + lanes + 64 + c * 16, v);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) y = fmaf(vw3[c * 16 + k], gelu(v[k] + vb2[c * 16 + k]), y);
-    }
-    const float inv_b = 1.0f / (float)batch_size;
-    const float e = valid ? (y - target) : 0.0f;
-    const float dy = 2.0f * e * inv_b;
-    atomicAdd(rloss, e * e);
-    atomicAdd(rb3, dy);
-    for (int c = 0; c < 4; ++c) {
-        float v[16], d[16];
-        tc::tmem_ld16(tmem + lanes + 64 + c * 16, v);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const int o = c * 16 + k;
-            const float z = v[k] + vb2[o];
-            d[k] = dy * vw3[o] * gelu_d(z);
-            atomicAdd(&rw3[o], dy * gelu(z));
-            atomicAdd(&rb2[o], d[k]);
-            store1(sm + kAD2T, o, t, 128, d[k]);
+        if (!first) wait_mma();   // the previous tile's gradient MMAs have read both tiles
+        if (half == 0) store8(sm + kSmA, row, kH, kColsA, f);
+        sync_for_mma();
+        tmem = *slot;
+        // layer 1: z1 -> columns [0, 64)
+        if (t == 0) {
+            tc::mma_bf16(tmem, tc::smem_desc(sb + kSmA + (kH / 8) * 128, 128, kColsA * 16),
+                         tc::smem_desc(sb + kSmW1, 128, 256), id_layer, 0);
+            tc::mma_commit(bar);
         }
-        store8(sm + kAD2, t, c * 16, kH, d);
-        store8(sm + kAD2, t, c * 16 + 8, kH, d + 8);
-    }
-    sync_for_mma();
-    // delta2 W2 -> columns [128, 192)
-    if (t == 0) {
-        for (int k = 0; k < 4; ++k)
-            tc::mma_bf16(tmem + 128, tc::smem_desc(sb + kAD2 + k * 256, 128, 1024),
-                         tc::smem_desc(sb + kB2T + k * 256, 128, 1024), id64, k > 0);
-        tc::mma_commit(bar);
-    }
-    wait_mma();
-    for (int c = 0; c < 4; ++c) {
-        float g[16], z[16];
-        tc::tmem_ld16(tmem + lanes + 128 + c * 16, g);
-        tc::tmem_ld16(tmem + lanes + c * 16, z);
+        wait_mma();
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const int o = c * 16 + k;
-            const float d1 = g[k] * gelu_d(z[k] + vb1[o]);
-            atomicAdd(&rb1[o], d1);
-            store1(sm + kAD1T, o, t, 128, d1);
-        }
-    }
-    sync_for_mma();
-    // dW2 = delta2^T a1 -> columns [192, 256); dW1 = delta1^T F -> columns [0, 16)
-    if (t == 0) {
-        for (int k = 0; k < 8; ++k)
-            tc::mma_bf16(tmem + 192, tc::smem_desc(sb + kAD2T + k * 256, 128, 2048),
-                         tc::smem_desc(sb + kBA1T + k * 256, 128, 2048), id64, k > 0);
-        for (int k = 0; k < 8; ++k)
-            tc::mma_bf16(tmem, tc::smem_desc(sb + kAD1T + k * 256, 128, 2048),
-                         tc::smem_desc(sb + kBFT + k * 256, 128, 2048), id16, k > 0);
-        tc::mma_commit(bar);
-    }
-    wait_mma();
-    if (warp < 2) {                                   // rows 0..63 hold the 64 weight rows
-        const int o = t;
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
             float v[16];
-            tc::tmem_ld16(tmem + lanes + 192 + c * 16, v);
+            tc::tmem_ld16(tmem + lanes + c0 + c * 16, v);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) atomicAdd(&grad[kOffW2 + o * kH + c * 16 + k], v[k]);
+            for (int k = 0; k < 16; k += 2) {
+                const int o = c0 + c * 16 + k;
+                gelu::upk(gelu::gelu_pair(fmaf(0.5f, v[k], vb1[o]), fmaf(0.5f, v[k + 1], vb1[o + 1])), v[k], v[k + 1]);
+            }
+            store8(sm + kSmA, row, c0 + c * 16, kColsA, v);
+            store8(sm + kSmA, row, c0 + c * 16 + 8, kColsA, v + 8);
         }
-        float v[16];
-        tc::tmem_ld16(tmem + lanes, v);
+        sync_for_mma();
+        // layer 2: z2 -> columns [64, 128)
+        if (t == 0) {
+            for (int k = 0; k < 4; ++k)
+                tc::mma_bf16(tmem + kColZ2, tc::smem_desc(sb + kSmA + k * 256, 128, kColsA * 16),
+                             tc::smem_desc(sb + kSmW2 + k * 256, 128, 1024), id_layer, k > 0);
+            tc::mma_commit(bar);
+        }
+        wait_mma();
+        float a2[32], g2[32];
+        float y = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) atomicAdd(&grad[kOffW1 + o * kF + k], v[k]);
+        for (int c = 0; c < 2; ++c) {
+            float v[16];
+            tc::tmem_ld16(tmem + lanes + kColZ2 + c0 + c * 16, v);
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) {
+                const int o = c0 + c * 16 + k, q = c * 16 + k;
+                gelu::f2 a, d;
+                gelu::gelu_grad_pair(fmaf(0.5f, v[k], vb2[o]), fmaf(0.5f, v[k + 1], vb2[o + 1]), a, d);
+                gelu::upk(a, a2[q], a2[q + 1]);
+                gelu::upk(d, g2[q], g2[q + 1]);
+                y = fmaf(vw3[o], a2[q], y);
+                y = fmaf(vw3[o + 1], a2[q + 1], y);
+            }
+        }
+        ypart[half * 128 + row] = y;
+        __syncthreads();
+        y = b3 + (ypart[row] + ypart[128 + row]);
+        const float e = valid ? (y - target) : 0.0f;
+        const float dy = 2.0f * e * inv_b;
+        if (half == 0) {
+            s_loss += (double)e * (double)e;
+            s_b3 += dy;
+        }
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            g2[k] *= dy * vw3[c0 + k];
+            a2[k] *= dy;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) store8(sm + kSmD, row, c0 + c * 8, kColsD, g2 + c * 8);
+        s_w3 += column_sums(a2);
+        s_b2 += column_sums(g2);
+        sync_for_mma();
+        // delta2 W2 -> columns [64, 128) (z2 has been read)
+        if (t == 0) {
+            for (int k = 0; k < 4; ++k)
+                tc::mma_bf16(tmem + kColZ2, tc::smem_desc(sb + kSmD + k * 256, 128, kColsD * 16),
+                             tc::smem_desc(sb + kSmW2 + k * 2048, 1024, 128), id_layer_t, k > 0);
+            tc::mma_commit(bar);
+        }
+        wait_mma();
+        float d1[32];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            float g[16], z[16];
+            tc::tmem_ld16(tmem + lanes + kColZ2 + c0 + c * 16, g);
+            tc::tmem_ld16(tmem + lanes + c0 + c * 16, z);
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) {
+                const int o = c0 + c * 16 + k, q = c * 16 + k;
+                gelu::f2 a, d;
+                gelu::gelu_grad_pair(fmaf(0.5f, z[k], vb1[o]), fmaf(0.5f, z[k + 1], vb1[o + 1]), a, d);
+                gelu::upk(gelu::mul2(d, gelu::pk(g[k], g[k + 1])), d1[q], d1[q + 1]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) store8(sm + kSmD, row, kH + c0 + c * 8, kColsD, d1 + c * 8);
+        s_b1 += column_sums(d1);
+        sync_for_mma();
+        // [delta2 | delta1]^T [a1 | F], accumulated over the CTA's tiles -> columns [128, 208)
+        if (t == 0) {
+            for (int k = 0; k < 8; ++k)
+                tc::mma_bf16(tmem + kColG, tc::smem_desc(sb + kSmD + k * 4096, 2048, 128),
+                             tc::smem_desc(sb + kSmA + k * 2560, 1280, 128), id_grad, (!first || k > 0) ? 1u : 0u);
+            tc::mma_commit(bar);
+        }
+        first = false;
     }
-    __syncthreads();
-    if (t < kH) {
-        atomicAdd(&grad[kOffW3 + t], rw3[t]);
-        atomicAdd(&grad[kOffB2 + t], rb2[t]);
-        atomicAdd(&grad[kOffB1 + t], rb1[t]);
+    if (!first) wait_mma();
+    const bool vec = (reinterpret_cast<uintptr_t>(grad) & 15u) == 0;
+    if (!first) {
+        const int lrow = (warp & 3) * 32 + lane;      // gradient row of this thread
+        if (lrow < kH) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                float v[16];
+                tc::tmem_ld16(tmem + lanes + kColG + c0 + c * 16, v);
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) add4(grad + kOffW2 + lrow * kH + c0 + c * 16 + k, v + k, vec);
+            }
+        } else if (half == 0) {
+            float v[16];
+            tc::tmem_ld16(tmem + lanes + kColG + kH, v);
+            add4(grad + kOffW1 + (lrow - kH) * kF, v, vec);
+        }
     }
-    if (t == 0) {
-        atomicAdd(&grad[kOffB3], *rb3);
-        atomicAdd(loss, (double)*rloss);
+    float *red = reinterpret_cast<float *>(sm + kSmRed);
+    red[warp * 96 + lane] = s_w3;
+    red[warp * 96 + 32 + lane] = s_b2;
+    red[warp * 96 + 64 + lane] = s_b1;
+    if (half == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s_b3 += __shfl_xor_sync(0xffffffffu, s_b3, o);
+            s_loss += __shfl_xor_sync(0xffffffffu, s_loss, o);
+        }
+        if (lane == 0) {
+            *reinterpret_cast<double *>(sm + kSmSum + warp * 16) = s_loss;
+            *reinterpret_cast<float *>(sm + kSmSum + warp * 16 + 8) = s_b3;
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
+    if (t < 192) {
+        // quantity t / 64 (dW3, db2, db1), column t % 64: the four warps of its half
+        const int q = t >> 6, c = t & 63;
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v += red[((c >> 5) * 4 + k) * 96 + q * 32 + (c & 31)];
+        atomicAdd(&grad[(q == 0 ? kOffW3 : (q == 1 ? kOffB2 : kOffB1)) + c], v);
+    }
+    if (t == 192) {
+        float v = 0.0f;
+        double l = 0.0;
+        for (int k = 0; k < 4; ++k) {
+            l += *reinterpret_cast<double *>(sm + kSmSum + k * 16);
+            v += *reinterpret_cast<float *>(sm + kSmSum + k * 16 + 8);
+        }
+        atomicAdd(&grad[kOffB3], v);
+        atomicAdd(loss, l);
+    }
     if (!good && t == 0) {
         tc::mbar_wait_bounded(bar, (phase - 1) & 1u, kWaitLimit);
         atomicExch(err, 1);
     }
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+    if (warp == 0) tc::tmem_dealloc(*slot, kCols);
 }
 
 // Adam (Kingma & Ba) on the FP32 master weights; clears the gradient.
@@ -375,6 +445,16 @@ cudaError_t set_attr()
     return cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
+// CTAs of the gradient kernel over a batch: one per tile, at most two per SM.
+unsigned grad_grid(int64_t batch)
+{
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
+        nsm = 1;
+    return (unsigned)std::min<int64_t>((batch + 127) / 128, (int64_t)nsm * kCtasPerSm);
+}
+
 }  // namespace
 
 }  // namespace sph
@@ -390,9 +470,8 @@ extern "C" sph_status sph_mlp_grad(const float *params, const float *features, c
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaMemsetAsync(grad, 0, sizeof(float) * kNW, s) != cudaSuccess) return SPH_ECUDA;
     if (cudaMemsetAsync(loss, 0, sizeof(double), s) != cudaSuccess) return SPH_ECUDA;
-    k_mlp_grad<<<(unsigned)((n + 127) / 128), 128, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features),
-                                                               labels, n, 0, n, 1, 0, grad, loss,
-                                                               reinterpret_cast<int *>(error));
+    k_mlp_grad<<<grad_grid(n), kThreads, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features), labels, n, 0, n,
+                                                     1, 0, grad, loss, reinterpret_cast<int *>(error));
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
 }
 
@@ -436,8 +515,8 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
         const uint64_t c = mix64(seed ^ (0xA5A5A5A5ull + (uint64_t)e)) % (uint64_t)n;
         for (int64_t b0 = 0; b0 < n; b0 += B) {
             const int64_t bs = std::min<int64_t>(B, n - b0);
-            k_mlp_grad<<<(unsigned)((bs + 127) / 128), 128, kSmem, s>>>(params, Fs, Ts, n, b0, bs, a, c, grad, acc,
-                                                                        reinterpret_cast<int *>(error));
+            k_mlp_grad<<<grad_grid(bs), kThreads, kSmem, s>>>(params, Fs, Ts, n, b0, bs, a, c, grad, acc,
+                                                              reinterpret_cast<int *>(error));
             ++step;
             k_mlp_adam<<<(kNW + 255) / 256, 256, 0, s>>>(params, m, v, grad, step, lr, 0.9f, 0.999f, 1e-8f);
         }

@@ -42,6 +42,12 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t M, uint32_t N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
+// Operand A (B) with its M (N) dimension contiguous instead of K: added to the instruction
+// descriptor.  The same core-matrix tiles then read the other way: the leading byte offset
+// is the distance of 8-element groups along K, the stride byte offset along M (N).
+constexpr uint32_t kIdescAMajorM = 1u << 15;
+constexpr uint32_t kIdescBMajorN = 1u << 16;
+
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols)
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(dst_smem)),

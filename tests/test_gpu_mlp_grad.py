@@ -1,0 +1,40 @@
+"""The network's gradient kernel at the edges of its 128-sample tiles, over several tiles a
+CTA and into a gradient buffer that is not 16-byte aligned, against the oracle's FP64 one."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2403_11156_gb300 import sph
+
+from gpu_util import gpu_ctx  # noqa: F401  (builds the library)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,offset", [(1, 0), (127, 0), (128, 1), (129, 2), (3 * 128 - 1, 0), (128 * 304 + 1, 0),
+                                      (128 * 650 + 77, 3)])
+def test_gradient_tiles(n, offset):
+    import torch
+    rng = np.random.default_rng(n)
+    p = np.zeros(sph.MLP_PARAMS, np.float32)
+    p[:sph.MLP_WEIGHTS] = rng.normal(scale=0.3, size=sph.MLP_WEIGHTS)
+    p[sph.MLP_WEIGHTS + 4:sph.MLP_WEIGHTS + 8] = 1.0
+    p[-1] = 1.0
+    f = rng.normal(size=(n, 4)).astype(np.float32)
+    t = (rng.normal(size=n) + 8.0).astype(np.float32)   # labels off the outputs: no cancellation in dy
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    buf = torch.full((sph.MLP_WEIGHTS + 8,), 7.0, device="cuda")
+    g = buf[offset:offset + sph.MLP_WEIGHTS]
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert sph.sph_mlp_grad(dev(p), dev(f), dev(t), n, g, loss, err) == sph.SPH_OK
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    ref_loss, ref = oracle.mlp_loss_grad(p.astype(np.float64), f.astype(np.float64), t.astype(np.float64))
+    # BF16 operands (2^-9 each) through three products: normwise 2e-2, as in test_gpu_mlp
+    assert float(loss.item()) / n == pytest.approx(ref_loss, rel=2e-2)
+    got = g.cpu().numpy().astype(np.float64)
+    for lo, hi in [(0, 4545), (0, 256), (256, 320), (320, 4416), (4416, 4480), (4480, 4544), (4544, 4545)]:
+        assert np.linalg.norm(got[lo:hi] - ref[lo:hi]) <= 2e-2 * np.linalg.norm(ref[lo:hi])
+    rest = torch.cat([buf[:offset], buf[offset + sph.MLP_WEIGHTS:]])
+    assert bool((rest == 7.0).all())
