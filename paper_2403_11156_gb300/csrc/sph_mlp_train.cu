@@ -118,6 +118,21 @@ __device__ __forceinline__ void add4(float *g, const float *v, bool vec)
     }
 }
 
+// gelu and its derivative of a pair z = 2 h by the library's erff.
+__device__ __forceinline__ void gelu_grad_erff(float h0, float h1, gelu::f2 &g, gelu::f2 &d)
+{
+    float a[2], b[2];
+    const float z[2] = {2.0f * h0, 2.0f * h1};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float e = erff(z[k] * 0.70710678118654752f);
+        a[k] = 0.5f * z[k] * (1.0f + e);
+        b[k] = 0.5f * (1.0f + e) + z[k] * 0.39894228040143268f * __expf(-0.5f * z[k] * z[k]);
+    }
+    g = gelu::pk(a[0], a[1]);
+    d = gelu::pk(b[0], b[1]);
+}
+
 // Gradient of the batch's mean squared error (standardised features and labels).  A
 // persistent grid of at most two CTAs per SM walks 128-sample tiles; warps w and w + 4 share
 // the rows of tensor-memory lanes 32 (w mod 4) and take 32 of the 64 columns each.  Bound by
@@ -125,6 +140,11 @@ __device__ __forceinline__ void add4(float *g, const float *v, bool vec)
 // per 32 columns.  200,000 samples: 56 us (86 TFLOP/s), 6,950 us before, when every row added
 // its 192 terms to 192 shared words atomically, each tile added 4.5k weight gradients to
 // memory and the transposed copies of the operands held a CTA at 146 KB.
+// One gradient (ONCE) takes the polynomial GELU.  Training keeps erff and one summation order
+// of the output: Adam divides by the gradient's own size, so that over hundreds of steps a
+// last-bit change of an activation, where it moves a BF16 operand's rounding, grows a
+// thousandfold (small batches are bound by latency, not by the formula).
+template <bool ONCE>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     k_mlp_grad(const float *__restrict__ w, const float4 *__restrict__ F, const float *__restrict__ T, int64_t n,
                int64_t batch_begin, int64_t batch_size, uint64_t pa, uint64_t pc, float *grad, double *loss, int *err)
@@ -206,7 +226,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 #pragma unroll
             for (int k = 0; k < 16; k += 2) {
                 const int o = c0 + c * 16 + k;
-                gelu::upk(gelu::gelu_pair(fmaf(0.5f, v[k], vb1[o]), fmaf(0.5f, v[k + 1], vb1[o + 1])), v[k], v[k + 1]);
+                const float h0 = fmaf(0.5f, v[k], vb1[o]), h1 = fmaf(0.5f, v[k + 1], vb1[o + 1]);
+                if (ONCE) {
+                    gelu::upk(gelu::gelu_pair(h0, h1), v[k], v[k + 1]);
+                } else {
+                    v[k] = h0 * (1.0f + erff(2.0f * h0 * 0.70710678118654752f));
+                    v[k + 1] = h1 * (1.0f + erff(2.0f * h1 * 0.70710678118654752f));
+                }
             }
             store8(sm + kSmA, row, c0 + c * 16, kColsA, v);
             store8(sm + kSmA, row, c0 + c * 16 + 8, kColsA, v + 8);
@@ -221,7 +247,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         }
         wait_mma();
         float a2[32], g2[32];
-        float y = 0.0f;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             float v[16];
@@ -230,16 +255,30 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
             for (int k = 0; k < 16; k += 2) {
                 const int o = c0 + c * 16 + k, q = c * 16 + k;
                 gelu::f2 a, d;
-                gelu::gelu_grad_pair(fmaf(0.5f, v[k], vb2[o]), fmaf(0.5f, v[k + 1], vb2[o + 1]), a, d);
+                const float h0 = fmaf(0.5f, v[k], vb2[o]), h1 = fmaf(0.5f, v[k + 1], vb2[o + 1]);
+                if (ONCE) gelu::gelu_grad_pair(h0, h1, a, d);
+                else gelu_grad_erff(h0, h1, a, d);
                 gelu::upk(a, a2[q], a2[q + 1]);
                 gelu::upk(d, g2[q], g2[q + 1]);
-                y = fmaf(vw3[o], a2[q], y);
-                y = fmaf(vw3[o + 1], a2[q + 1], y);
             }
         }
-        ypart[half * 128 + row] = y;
+        // y = b3 + w3 . a2, in column order: the second half goes on from the first's sum
+        auto dot = [&](float y) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) y = fmaf(vw3[c0 + k], a2[k], y);
+            return y;
+        };
+        if (half == 0) ypart[row] = dot(b3);
+        else if (ONCE) ypart[128 + row] = dot(0.0f);
         __syncthreads();
-        y = b3 + (ypart[row] + ypart[128 + row]);
+        float y;
+        if (ONCE) {
+            y = ypart[row] + ypart[128 + row];
+        } else {
+            if (half == 1) ypart[128 + row] = dot(ypart[row]);
+            __syncthreads();
+            y = ypart[128 + row];
+        }
         const float e = valid ? (y - target) : 0.0f;
         const float dy = 2.0f * e * inv_b;
         if (half == 0) {
@@ -274,7 +313,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
             for (int k = 0; k < 16; k += 2) {
                 const int o = c0 + c * 16 + k, q = c * 16 + k;
                 gelu::f2 a, d;
-                gelu::gelu_grad_pair(fmaf(0.5f, z[k], vb1[o]), fmaf(0.5f, z[k + 1], vb1[o + 1]), a, d);
+                const float h0 = fmaf(0.5f, z[k], vb1[o]), h1 = fmaf(0.5f, z[k + 1], vb1[o + 1]);
+                if (ONCE) gelu::gelu_grad_pair(h0, h1, a, d);
+                else gelu_grad_erff(h0, h1, a, d);
                 gelu::upk(gelu::mul2(d, gelu::pk(g[k], g[k + 1])), d1[q], d1[q + 1]);
             }
         }
@@ -442,7 +483,9 @@ uint64_t gcd64(uint64_t a, uint64_t b)
 
 cudaError_t set_attr()
 {
-    return cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_mlp_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
 // CTAs of the gradient kernel over a batch: one per tile, at most two per SM.
@@ -470,7 +513,7 @@ extern "C" sph_status sph_mlp_grad(const float *params, const float *features, c
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaMemsetAsync(grad, 0, sizeof(float) * kNW, s) != cudaSuccess) return SPH_ECUDA;
     if (cudaMemsetAsync(loss, 0, sizeof(double), s) != cudaSuccess) return SPH_ECUDA;
-    k_mlp_grad<<<grad_grid(n), kThreads, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features), labels, n, 0, n,
+    k_mlp_grad<true><<<grad_grid(n), kThreads, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features), labels, n, 0, n,
                                                      1, 0, grad, loss, reinterpret_cast<int *>(error));
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
 }
@@ -515,7 +558,7 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
         const uint64_t c = mix64(seed ^ (0xA5A5A5A5ull + (uint64_t)e)) % (uint64_t)n;
         for (int64_t b0 = 0; b0 < n; b0 += B) {
             const int64_t bs = std::min<int64_t>(B, n - b0);
-            k_mlp_grad<<<grad_grid(bs), kThreads, kSmem, s>>>(params, Fs, Ts, n, b0, bs, a, c, grad, acc,
+            k_mlp_grad<false><<<grad_grid(bs), kThreads, kSmem, s>>>(params, Fs, Ts, n, b0, bs, a, c, grad, acc,
                                                               reinterpret_cast<int *>(error));
             ++step;
             k_mlp_adam<<<(kNW + 255) / 256, 256, 0, s>>>(params, m, v, grad, step, lr, 0.9f, 0.999f, 1e-8f);
