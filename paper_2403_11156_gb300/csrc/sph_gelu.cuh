@@ -12,6 +12,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace sph {
 namespace gelu {
@@ -72,6 +73,53 @@ __device__ __forceinline__ f2 gelu_pair(float h0, float h1)
 {
     const f2 s = pk(fmaxf(-fabsf(h0), -3.0f), fmaxf(-fabsf(h1), -3.0f));
     return fma2(s, erfc_pair(s), pk(h0 + fabsf(h0), h1 + fabsf(h1)));
+}
+
+// Hidden activations become BF16 operands, where a last-bit difference of the FP32 value can
+// move the rounding by 2^-8.  So that operands are rounded as erff's formula rounds them, values
+// within 16 ulp of a rounding boundary (low half within 16 of 0x8000) are found with two packed
+// 16-bit operations a pair and taken from the formula; 16 columns of a warp hold one time in
+// five such a value.  (The two formulas differ by at most 15 ulp where |gelu| >= 1/16, and by
+// more only in the tail z < -1.9, where the formula cancels; below 1/64 a BF16 step is too
+// small to matter and is left.)
+__device__ __forceinline__ uint32_t tie_key(uint32_t m, float a, float b)
+{
+    uint32_t x = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x5410);
+    asm("add.u16x2 %0, %0, %1;" : "+r"(x) : "r"(0x80108010u));
+    asm("min.u16x2 %0, %0, %1;" : "+r"(m) : "r"(x));
+    return m;
+}
+__device__ __forceinline__ bool tie_found(uint32_t m) { return (m & 0xffffu) < 32u || (m >> 16) < 32u; }
+__device__ __forceinline__ float at_tie(float g, float h)
+{
+    if (((__float_as_uint(g) + 0x8010u) & 0xffffu) >= 32u || fabsf(g) < 0.015625f) return g;
+    return h * (1.0f + erff(2.0f * h * 0.70710678118654752f));
+}
+
+// gelu of 16 columns to be rounded to BF16: v holds the accumulators, half() gives the halved
+// pre-activations from them, reload() the accumulators again (every lane of the warp calls it).
+template <typename Half, typename Reload>
+__device__ __forceinline__ void gelu16(float (&v)[16], Half &&half, Reload &&reload)
+{
+    uint32_t m = 0xffffffffu;
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+        float h0, h1;
+        upk(half(k, v[k], v[k + 1]), h0, h1);
+        upk(gelu_pair(h0, h1), v[k], v[k + 1]);
+        m = tie_key(m, v[k], v[k + 1]);
+    }
+    if (__any_sync(0xffffffffu, tie_found(m))) {
+        float a[16];
+        reload(a);
+#pragma unroll
+        for (int k = 0; k < 16; k += 2) {
+            float h0, h1;
+            upk(half(k, a[k], a[k + 1]), h0, h1);
+            v[k] = at_tie(v[k], h0);
+            v[k + 1] = at_tie(v[k + 1], h1);
+        }
+    }
 }
 
 // gelu and its derivative Phi(z) + z phi(z) of a pair z = 2 h.

@@ -7,13 +7,16 @@
 // in tensor memory) for tiles of 128 rows; the 64-wide output dot product runs on the
 // CUDA cores while the second layer's accumulators are read back.  The kernels are
 // persistent: a CTA allocates its tensor memory and stages the weights once, then walks
-// its tiles.  Inside a step only the particles whose gate is open are rows.
+// its tiles.  Inside a step only the particles whose gate is open are rows.  Bound by the
+// 128 GELUs a row on the CUDA cores: 1.2M rows take 96 us (205 us with erff and four CTAs
+// an SM; 83 us without the rounding ties of sph_gelu.cuh).
 //
 // Parameter block (float, length kMlpParams): W1[64][4], b1[64], W2[64][64], b2[64],
 // W3[64], b3, feature mean[4], feature std[4], label mean, label std.
 #include <cuda_bf16.h>
 
 #include "sph.h"
+#include "sph_gelu.cuh"
 #include "sph_internal.cuh"
 #include "sph_tc.cuh"
 
@@ -39,20 +42,19 @@ static_assert(kMlpParams == SPH_MLP_PARAMS, "parameter block layout");
 
 // shared-memory map of one CTA (bytes)
 constexpr uint32_t kSmA1 = 0;          // 128 x 16 bf16
-constexpr uint32_t kSmB1 = 4096;       // 64 x 16 bf16
-constexpr uint32_t kSmA2 = 8192;       // 128 x 64 bf16
-constexpr uint32_t kSmB2 = 24576;      // 64 x 64 bf16
-constexpr uint32_t kSmVec = 32768;     // b1, b2, w3 (float[64] each)
-constexpr uint32_t kSmBar = 33536;     // mbarrier
-constexpr uint32_t kSmTmem = 33544;    // tensor-memory address
-constexpr uint32_t kSmUsed = 33600;
-// requested dynamic shared memory: caps residency at 4 CTAs per SM (4 x (52 + 1) KB of the
-// SM's 228 KB; a fifth would need 265), so 4 x 128 tensor-memory columns never exceed 512
-constexpr uint32_t kSmRequest = 52 * 1024;
-constexpr uint32_t kTmemCols = 128;
+constexpr uint32_t kSmB1 = 4096;       // 64 x 16 bf16, W1 / 2
+constexpr uint32_t kSmB2 = 6144;       // 64 x 64 bf16, W2 / 2
+constexpr uint32_t kSmA2 = 14336;      // 128 x 64 bf16
+constexpr uint32_t kSmVec = 30720;     // b1 / 2, b2 / 2, w3 (float[64] each)
+constexpr uint32_t kSmBar = 31488;     // mbarrier
+constexpr uint32_t kSmTmem = 31496;    // tensor-memory address
+// requested dynamic shared memory: caps residency at 7 CTAs per SM (an eighth would need
+// 8 x (31 + 1) KB of the SM's 228 KB), whose tensor-memory columns (64 each: the second
+// layer's accumulators take the place of the first's) stay within 512
+constexpr uint32_t kSmRequest = 31 * 1024;
+static_assert(kSmTmem + 4 <= kSmRequest, "shared-memory map");
+constexpr uint32_t kTmemCols = 64;
 constexpr uint32_t kWaitLimit = 1u << 20;
-
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b)
 {
@@ -86,24 +88,25 @@ __device__ bool mlp_tiles(const float *__restrict__ w, unsigned char *sm, int64_
     if (warp == 0) tc::tmem_alloc(tmem_slot, kTmemCols);
     if (t == 0) tc::mbar_init(bar, 1);
     // layer-1 operand A: row t = (f0..f3, 0 x 12), the zero half written once; B1 row n =
-    // W1[n][0..3], 0 x 12; W2 as the layer-2 operand B
+    // W1[n][0..3] / 2, 0 x 12; W2 / 2 as the layer-2 operand B (the halving is exact: the
+    // layers give the halved pre-activations that gelu_pair takes)
     {
         const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         store8(sm + kSmA1, t, 8, 16, z);
         if (t < kH) {
-            float u[8] = {w[kOffW1 + t * kF + 0], w[kOffW1 + t * kF + 1], w[kOffW1 + t * kF + 2],
-                          w[kOffW1 + t * kF + 3], 0.f, 0.f, 0.f, 0.f};
+            float u[8] = {0.5f * w[kOffW1 + t * kF + 0], 0.5f * w[kOffW1 + t * kF + 1], 0.5f * w[kOffW1 + t * kF + 2],
+                          0.5f * w[kOffW1 + t * kF + 3], 0.f, 0.f, 0.f, 0.f};
             store8(sm + kSmB1, t, 0, 16, u);
             store8(sm + kSmB1, t, 8, 16, z);
-            b1[t] = w[kOffB1 + t];
-            b2[t] = w[kOffB2 + t];
+            b1[t] = 0.5f * w[kOffB1 + t];
+            b2[t] = 0.5f * w[kOffB2 + t];
             w3[t] = w[kOffW3 + t];
         }
         for (int idx = t; idx < kH * 8; idx += blockDim.x) {
             const int n = idx >> 3, kc = (idx & 7) * 8;
             float u[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) u[q] = w[kOffW2 + n * kH + kc + q];
+            for (int q = 0; q < 8; ++q) u[q] = 0.5f * w[kOffW2 + n * kH + kc + q];
             store8(sm + kSmB2, n, kc, kH, u);
         }
     }
@@ -138,12 +141,16 @@ __device__ bool mlp_tiles(const float *__restrict__ w, unsigned char *sm, int64_
         good = tc::mbar_wait_bounded(bar, 0, kWaitLimit);
         tc::fence_after_sync();
         // hidden layer 1: bias, GELU, BF16 -> layer-2 operand A (row t)
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < kH / 16; ++c) {
             float v[16];
             tc::tmem_ld16(tmem + lane_base + c * 16, v);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) v[k] = gelu(v[k] + b1[c * 16 + k]);
+            gelu::gelu16(
+                v,
+                [&](int k, float a, float b) {
+                    return gelu::add2(gelu::pk(a, b), *reinterpret_cast<const gelu::f2 *>(b1 + c * 16 + k));
+                },
+                [&](float (&a)[16]) { tc::tmem_ld16(tmem + lane_base + c * 16, a); });
             store8(sm + kSmA2, t, c * 16, kH, v);
             store8(sm + kSmA2, t, c * 16 + 8, kH, v + 8);
         }
@@ -155,21 +162,27 @@ __device__ bool mlp_tiles(const float *__restrict__ w, unsigned char *sm, int64_
             // D2[128 x 64] = A2[128 x 64] W2^T in four K = 16 steps (two core matrices each)
 #pragma unroll
             for (int k = 0; k < kH / 16; ++k)
-                tc::mma_bf16(tmem + kH, tc::smem_desc(sbase + kSmA2 + k * 256, 128, 1024),
+                tc::mma_bf16(tmem, tc::smem_desc(sbase + kSmA2 + k * 256, 128, 1024),
                              tc::smem_desc(sbase + kSmB2 + k * 256, 128, 1024), idesc, k > 0 ? 1u : 0u);
             tc::mma_commit(bar);
         }
         good = tc::mbar_wait_bounded(bar, 1, kWaitLimit);
         tc::fence_after_sync();
-        float y = b3;
+        gelu::f2 acc = 0;   // even and odd columns
 #pragma unroll
         for (int c = 0; c < kH / 16; ++c) {
             float v[16];
-            tc::tmem_ld16(tmem + lane_base + kH + c * 16, v);
+            tc::tmem_ld16(tmem + lane_base + c * 16, v);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) y = fmaf(w3[c * 16 + k], gelu(v[k] + b2[c * 16 + k]), y);
+            for (int k = 0; k < 16; k += 2) {
+                float h0, h1;
+                gelu::upk(gelu::add2(gelu::pk(v[k], v[k + 1]), *reinterpret_cast<const gelu::f2 *>(b2 + c * 16 + k)), h0, h1);
+                acc = gelu::fma2(*reinterpret_cast<const gelu::f2 *>(w3 + c * 16 + k), gelu::gelu_pair(h0, h1), acc);
+            }
         }
-        if (valid) rows.store(tile, t, y);
+        float y0, y1;
+        gelu::upk(acc, y0, y1);
+        if (valid) rows.store(tile, t, b3 + (y0 + y1));
     }
     tc::fence_before_sync();
     good = __syncthreads_and(good);
@@ -203,7 +216,7 @@ struct DenseRows {
     __device__ void store(int64_t tile, int t, float out) const { y[tile * 128 + t] = out; }
 };
 
-__global__ void __launch_bounds__(128) k_mlp_forward(const float *__restrict__ w, const float4 *__restrict__ feat,
+__global__ void __launch_bounds__(128, 7) k_mlp_forward(const float *__restrict__ w, const float4 *__restrict__ feat,
                                                      int64_t n, float *__restrict__ y, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -255,7 +268,7 @@ struct GatedRows {
 
 // Learned warm start inside a step: a persistent grid over the gated rows (their count
 // is known only on the device).
-__global__ void __launch_bounds__(128) k_mlp_warm(Ptrs P)
+__global__ void __launch_bounds__(128, 7) k_mlp_warm(Ptrs P)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     kernel_enter(P.ctl, KID_MLP_WARM);
@@ -268,9 +281,8 @@ __global__ void __launch_bounds__(128) k_mlp_warm(Ptrs P)
         atomicExch(&P.ctl->error, 4);
 }
 
-// Resident CTAs of the network kernels per SM: the shared-memory request caps it, so that
-// their tensor-memory columns (128 each) never exceed the SM's 512.
-constexpr int kMlpCtasPerSm = 4;
+// Resident CTAs of the network kernels per SM (as the shared-memory request caps it).
+constexpr int kMlpCtasPerSm = 7;
 
 int mlp_grid(int64_t tiles)
 {

@@ -38,3 +38,27 @@ def test_gradient_tiles(n, offset):
         assert np.linalg.norm(got[lo:hi] - ref[lo:hi]) <= 2e-2 * np.linalg.norm(ref[lo:hi])
     rest = torch.cat([buf[:offset], buf[offset + sph.MLP_WEIGHTS:]])
     assert bool((rest == 7.0).all())
+
+
+@pytest.mark.parametrize("n", [1, 128, 129, 128 * 152 * 7 + 5])
+def test_forward_non_finite_rows(n):
+    """A NaN or infinite feature gives NaN in its own row and changes no other."""
+    import torch
+    rng = np.random.default_rng(n)
+    p = np.zeros(sph.MLP_PARAMS, np.float32)
+    p[:sph.MLP_WEIGHTS] = rng.normal(scale=0.3, size=sph.MLP_WEIGHTS)
+    f = torch.tensor(rng.normal(size=(n, 4)).astype(np.float32), device="cuda")
+    dp = torch.tensor(p, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    y = [torch.empty(n, device="cuda") for _ in range(2)]
+    assert sph.sph_mlp_forward(dp, f, n, y[0], err) == sph.SPH_OK
+    bad = sorted({0, n // 2, n - 1})
+    for k, i in enumerate(bad):
+        f[i, k % 4] = [float("nan"), float("inf"), float("-inf")][k]
+    assert sph.sph_mlp_forward(dp, f, n, y[1], err) == sph.SPH_OK
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    keep = torch.ones(n, dtype=torch.bool, device="cuda")
+    keep[bad] = False
+    assert bool(torch.isnan(y[1][~keep]).all())
+    assert torch.equal(y[0][keep], y[1][keep])
