@@ -322,6 +322,26 @@ __global__ void k_read_fluid(Ptrs P, int scene, int field, void *out)
     }
 }
 
+// The state fields of one scene in original particle order, those asked for, in one launch.
+__global__ void k_read_state(Ptrs P, int scene, float *__restrict__ x, float *__restrict__ vel,
+                             float *__restrict__ rho, float *__restrict__ pressure)
+{
+    const SceneDev &sc = P.scenes[scene];
+    const int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (local >= sc.nf) return;
+    const int64_t i = sc.f_off + local, o = P.id_c[i];
+    if (x) {
+        const float4 p = P.pos_c[i];
+        x[3 * o] = p.x; x[3 * o + 1] = p.y; x[3 * o + 2] = p.z;
+    }
+    if (vel || rho || pressure) {
+        const float4 v = P.vel_c[i];
+        if (vel) { vel[3 * o] = v.x; vel[3 * o + 1] = v.y; vel[3 * o + 2] = v.z; }
+        if (rho) rho[o] = v.w;
+        if (pressure) pressure[o] = P.ksum[i] * v.w;
+    }
+}
+
 __global__ void k_read_boundary(Ptrs P, int scene, int field, void *out)
 {
     const SceneDev &sc = P.scenes[scene];
@@ -344,12 +364,14 @@ __global__ void k_read_boundary(Ptrs P, int scene, int field, void *out)
     }
 }
 
-// Bring one scene's canonical arrays back to original particle order (through the
-// sorted arrays as scratch), so that a checkpoint can be written in that order.
+// A state written by the caller replaces the canonical arrays in original particle order.
+// First launch: the present state goes to that order through the sorted arrays (what the
+// caller does not give keeps its value), and the next step's size starts from its maximum.
 __global__ void k_unpermute_to_sorted(Ptrs P, int scene)
 {
     const SceneDev &sc = P.scenes[scene];
     int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (local == 0) P.st[scene].dt_next = sc.dt_max;
     if (local >= sc.nf) return;
     int64_t i = sc.f_off + local;
     int64_t d = sc.f_off + P.id_c[i];
@@ -358,50 +380,52 @@ __global__ void k_unpermute_to_sorted(Ptrs P, int scene)
     P.kprev_s[d] = P.kprev_c[i];
     P.kvprev_s[d] = P.kvprev_c[i];
 }
-__global__ void k_sorted_to_canonical(Ptrs P, int scene)
+
+// Second launch: the canonical arrays in original order from the caller's packed [n][3] and
+// [n] device arrays (null: the present value) and the CFL step of the new velocities,
+// min(dt_max, cfl 2r / max|v|).  Each block takes the step of its own largest speed and the
+// scene's is the minimum over the blocks: division and square root round monotonically, so
+// that is the step of the largest speed.  (As seven launches with a one-block maximum, which
+// read 1.2M velocities in 382 us, writing and reading back that state made a one-step pass
+// 2827 us; with this and the one-launch read it is 2401 us.)
+constexpr int kWriteThreads = 256;
+__global__ void __launch_bounds__(kWriteThreads)
+    k_write_canonical(Ptrs P, int scene, const float *__restrict__ x, const float *__restrict__ vel,
+                      const float *__restrict__ kp, const float *__restrict__ kvp)
 {
+    __shared__ float sh[kWriteThreads / 32];
     const SceneDev &sc = P.scenes[scene];
-    int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (local >= sc.nf) return;
-    int64_t i = sc.f_off + local;
-    P.pos_c[i] = P.pos_s[i];
-    float4 v = P.vel_s[i];
-    v.w = 0.0f;
-    P.vel_c[i] = v;
-    P.kprev_c[i] = P.kprev_s[i];
-    P.kvprev_c[i] = P.kvprev_s[i];
-    P.id_c[i] = (int32_t)local;
-    P.id_s[i] = (int32_t)local;
-    P.ksum[i] = 0.0f;
-    P.kvsum[i] = 0.0f;
-}
-// Write [n][3] (packed) into a float4 array, original order == canonical order here.
-__global__ void k_pack3(float4 *dst, const float *src, int64_t n, float w)
-{
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    dst[k] = make_float4(src[3 * k], src[3 * k + 1], src[3 * k + 2], w);
-}
-__global__ void k_scene_cfl(Ptrs P, int scene)
-{
-    __shared__ float sh[256];
-    const SceneDev &sc = P.scenes[scene];
+    const int64_t local = (int64_t)blockIdx.x * kWriteThreads + threadIdx.x;
     float m = 0.0f;
-    for (int64_t k = threadIdx.x; k < sc.nf; k += blockDim.x) {
-        float4 v = P.vel_c[sc.f_off + k];
-        m = fmaxf(m, v.x * v.x + v.y * v.y + v.z * v.z);
+    if (local < sc.nf) {
+        const int64_t i = sc.f_off + local;
+        float4 p = P.pos_s[i], v = P.vel_s[i];
+        if (x) p = make_float4(x[3 * local], x[3 * local + 1], x[3 * local + 2], 0.0f);
+        if (vel) v = make_float4(vel[3 * local], vel[3 * local + 1], vel[3 * local + 2], 0.0f);
+        v.w = 0.0f;
+        P.pos_c[i] = p;
+        P.vel_c[i] = v;
+        P.kprev_c[i] = kp ? kp[local] : P.kprev_s[i];
+        P.kvprev_c[i] = kvp ? kvp[local] : P.kvprev_s[i];
+        P.id_c[i] = (int32_t)local;
+        P.id_s[i] = (int32_t)local;
+        P.ksum[i] = 0.0f;
+        P.kvsum[i] = 0.0f;
+        m = v.x * v.x + v.y * v.y + v.z * v.z;
     }
-    sh[threadIdx.x] = m;
+    if (!(sc.cfl > 0.0f)) return;
+    m = fmaxf(m, 0.0f);   // a NaN counts as no speed
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] = fmaxf(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        float vm = sqrtf(sh[0]);
-        float dt = sc.dt_max;
-        if (sc.cfl > 0.0f && vm > 0.0f) dt = fminf(dt, sc.cfl * sc.two_r / vm);
-        P.st[scene].dt_next = dt;
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kWriteThreads / 32; ++w) m = fmaxf(m, sh[w]);
+    const float vm = sqrtf(m);
+    if (vm > 0.0f) {
+        // steps are not negative: their order is that of their bit patterns
+        const float dt = sc.cfl * sc.two_r / vm;
+        if (dt < sc.dt_max) atomicMin(reinterpret_cast<int *>(&P.st[scene].dt_next), __float_as_int(dt));
     }
 }
 
@@ -1376,11 +1400,17 @@ sph_status sph_read_state(sph_ctx *c, int32_t scene, float *x, float *v, float *
                                 {103, pressure, 4 * nf, false}};
         return read_host_async(c, scene, f, 4);
     }
+    if (on_device != 0) {
+        if (x || v || rho || pressure) k_read_state<<<(int)((nf + 255) / 256), 256, 0, c->stream>>>(c->P, scene, x, v, rho, pressure);
+        if ((st = check_async(c)) != SPH_OK) return st;
+        if (on_device == 1) CK(cudaStreamSynchronize(c->stream));
+        return SPH_OK;
+    }
     if ((st = read_into(c, scene, 100, x, 12 * nf, false, on_device)) != SPH_OK) return st;
     if ((st = read_into(c, scene, 101, v, 12 * nf, false, on_device)) != SPH_OK) return st;
     if ((st = read_into(c, scene, 102, rho, 4 * nf, false, on_device)) != SPH_OK) return st;
     if ((st = read_into(c, scene, 103, pressure, 4 * nf, false, on_device)) != SPH_OK) return st;
-    if (on_device <= 1) CK(cudaStreamSynchronize(c->stream));
+    CK(cudaStreamSynchronize(c->stream));
     return SPH_OK;
 }
 
@@ -1425,7 +1455,7 @@ sph_status sph_write_state(sph_ctx *c, int32_t scene, const float *x, const floa
     const SceneDev &q = c->scenes[scene];
     const int64_t nf = q.nf;
     cudaStream_t s = c->stream;
-    int blocks = (int)((nf + 255) / 256);
+    const int blocks = (int)((nf + kWriteThreads - 1) / kWriteThreads);
     // host inputs are staged into one device buffer before anything of the scene changes,
     // so that a failed staging leaves it as it was; the buffer is freed on every exit
     struct Stage {
@@ -1450,16 +1480,14 @@ sph_status sph_write_state(sph_ctx *c, int32_t scene, const float *x, const floa
             dv = stage.p + 3 * nf;
         }
     }
-    k_unpermute_to_sorted<<<blocks, 256, 0, s>>>(c->P, scene);
-    k_sorted_to_canonical<<<blocks, 256, 0, s>>>(c->P, scene);
+    k_unpermute_to_sorted<<<blocks, kWriteThreads, 0, s>>>(c->P, scene);
+    k_write_canonical<<<blocks, kWriteThreads, 0, s>>>(c->P, scene, dx, dv, on_device ? kappa_prev : nullptr,
+                                                       on_device ? kappa_v_prev : nullptr);
     if ((st = check_async(c)) != SPH_OK) return st;
-    if (x) k_pack3<<<blocks, 256, 0, s>>>(c->P.pos_c + q.f_off, dx, nf, 0.0f);
-    if (v) k_pack3<<<blocks, 256, 0, s>>>(c->P.vel_c + q.f_off, dv, nf, 0.0f);
-    cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (kappa_prev) CK(cudaMemcpyAsync(c->P.kprev_c + q.f_off, kappa_prev, 4 * nf, kind, s));
-    if (kappa_v_prev) CK(cudaMemcpyAsync(c->P.kvprev_c + q.f_off, kappa_v_prev, 4 * nf, kind, s));
-    k_scene_cfl<<<1, 256, 0, s>>>(c->P, scene);
-    if ((st = check_async(c)) != SPH_OK) return st;
+    if (!on_device && kappa_prev)
+        CK(cudaMemcpyAsync(c->P.kprev_c + q.f_off, kappa_prev, 4 * nf, cudaMemcpyHostToDevice, s));
+    if (!on_device && kappa_v_prev)
+        CK(cudaMemcpyAsync(c->P.kvprev_c + q.f_off, kappa_v_prev, 4 * nf, cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
     return SPH_OK;
 }
