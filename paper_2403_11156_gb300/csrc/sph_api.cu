@@ -86,6 +86,7 @@ struct sph_ctx {
     std::vector<int32_t> fblk_scene, bblk_scene, tblk_scene;
     std::vector<int32_t> nbody_scene;
     int max_bodies = 0;
+    int64_t nbr_entries = 0;             // of the fluid neighbour lists
     bool any_moving = false, any_div = false, any_warm_div = false, any_warm = false,
          any_learned = false, any_bodies = false, any_implicit = false, any_wcsph = false, any_strong = false;
     Ptrs P{};
@@ -784,6 +785,7 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
     P.NB = NB;
     P.NC = NC;
     c->reported_flags.assign(n, 0);
+    c->nbr_entries = NF * cap_f;
 
     bool ok = true;
     SceneState *st = nullptr;
@@ -1185,8 +1187,7 @@ sph_status sph_surface_field(sph_ctx *c, int32_t scene, const float origin[3], f
     }
     if (nodes > ((int64_t)1 << 31)) return fail(c, SPH_EINVAL, "surface field: grid too large");
     const SceneDev &q = c->scenes[scene];
-    cudaError_t e = post_surface_field(q, c->P.pos_c + q.f_off, c->P.vel_c + q.f_off, origin, spacing, dims, field,
-                                       c->stream);
+    cudaError_t e = post_surface_field(c->P, q, c->nbr_entries, origin, spacing, dims, field, c->stream);
     if (e != cudaSuccess) return fail(c, SPH_ECUDA, "surface field: %s", cudaGetErrorString(e));
     return SPH_OK;
 }

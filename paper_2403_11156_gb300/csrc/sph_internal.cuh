@@ -380,7 +380,7 @@ void launch_cg_beta(const Ptrs &P, cudaGraphConditionalHandle h, int use_handle,
 void launch_cg_p(const Ptrs &P, cudaStream_t s);
 
 // ------------------------------------------------------------------ post-processing (sph_post.cu)
-cudaError_t post_surface_field(const SceneDev &sc, const float4 *pos, const float4 *vel, const float origin[3],
+cudaError_t post_surface_field(const Ptrs &P, const SceneDev &sc, int64_t nbr_entries, const float origin[3],
                                float spacing, const int32_t dims[3], float *out, cudaStream_t s);
 cudaError_t post_height_map(const float4 *pos, int64_t n, const float lo[2], const float hi[2], int32_t w,
                             int32_t h, float radius, float *out, cudaStream_t s);
