@@ -495,6 +495,7 @@ sph_status enqueue_step(sph_ctx *c, cudaStream_t s, bool capture)
         run(c, b, "bsort_scan", [&] { launch_scan_cells(P, SORT_BOUNDARY, b); });
         run(c, b, "bsort_scatter", [&] { launch_scatter(P, SORT_BOUNDARY, b); });
         run(c, b, "bsort_rank_gather", [&] { launch_rank_gather(P, SORT_BOUNDARY, b); });
+        run(c, b, "boundary_near", [&] { launch_boundary_near(P, b); });
         run(c, b, "boundary_psi", [&] { launch_boundary_psi(P, b); });
         CK(cudaEventRecord(c->join, b));
     }
@@ -747,6 +748,22 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
             const double margin = 1e-3 * h + 1e-6 * mag;
             q.cull2 = (float)((h + margin) * (h + margin));
         }
+        {
+            // candidate filter of the density sweep (steps of h/512): a neighbour's coordinate
+            // differences are off by at most one step of rounding, one of carry and the float
+            // rounding of coordinates up to qmax; the half-precision sum of squares by 2e-3 more
+            double mag = 0.0;
+            for (int a = 0; a < 3; ++a)
+                mag = std::max(mag, std::max(std::fabs((double)d.domain_min[a]), std::fabs((double)d.domain_max[a])));
+            const double qmax = 2.0 * mag + 16.0 * h;
+            const double off = 2.0 / 512.0 + 16.0 * std::ldexp(qmax, -22) / h;
+            const double thr = std::pow(1.0 + 1.7321 * off, 2.0) * 1.002;
+            q.qscale = (float)(512.0 / h);
+            q.qmax = (float)qmax;
+            // steps of 2^-10 from 1 to 2, rounded up; past 2 nothing is filtered out (half infinity)
+            const uint32_t half = thr < 2.0 ? 0x3c00u + (uint32_t)std::ceil((thr - 1.0) * 1024.0) : 0x7c00u;
+            q.qthr = half | half << 16;
+        }
         q.cg_tol = d.cg_tol > 0.0f ? d.cg_tol : 1e-4f;
         q.cg_max = d.cg_max_iter > 0 ? d.cg_max_iter : 500;
         cap_f = std::max(cap_f, q.cap_f);
@@ -804,6 +821,7 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
     ok &= dalloc(c, P.id_c, NF) && dalloc(c, P.id_s, NF) && dalloc(c, P.nnf, NF) && dalloc(c, P.nnb, NF);
     ok &= dalloc(c, P.nbr, (size_t)NF * cap_f) && dalloc(c, P.bnbr, (size_t)NF * cap_b);
     ok &= dalloc(c, P.feat, (size_t)NF * 4);
+    ok &= dalloc(c, P.qpos, (size_t)NF / 2 + 8);
     ok &= dalloc(c, P.cell_count, NC) && dalloc(c, P.cell_start, NC + 1);
     ok &= dalloc(c, P.key_tmp, NF) && dalloc(c, P.slot_tmp, NF) && dalloc(c, P.sid_tmp, NF) &&
           dalloc(c, P.src_tmp, NF) && dalloc(c, P.cell_tmp, NF);
@@ -811,7 +829,7 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
     ok &= dalloc(c, P.bx_o, NBa) && dalloc(c, P.bv_o, NBa) && dalloc(c, P.br0, NBa) && dalloc(c, P.bbody, NBa);
     ok &= dalloc(c, P.bpos_s, NBa) && dalloc(c, P.bvel_s, NBa) && dalloc(c, P.bid_s, NBa) &&
           dalloc(c, P.bbody_s, NBa);
-    ok &= dalloc(c, P.bcell_count, NC) && dalloc(c, P.bcell_start, NC + 1);
+    ok &= dalloc(c, P.bcell_count, NC) && dalloc(c, P.bcell_start, NC + 1) && dalloc(c, P.bnear, NC);
     ok &= dalloc(c, P.large_f, large_capacity(NF)) && dalloc(c, P.large_b, large_capacity(NBa));
     ok &= dalloc(c, P.bkey_tmp, NBa) && dalloc(c, P.bslot_tmp, NBa) && dalloc(c, P.bsid_tmp, NBa) &&
           dalloc(c, P.bsrc_tmp, NBa) && dalloc(c, P.bcell_tmp, NBa);
@@ -971,6 +989,8 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
     ok &= cudaMemsetAsync(P.k0, 0, sizeof(float) * NF, s) == cudaSuccess;
     ok &= cudaMemsetAsync(P.nnf, 0, sizeof(int32_t) * NF, s) == cudaSuccess;
     ok &= cudaMemsetAsync(P.nnb, 0, sizeof(int32_t) * NF, s) == cudaSuccess;
+    ok &= cudaMemsetAsync(P.bnear, 0, (size_t)NC, s) == cudaSuccess;
+    ok &= cudaMemsetAsync(P.qpos, 0, sizeof(uint4) * ((size_t)NF / 2 + 8), s) == cudaSuccess;
     ok &= cudaMemsetAsync(P.feat, 0, sizeof(float) * 4 * NF, s) == cudaSuccess;
     if (!ok) return bail(fail(c, SPH_ECUDA, "upload failed"));
 
@@ -980,6 +1000,7 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
         launch_scan_cells(P, SORT_BOUNDARY, s);
         launch_scatter(P, SORT_BOUNDARY, s);
         launch_rank_gather(P, SORT_BOUNDARY, s);
+        launch_boundary_near(P, s);
         launch_boundary_psi(P, s);
         sph_status cs = check_async(c);
         if (cs != SPH_OK) return bail(cs);

@@ -3,13 +3,14 @@
 // T threads (lanes, T = 1, 2, 4 or 8) own one fluid particle in grid order.  The density
 // sweep walks the (2R+1)^3-cell neighbourhood ((2R+1)^2 contiguous index ranges) once
 // per step and records the particle's neighbours in one k-major list, in candidate order
-// (with T > 1 the lanes test T consecutive candidates at a time and append the hits by a
-// ballot over the group, so the list is the same for every T).  Every later sweep of the
+// (one thread a particle; with T = 8 eight lanes test eight consecutive candidates at a time:
+// the list is the same).  Every later sweep of the
 // step (divergence and density Jacobi passes, non-pressure forces, warm starts) gathers
 // through that list, lane s taking entries s, s + T, ..., and combines the T partial sums
 // with warp shuffles.  The solvers' error sums are accumulated per block in FP64 by pass A,
 // folded by pass B and summed in a fixed order by a one-block check kernel, which also
 // decides the loop condition on the device (CUDA graph conditional node).
+#include <cuda_fp16.h>
 #include <math_constants.h>
 
 #include <type_traits>
@@ -115,179 +116,250 @@ __global__ void k_step_begin(Ptrs P)
 
 // ------------------------------------------------------------------------------------
 // Density (Eq. density + Sec. 3.5 boundary term), DFSPH alpha, neighbour lists, and the
-// gate of the divergence warm start (D rho/Dt with the velocities at step start).
-// Nine resident blocks per SM with one lane (56 registers; left to itself the compiler picks
-// 48 and spills, measured 4 % slower on the 1.2M scene), eight with several (64 registers
-// for the batched cooperative append).
-template <int T>
-__global__ void __launch_bounds__(kBlock, T == 1 ? 9 : 8) k_density_alpha(Ptrs P)
+// gate of the divergence warm start (D rho/Dt with the velocities at step start); one thread
+// a particle (SUM = false: only the lists, k_density_sum follows).
+//
+// Phase 1 filters the stencil's rows: the candidates' coordinates in 16-bit steps of h/512 (the
+// reorder writes them negated, two particles a 16-byte word) give (d/h)^2 of two candidates at
+// a time in half precision, from one load and eleven instructions.  A difference q - c modulo
+// 2^16, added to the bits of the half 1536, is that half plus the difference (a half's step is 1
+// from 1024 to 2048, which covers differences up to h; beyond, the value only has to stay
+// beyond), so no conversion is needed; one 32-bit addition serves both, its carry being one step
+// in the second.  The threshold lies above 1 by more than all rounding (SceneDev::qthr), so every
+// neighbour passes, with 2 to 4 % more.  Phase 2 walks the passed ones with the exact predicate,
+// drops those that fail from the list in place, and sums: list, counts and sums are those of
+// the exact test on every candidate, in the same order.
+//
+// A particle whose passed candidates exceed the list, or that has left the range the filter
+// holds for (SceneDev::qmax), takes the exact predicate over its rows instead.
+//
+// Bound by instruction issue and gather latency in turn: at 500k particles 154 us (167 with the
+// exact predicate on every candidate and boundary rows looked up by all), of which the filter
+// takes about 50, the list writes 38 and phase 2 53; 1.2M with bodies 357 us (396).  With two and
+// four lanes the lists are built here and the lanes only sum: 100k particles 160 -> 58 us.
+__device__ __forceinline__ uint32_t query_pair(uint32_t word, uint32_t odd)
+{
+    return ((0x6600u - (odd ? word >> 16 : word)) & 0xffffu) * 0x10001u;
+}
+__device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<__half2 *>(&v); }
+struct Stencil {
+    uint32_t row;            // first row's cell of column 0
+    uint32_t dx, dxy;        // cells of a row, of a layer
+    int32_t x0, x1;          // first and last cell of every row
+    int32_t ny, nz, centre;  // rows a layer, layers, number of the particle's own row
+};
+
+// The exact predicate over the stencil: writes the list, returns the neighbour count.
+__device__ __noinline__ int exact_list(const Ptrs &P, const Stencil &st, int64_t i, float4 pi, float h2, int cap)
+{
+    int n = 0;
+    for (int32_t k = 0, y = 0, z = 0; k < st.ny * st.nz; ++k) {
+        const uint32_t row = st.row + (uint32_t)y * st.dx + (uint32_t)z * st.dxy;
+        if (++y == st.ny) { y = 0; ++z; }
+        const uint32_t je = P.cell_start[row + (uint32_t)st.x1 + 1u];
+        for (uint32_t j = P.cell_start[row + (uint32_t)st.x0]; j < je; ++j) {
+            float dx, dy, dz;
+            if (j != (uint32_t)i && pred_d2(pi, __ldg(P.pos_s + j), dx, dy, dz) < h2) {
+                if (n < cap) P.nbr[(int64_t)n * P.NF + i] = (int32_t)j;
+                ++n;
+            }
+        }
+    }
+    return n;
+}
+
+template <bool SUM>
+__global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ Ptrs P)
 {
     kernel_enter(P.ctl, KID_DENSITY);
-    const Lane<T> c = lane_ctx<T>(P);
+    const BlockCtx c = fluid_ctx(P);
     const SceneDev &sc = *c.sc;
     const int64_t i = c.i, NF = P.NF;
-    const int s = c.s;
     const bool gate = sc.warm != 0 && sc.div_on;
-    int nn_f = 0, nn_b = 0;  // this lane's neighbours (may exceed its capacity)
-    // this lane's shares of rho - m W(0), sum grad W, sum |grad W|^2 and D rho/Dt
-    float rho_l = 0.0f, s1x = 0.0f, s1y = 0.0f, s1z = 0.0f, s2 = 0.0f, div_l = 0.0f;
-    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    int nn_f = 0, nn_b = 0;   // neighbours (may exceed the capacity)
     if (c.valid) {
-        pi = P.pos_s[i];
-        const float4 vi = P.vel_s[i];
-        const int32_t cx = cell_coord(pi.x, sc.origin[0], sc.cell, sc.dims[0]);
-        const int32_t cy = cell_coord(pi.y, sc.origin[1], sc.cell, sc.dims[1]);
-        const int32_t cz = cell_coord(pi.z, sc.origin[2], sc.cell, sc.dims[2]);
-        const int32_t R = sc.R;
-        const float h2 = sc.h2, cull2 = sc.cull2, cs = sc.cell;
-        const unsigned long long pixy = pack_xy(pi.x, pi.y);   // for the packed candidate test
-        // offset of the particle inside its cell, per axis: the distance from the particle
-        // to a stencil cell d cells away is at least gap(d) (zero for d = 0)
-        const float ox = pi.x - fmaf((float)cx, cs, sc.origin[0]);
-        const float oy = pi.y - fmaf((float)cy, cs, sc.origin[1]);
-        const float oz = pi.z - fmaf((float)cz, cs, sc.origin[2]);
-        auto gap = [&](float o, int32_t d) {
-            const float g = d < 0 ? fmaf((float)(-d - 1), cs, o) : (d > 0 ? fmaf((float)d, cs, -o) : 0.0f);
-            return fmaxf(g, 0.0f);
-        };
+        const float4 pi = P.pos_s[i];
         const int cap_f = sc.cap_f, cap_b = sc.cap_b;
+        const float h2 = sc.h2;
+        Stencil st;
+        bool walls;   // a boundary particle in the stencil
+        {
+            const int32_t cx = cell_coord(pi.x, sc.origin[0], sc.cell, sc.dims[0]);
+            const int32_t cy = cell_coord(pi.y, sc.origin[1], sc.cell, sc.dims[1]);
+            const int32_t cz = cell_coord(pi.z, sc.origin[2], sc.cell, sc.dims[2]);
+            const int32_t R = sc.R, nx = sc.dims[0], ny = sc.dims[1], nz = sc.dims[2];
+            const int32_t y0 = max(cy - R, 0), z0 = max(cz - R, 0);
+            st.x0 = max(cx - R, 0);
+            st.x1 = min(cx + R, nx - 1);
+            st.ny = min(cy + R, ny - 1) - y0 + 1;
+            st.nz = min(cz + R, nz - 1) - z0 + 1;
+            st.centre = (cz - z0) * st.ny + (cy - y0);
+            st.dx = (uint32_t)nx;
+            st.dxy = (uint32_t)nx * (uint32_t)ny;
+            const uint32_t c0 = (uint32_t)sc.c_off;
+            st.row = c0 + (uint32_t)nx * ((uint32_t)y0 + (uint32_t)ny * (uint32_t)z0);
+            walls = P.bnear[c0 + (uint32_t)cx + (uint32_t)nx * ((uint32_t)cy + (uint32_t)ny * (uint32_t)cz)] != 0;
+        }
         const uint32_t self = (uint32_t)i;
-        int32_t *slot_f = P.nbr + i;   // this particle's next list entry (one lane per particle)
-        // the group's lanes relative to this one (cooperative append for T > 1)
-        const unsigned gmask = group_mask<T>();
-        const int gshift = (int)(threadIdx.x & 31u) & ~(T - 1);
-        const unsigned below = (1u << s) - 1u;
-        // phase 1: the float predicate over the stencil's index ranges only records
-        // neighbours; keeping the per-pair work out of this loop keeps the warp converged
-        // while most candidates are rejected.  Rows and end cells whose nearest point is
-        // farther than h (plus a margin above the rounding of these bounds) are skipped:
-        // they hold no particle that passes the predicate, so the lists are unchanged.
-        // With T > 1 the lanes test T consecutive candidates at a time and append the hits
-        // in candidate order (ballot over the group), so every T builds the same list.
-        for (int32_t dz = -R; dz <= R; ++dz) {
-            const int32_t z = cz + dz;
-            if (z < 0 || z >= sc.dims[2]) continue;
-            const float gz = T > 1 ? gap(oz, dz) : 0.0f;
-            for (int32_t dy = -R; dy <= R; ++dy) {
-                const int32_t y = cy + dy;
-                if (y < 0 || y >= sc.dims[1]) continue;
-                int32_t x0 = cx - R, x1 = cx + R;
-                if (T > 1) {   // with one lane the culling's registers cost more than it saves
-                    const float gy = gap(oy, dy);
-                    const float g2 = fmaf(gy, gy, gz * gz);
-                    if (g2 > cull2) continue;
-                    while (x0 < cx && fmaf(gap(ox, x0 - cx), gap(ox, x0 - cx), g2) > cull2) ++x0;
-                    while (x1 > cx && fmaf(gap(ox, x1 - cx), gap(ox, x1 - cx), g2) > cull2) --x1;
-                }
-                x0 = max(x0, 0);
-                x1 = min(x1, sc.dims[0] - 1);
-                const int64_t row = sc.c_off + (int64_t)sc.dims[0] * (y + (int64_t)sc.dims[1] * z);
-                const uint32_t jb = P.cell_start[row + x0], je = P.cell_start[row + x1 + 1];
-                if constexpr (T == 1) {
-                    if (je - jb <= 64u) {
-                        // a row of up to 64 candidates: the predicate only sets bits of a
-                        // mask (no store or counter per candidate, most are rejected), and
-                        // the hits are appended in candidate order from the mask
-                        auto bits = [&](uint32_t b0, uint32_t b1) {
-                            // four candidates per batch: their loads issue together, and their
-                            // hits are combined at fixed shifts before one shift into place
-                            uint32_t mk = 0u;
-                            uint32_t j = b0;
-                            for (; j + 3u < b1; j += 4u) {
-                                float4 pc[4];
+        int passed = 0;
+        {
+            const uint4 own = P.qpos[self >> 1];
+            const uint32_t qx = query_pair(own.x, self & 1u), qy = query_pair(own.y, self & 1u),
+                           qz = query_pair(own.z, self & 1u);
+            const __half2 thr = as_half2(sc.qthr), unit = __float2half2_rn(1.0f / 512.0f), bias = __float2half2_rn(-3.0f);
+            int32_t *slot = P.nbr + i;
+            const int32_t rows = st.ny * st.nz;
+            uint32_t row = st.row;
+            for (int32_t k = 0, y = 0; k < rows; ++k) {
+                const uint32_t jb = P.cell_start[row + (uint32_t)st.x0], je = P.cell_start[row + (uint32_t)st.x1 + 1u];
+                row += st.dx;
+                if (++y == st.ny) { y = 0; row += st.dxy - (uint32_t)st.ny * st.dx; }
+                // 32 candidates from an even index on, eight at a time; a bit set: farther than h
+                for (uint32_t c0 = jb & ~1u; c0 < je; c0 += 32u) {
+                    const uint32_t n = min(je - c0, 32u);
+                    uint32_t far = 0u;
+                    const uint4 *w = P.qpos + (c0 >> 1);
+                    for (uint32_t q = 0u; q < n; q += 8u, w += 4) {
+                        uint4 p[4];
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) pc[u] = __ldg(P.pos_s + j + u);
-                                uint32_t q = 0u;
+                        for (int u = 0; u < 4; ++u) p[u] = __ldg(w + u);
+                        int bits = 0;
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) q |= (uint32_t)(pred_d2_xy2(pixy, pi.z, pc[u]) < h2) << u;
-                                mk |= q << (j - b0);
-                            }
-                            for (; j < b1; ++j) mk |= (uint32_t)(pred_d2_xy2(pixy, pi.z, __ldg(P.pos_s + j)) < h2) << (j - b0);
-                            return mk;
-                        };
-                        uint64_t m = bits(jb, min(je, jb + 32u));
-                        if (je > jb + 32u) m |= (uint64_t)bits(jb + 32u, je) << 32;
-                        // only the stencil's centre row holds the particle itself
-                        if (dz == 0 && dy == 0) m &= ~(1ull << (self - jb));
-                        for (; m != 0ull; m &= m - 1ull) {
-                            if (nn_f < cap_f) *slot_f = (int32_t)(jb + (uint32_t)(__ffsll((long long)m) - 1));
-                            slot_f += NF;
-                            ++nn_f;
+                        for (int u = 0; u < 4; ++u) {
+                            const __half2 dx = __hfma2(as_half2(qx + p[u].x), unit, bias);
+                            const __half2 dy = __hfma2(as_half2(qy + p[u].y), unit, bias);
+                            const __half2 dz = __hfma2(as_half2(qz + p[u].z), unit, bias);
+                            const uint32_t f = __hgt2_mask(__hfma2(dx, dx, __hfma2(dy, dy, __hmul2(dz, dz))), thr);
+                            // bytes 0 and 2 of the masks (-1 or 0) times -4^u and -2 4^u: bits 2u, 2u + 1
+                            bits = __dp4a((int)f, (int)((uint32_t)(uint8_t)(-(1 << (2 * u))) | (uint32_t)(uint8_t)(-(2 << (2 * u))) << 16), bits);
                         }
-                    } else {
-                        // longer rows: a predicated store through a running slot pointer
-                        auto scan = [&](auto check_self) {
-                            for_range<4, 1>(P.pos_s, jb, je, [&](uint32_t j, float4 pj) {
-                                float dx, dy2, dz2;
-                                const float d2 = pred_d2(pi, pj, dx, dy2, dz2);
-                                const bool hit = d2 < h2 && (!decltype(check_self)::value || j != self);
-                                if (hit && nn_f < cap_f) *slot_f = (int32_t)j;
-                                slot_f += hit ? NF : 0;
-                                nn_f += hit;
-                            });
-                        };
-                        if (dz == 0 && dy == 0) scan(std::true_type{});
-                        else scan(std::false_type{});
+                        far |= (uint32_t)bits << q;
                     }
-                } else {
-                    // the group's lanes test T consecutive candidates at a time and append the
-                    // hits in candidate order; full batches of kCand groups load all their
-                    // candidates before the first test (one memory latency per batch)
-                    auto append = [&](uint32_t j, bool hit) {
-                        const unsigned bits = __ballot_sync(gmask, hit) >> gshift;
-                        const int slot = nn_f + __popc(bits & below);
-                        if (hit && slot < cap_f) P.nbr[(int64_t)slot * NF + i] = (int32_t)j;
-                        nn_f += __popc(bits);
-                    };
-                    constexpr int kCand = 4;
-                    uint32_t j0 = jb;
-                    for (; j0 + (uint32_t)(kCand * T) <= je; j0 += (uint32_t)(kCand * T)) {   // uniform in the group
-                        float4 pc[kCand];
-#pragma unroll
-                        for (int u = 0; u < kCand; ++u) pc[u] = __ldg(P.pos_s + j0 + (uint32_t)(u * T + s));
-#pragma unroll
-                        for (int u = 0; u < kCand; ++u) {
-                            const uint32_t j = j0 + (uint32_t)(u * T + s);
-                            float dx, dy2, dz2;
-                            append(j, pred_d2(pi, pc[u], dx, dy2, dz2) < h2 && j != self);
-                        }
-                    }
-                    for (; j0 < je; j0 += (uint32_t)T) {   // uniform in the group
-                        const uint32_t j = j0 + (uint32_t)s;
-                        bool hit = false;
-                        if (j < je) {
-                            float dx, dy2, dz2;
-                            hit = pred_d2(pi, __ldg(P.pos_s + j), dx, dy2, dz2) < h2 && j != self;
-                        }
-                        append(j, hit);
-                    }
-                }
-                if (sc.nb > 0) {
-                    const uint32_t bb = P.bcell_start[row + x0], be = P.bcell_start[row + x1 + 1];
-                    for (uint32_t b0 = bb; b0 < be; b0 += (uint32_t)T) {
-                        const uint32_t b = b0 + (uint32_t)s;
-                        bool hit = false;
-                        if (b < be) {
-                            float dx, dy2, dz2;
-                            hit = pred_d2(pi, __ldg(P.bpos_s + b), dx, dy2, dz2) < h2;
-                        }
-                        const unsigned bits = T == 1 ? (unsigned)hit : (__ballot_sync(gmask, hit) >> gshift);
-                        const int slot = nn_b + __popc(bits & below);
-                        if (hit && slot < cap_b) P.bnbr[(int64_t)slot * NF + i] = (int32_t)b;
-                        nn_b += __popc(bits);
+                    uint32_t near = ~far & (0xffffffffu >> (32u - n));
+                    if (c0 < jb) near &= ~1u;
+                    if (k == st.centre && self - c0 < 32u) near &= ~(1u << (self - c0));
+                    passed += __popc(near);
+                    if (passed > cap_f) near = 0u;   // the exact predicate builds the list instead
+                    for (; near != 0u; near &= near - 1u) {
+                        *slot = (int32_t)(c0 + (uint32_t)__ffs((int)near) - 1u);
+                        slot += NF;
                     }
                 }
             }
         }
-        // the lists were written by the group's lanes: order them before the reads below
-        if (T > 1) __syncwarp(gmask);
+        if (walls) {
+            uint32_t row = st.row;
+            for (int32_t k = 0, y = 0; k < st.ny * st.nz; ++k) {
+                const uint32_t be = P.bcell_start[row + (uint32_t)st.x1 + 1u];
+                for (uint32_t b = P.bcell_start[row + (uint32_t)st.x0]; b < be; ++b) {
+                    float dx, dy, dz;
+                    if (pred_d2(pi, __ldg(P.bpos_s + b), dx, dy, dz) < h2) {
+                        if (nn_b < cap_b) P.bnbr[(int64_t)nn_b * NF + i] = (int32_t)b;
+                        ++nn_b;
+                    }
+                }
+                row += st.dx;
+                if (++y == st.ny) { y = 0; row += st.dxy - (uint32_t)st.ny * st.dx; }
+            }
+        }
+        int total = -1;   // exact count, where the list was built by the exact predicate
+        if (passed > cap_f || !(fmaxf(fmaxf(fabsf(pi.x), fabsf(pi.y)), fabsf(pi.z)) <= sc.qmax)) {
+            total = exact_list(P, st, i, pi, h2, cap_f);
+            passed = min(total, cap_f);
+        }
+        // phase 2: the exact predicate, density, alpha and the warm-start gate
+        const float4 vi = P.vel_s[i];
+        const Spline sp(sc);
+        float w_sum = 0.0f, s1x = 0.0f, s1y = 0.0f, s1z = 0.0f, s2 = 0.0f, div_l = 0.0f;
+        int k = 0;
+        for_list<2, 1, false>(P.nbr, NF, i, 0, passed, [&](int32_t j) {
+            const float4 pj = __ldg(P.pos_s + j);
+            float dx, dy2, dz2;
+            const float d2 = pred_d2(pi, pj, dx, dy2, dz2);
+            if (d2 < h2) {
+                if (nn_f != k) P.nbr[(int64_t)nn_f * NF + i] = j;
+                ++nn_f;
+            }
+            ++k;
+            if (SUM && d2 < h2) {
+                w_sum += spline_w(sqrtf(d2) * sp.inv_h);
+                const float f = grad_factor(sp, d2);
+                const float gx = f * dx, gy = f * dy2, gz = f * dz2;
+                s1x += gx; s1y += gy; s1z += gz;
+                s2 = fmaf(gx, gx, fmaf(gy, gy, fmaf(gz, gz, s2)));
+                if (gate) {
+                    const float4 vj = __ldg(P.vel_s + j);
+                    div_l += (vi.x - vj.x) * gx + (vi.y - vj.y) * gy + (vi.z - vj.z) * gz;
+                }
+            }
+        });
+        const int nb = min(nn_b, cap_b);
+        P.nnf[i] = nn_f;
+        P.nnb[i] = nb;
+        if constexpr (SUM) {
+            float rho_l = sc.m * sc.sigma * w_sum;
+            s1x = sc.m * s1x; s1y = sc.m * s1y; s1z = sc.m * s1z;
+            s2 *= sc.m * sc.m;
+            div_l = sc.m * div_l;
+            if (nb > 0) {
+                float wb = 0.0f, divb = 0.0f;
+                const bool moving = sc.has_moving != 0;
+                for_list<1, 1, false>(P.bnbr, NF, i, 0, nb, [&](int32_t b) {
+                    const float4 pb = __ldg(P.bpos_s + b);
+                    float dx, dy2, dz2;
+                    const float d2 = pred_d2(pi, pb, dx, dy2, dz2);
+                    const float psi = pb.w;
+                    wb += psi * spline_w(sqrtf(d2) * sp.inv_h);
+                    const float f = psi * grad_factor(sp, d2);
+                    const float gx = f * dx, gy = f * dy2, gz = f * dz2;
+                    s1x += gx; s1y += gy; s1z += gz;
+                    if (gate) {
+                        float4 vb = moving ? __ldg(P.bvel_s + b) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        divb += (vi.x - vb.x) * gx + (vi.y - vb.y) * gy + (vi.z - vb.z) * gz;
+                    }
+                });
+                rho_l += sc.sigma * wb;
+                div_l += divb;
+            }
+            const float rho = fmaf(sc.m, sc.sigma, rho_l);
+            const float den = fmaf(s1x, s1x, fmaf(s1y, s1y, fmaf(s1z, s1z, s2)));
+            P.alpha[i] = den > sc.eps_alpha ? rho / den : 0.0f;
+            set_w(P.vel_s, i, rho);
+            float kv0 = 0.0f;
+            if (gate && div_l > 0.0f) kv0 = sc.warm_frac * P.kvprev_s[i] / c.st->dt;
+            P.kvsum[i] = kv0;
+            set_w(P.pos_s, i, kv0 / rho);
+        }
+        if (total >= 0) nn_f = total;
+    }
+    // one atomic per warp: spread over this long sweep they cost less than a block barrier would
+    const int mf = warp_max(nn_f), mb = warp_max(nn_b);
+    if ((threadIdx.x & 31) == 0) {
+        if (mf > 0) atomicMax(&c.st->max_nn_f, mf);
+        if (mb > 0) atomicMax(&c.st->max_nn_b, mb);
+        if (mf > sc.cap_f || mb > sc.cap_b) atomicOr(&c.st->flags, 1);
+    }
+}
+
+// Density, alpha and the warm-start gate of a particle from its lists by T lanes, lane s taking
+// entries s, s + T, ... (every thread of the warp calls it).  FRESH: lists this warp has just
+// written.
+template <int T, bool FRESH>
+__device__ __forceinline__ void density_sums(const Ptrs &P, const Lane<T> &c, float4 pi, int nf, int nb)
+{
+    const SceneDev &sc = *c.sc;
+    const int64_t i = c.i, NF = P.NF;
+    const int s = c.s;
+    const bool gate = sc.warm != 0 && sc.div_on;
+    // this lane's shares of rho - m W(0), sum grad W, sum |grad W|^2 and D rho/Dt
+    float rho_l = 0.0f, s1x = 0.0f, s1y = 0.0f, s1z = 0.0f, s2 = 0.0f, div_l = 0.0f;
+    if (c.valid) {
+        const float4 vi = P.vel_s[i];
         const int32_t *__restrict__ nbr = P.nbr;
         const int32_t *__restrict__ bnbr = P.bnbr;
-        // phase 2: density, alpha and the warm-start gate over the recorded list (this
-        // lane's share of its entries)
         float w_sum = 0.0f, fx = 0.0f, fy = 0.0f, fz = 0.0f, div_f = 0.0f;
         const Spline sp(sc);
-        for_list<2, T, false>(nbr, NF, i, s, min(nn_f, cap_f), [&](int32_t j) {
+        for_list<2, T, !FRESH>(nbr, NF, i, s, nf, [&](int32_t j) {
             const float4 pj = __ldg(P.pos_s + j);
             float dx, dy2, dz2;
             const float d2 = pred_d2(pi, pj, dx, dy2, dz2);
@@ -305,11 +377,10 @@ __global__ void __launch_bounds__(kBlock, T == 1 ? 9 : 8) k_density_alpha(Ptrs P
         s1x = sc.m * fx; s1y = sc.m * fy; s1z = sc.m * fz;
         s2 *= sc.m * sc.m;
         div_l = sc.m * div_f;
-        const int nb = min(nn_b, cap_b);
         if (nb > 0) {
             float wb = 0.0f, divb = 0.0f;
             const bool moving = sc.has_moving != 0;
-            for_list<1, T, false>(bnbr, NF, i, s, nb, [&](int32_t b) {
+            for_list<1, T, !FRESH>(bnbr, NF, i, s, nb, [&](int32_t b) {
                 const float4 pb = __ldg(P.bpos_s + b);
                 float dx, dy2, dz2;
                 const float d2 = pred_d2(pi, pb, dx, dy2, dz2);
@@ -338,12 +409,139 @@ __global__ void __launch_bounds__(kBlock, T == 1 ? 9 : 8) k_density_alpha(Ptrs P
         const float alpha = den > sc.eps_alpha ? rho / den : 0.0f;
         P.alpha[i] = alpha;
         set_w(P.vel_s, i, rho);
-        P.nnf[i] = min(nn_f, sc.cap_f);
-        P.nnb[i] = min(nn_b, sc.cap_b);
         float kv0 = 0.0f;
         if (gate && div_l > 0.0f) kv0 = sc.warm_frac * P.kvprev_s[i] / c.st->dt;
         P.kvsum[i] = kv0;
         set_w(P.pos_s, i, kv0 / rho);
+    }
+}
+
+// The sums where one thread a particle built the lists (k_density<false>) but the context runs
+// two or four lanes.
+template <int T>
+__global__ void __launch_bounds__(kBlock) k_density_sum(Ptrs P)
+{
+    kernel_enter(P.ctl, KID_DENSITY_SUM);
+    const Lane<T> c = lane_ctx<T>(P);
+    const float4 pi = c.valid ? P.pos_s[c.i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    density_sums<T, false>(P, c, pi, c.valid ? P.nnf[c.i] : 0, c.valid ? P.nnb[c.i] : 0);
+}
+
+// The same sweep by T threads a particle, for contexts too small to fill the GPU otherwise: the
+// T lanes test T consecutive candidates at a time with the exact predicate and append the hits
+// in candidate order (ballot over the group), so the list is the same.  Eight blocks per SM (64
+// registers for the batched cooperative append).
+template <int T>
+__global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
+{
+    kernel_enter(P.ctl, KID_DENSITY);
+    const Lane<T> c = lane_ctx<T>(P);
+    const SceneDev &sc = *c.sc;
+    const int64_t i = c.i, NF = P.NF;
+    const int s = c.s;
+    int nn_f = 0, nn_b = 0;  // this lane's neighbours (may exceed its capacity)
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c.valid) {
+        pi = P.pos_s[i];
+        const int32_t cx = cell_coord(pi.x, sc.origin[0], sc.cell, sc.dims[0]);
+        const int32_t cy = cell_coord(pi.y, sc.origin[1], sc.cell, sc.dims[1]);
+        const int32_t cz = cell_coord(pi.z, sc.origin[2], sc.cell, sc.dims[2]);
+        const int32_t R = sc.R;
+        // a boundary particle in the stencil
+        const bool walls = P.bnear[sc.c_off + cx + (int64_t)sc.dims[0] * (cy + (int64_t)sc.dims[1] * cz)] != 0;
+        const float h2 = sc.h2, cull2 = sc.cull2, cs = sc.cell;
+        // offset of the particle inside its cell, per axis: the distance from the particle
+        // to a stencil cell d cells away is at least gap(d) (zero for d = 0)
+        const float ox = pi.x - fmaf((float)cx, cs, sc.origin[0]);
+        const float oy = pi.y - fmaf((float)cy, cs, sc.origin[1]);
+        const float oz = pi.z - fmaf((float)cz, cs, sc.origin[2]);
+        auto gap = [&](float o, int32_t d) {
+            const float g = d < 0 ? fmaf((float)(-d - 1), cs, o) : (d > 0 ? fmaf((float)d, cs, -o) : 0.0f);
+            return fmaxf(g, 0.0f);
+        };
+        const int cap_f = sc.cap_f, cap_b = sc.cap_b;
+        const uint32_t self = (uint32_t)i;
+        // the group's lanes relative to this one (cooperative append)
+        const unsigned gmask = group_mask<T>();
+        const int gshift = (int)(threadIdx.x & 31u) & ~(T - 1);
+        const unsigned below = (1u << s) - 1u;
+        // phase 1: the float predicate over the stencil's index ranges only records
+        // neighbours; keeping the per-pair work out of this loop keeps the warp converged
+        // while most candidates are rejected.  Rows and end cells whose nearest point is
+        // farther than h (plus a margin above the rounding of these bounds) are skipped:
+        // they hold no particle that passes the predicate, so the lists are unchanged.
+        for (int32_t dz = -R; dz <= R; ++dz) {
+            const int32_t z = cz + dz;
+            if (z < 0 || z >= sc.dims[2]) continue;
+            const float gz = gap(oz, dz);
+            for (int32_t dy = -R; dy <= R; ++dy) {
+                const int32_t y = cy + dy;
+                if (y < 0 || y >= sc.dims[1]) continue;
+                int32_t x0 = cx - R, x1 = cx + R;
+                const float gy = gap(oy, dy);
+                const float g2 = fmaf(gy, gy, gz * gz);
+                if (g2 > cull2) continue;
+                while (x0 < cx && fmaf(gap(ox, x0 - cx), gap(ox, x0 - cx), g2) > cull2) ++x0;
+                while (x1 > cx && fmaf(gap(ox, x1 - cx), gap(ox, x1 - cx), g2) > cull2) --x1;
+                x0 = max(x0, 0);
+                x1 = min(x1, sc.dims[0] - 1);
+                const int64_t row = sc.c_off + (int64_t)sc.dims[0] * (y + (int64_t)sc.dims[1] * z);
+                const uint32_t jb = P.cell_start[row + x0], je = P.cell_start[row + x1 + 1];
+                // the group's lanes test T consecutive candidates at a time and append the
+                // hits in candidate order; full batches of kCand groups load all their
+                // candidates before the first test (one memory latency per batch)
+                auto append = [&](uint32_t j, bool hit) {
+                    const unsigned bits = __ballot_sync(gmask, hit) >> gshift;
+                    const int slot = nn_f + __popc(bits & below);
+                    if (hit && slot < cap_f) P.nbr[(int64_t)slot * NF + i] = (int32_t)j;
+                    nn_f += __popc(bits);
+                };
+                constexpr int kCand = 4;
+                uint32_t j0 = jb;
+                for (; j0 + (uint32_t)(kCand * T) <= je; j0 += (uint32_t)(kCand * T)) {   // uniform in the group
+                    float4 pc[kCand];
+#pragma unroll
+                    for (int u = 0; u < kCand; ++u) pc[u] = __ldg(P.pos_s + j0 + (uint32_t)(u * T + s));
+#pragma unroll
+                    for (int u = 0; u < kCand; ++u) {
+                        const uint32_t j = j0 + (uint32_t)(u * T + s);
+                        float dx, dy2, dz2;
+                        append(j, pred_d2(pi, pc[u], dx, dy2, dz2) < h2 && j != self);
+                    }
+                }
+                for (; j0 < je; j0 += (uint32_t)T) {   // uniform in the group
+                    const uint32_t j = j0 + (uint32_t)s;
+                    bool hit = false;
+                    if (j < je) {
+                        float dx, dy2, dz2;
+                        hit = pred_d2(pi, __ldg(P.pos_s + j), dx, dy2, dz2) < h2 && j != self;
+                    }
+                    append(j, hit);
+                }
+                if (walls) {
+                    const uint32_t bb = P.bcell_start[row + x0], be = P.bcell_start[row + x1 + 1];
+                    for (uint32_t b0 = bb; b0 < be; b0 += (uint32_t)T) {
+                        const uint32_t b = b0 + (uint32_t)s;
+                        bool hit = false;
+                        if (b < be) {
+                            float dx, dy2, dz2;
+                            hit = pred_d2(pi, __ldg(P.bpos_s + b), dx, dy2, dz2) < h2;
+                        }
+                        const unsigned bits = __ballot_sync(gmask, hit) >> gshift;
+                        const int slot = nn_b + __popc(bits & below);
+                        if (hit && slot < cap_b) P.bnbr[(int64_t)slot * NF + i] = (int32_t)b;
+                        nn_b += __popc(bits);
+                    }
+                }
+            }
+        }
+        // the lists were written by the group's lanes: order them before the reads below
+        __syncwarp(gmask);
+    }
+    density_sums<T, true>(P, c, pi, min(nn_f, sc.cap_f), min(nn_b, sc.cap_b));
+    if (c.valid && s == 0) {
+        P.nnf[i] = min(nn_f, sc.cap_f);
+        P.nnb[i] = min(nn_b, sc.cap_b);
     }
     // the counts are the same in all lanes of a particle (one atomic per warp: spread over
     // this long sweep they cost less than a block barrier would)
@@ -843,9 +1041,18 @@ void launch_step_begin(const Ptrs &P, cudaStream_t s)
 // of the Jacobi passes from its tuning: (T, B) in {(1, 4), (1, 8), (2, 4), (4, 4)}.
 void launch_density_alpha(const Ptrs &P, cudaStream_t s)
 {
-#define SPH_L(T) k_density_alpha<T><<<P.ntblk, kBlock, 0, s>>>(P)
-    SPH_BY_LANES(P, SPH_L);
-#undef SPH_L
+    // Eight lanes a particle pay only where they are what fills the GPU (one thread against
+    // eight: 8k particles 43 and 28 us, 38k about even); four or two lanes never did (100k: 160 us
+    // with two, 55 with one).  Both write the same lists.
+    if (P.lanes == 8) {
+        k_density_lanes<8><<<P.ntblk, kBlock, 0, s>>>(P);
+    } else if (P.lanes == 1) {
+        k_density<true><<<P.nfblk, kBlock, 0, s>>>(P);
+    } else {
+        k_density<false><<<P.nfblk, kBlock, 0, s>>>(P);
+        if (P.lanes == 4) k_density_sum<4><<<P.ntblk, kBlock, 0, s>>>(P);
+        else k_density_sum<2><<<P.ntblk, kBlock, 0, s>>>(P);
+    }
 }
 void launch_pass_a(const Ptrs &P, int solver, int batch, cudaStream_t s)
 {

@@ -66,12 +66,18 @@ __global__ void __launch_bounds__(kBlock) k_scatter(Ptrs P)
 
 // Copy particle src of the canonical (or original boundary) arrays to sorted slot d.
 template <int WHAT>
-__device__ __forceinline__ void gather_one(const Ptrs &P, uint32_t d, uint32_t src, uint32_t id)
+__device__ __forceinline__ void gather_one(const Ptrs &P, const SceneDev &sc, uint32_t d, uint32_t src, uint32_t id)
 {
     if (WHAT == SORT_FLUID) {
         float4 p = P.pos_c[src];
         p.w = 0.0f;
         P.pos_s[d] = p;
+        // the density sweep's candidate filter: negated coordinates in steps of h/512,
+        // modulo 2^16
+        uint16_t *q = reinterpret_cast<uint16_t *>(P.qpos + (d >> 1)) + (d & 1u);
+        q[0] = (uint16_t)-__float2int_rn((p.x - sc.origin[0]) * sc.qscale);
+        q[2] = (uint16_t)-__float2int_rn((p.y - sc.origin[1]) * sc.qscale);
+        q[4] = (uint16_t)-__float2int_rn((p.z - sc.origin[2]) * sc.qscale);
         P.vel_s[d] = P.vel_c[src];
         P.kprev_s[d] = P.kprev_c[src];
         P.kvprev_s[d] = P.kvprev_c[src];
@@ -114,7 +120,7 @@ __global__ void __launch_bounds__(kBlock) k_rank_gather(Ptrs P)
     uint32_t my = sid[s];
     uint32_t rank = 0;
     for (uint32_t t = b; t < e; ++t) rank += (sid[t] < my) ? 1u : 0u;
-    gather_one<WHAT>(P, b + rank, (WHAT == SORT_FLUID ? P.src_tmp : P.bsrc_tmp)[s], my);
+    gather_one<WHAT>(P, sc, b + rank, (WHAT == SORT_FLUID ? P.src_tmp : P.bsrc_tmp)[s], my);
 }
 
 // 5) the queued crowded cells: each block takes cells of the queue in turn, sorts the
@@ -135,7 +141,9 @@ __global__ void __launch_bounds__(kLargeThreads) k_rank_large(Ptrs P)
         const uint32_t cell = large[q];
         const uint32_t b = start[cell], e = start[cell + 1];
         block_sort_segment(sid, src, sid2, src2, b, e);
-        for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) gather_one<WHAT>(P, d, src[d], sid[d]);
+        int32_t s0 = 0;   // the cell's scene: cells of a context are numbered scene after scene
+        while (s0 + 1 < P.nscenes && (int64_t)cell >= P.scenes[s0 + 1].c_off) ++s0;
+        for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) gather_one<WHAT>(P, P.scenes[s0], d, src[d], sid[d]);
         __syncthreads();
     }
 }

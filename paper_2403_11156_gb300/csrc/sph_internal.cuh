@@ -58,6 +58,8 @@ struct SceneDev {
     int32_t strong;                   // strong rigid coupling: bodies pushed during the solves
     float learned_frac;               // fraction of the network's stiffness warm-starting it
     int32_t learned_gate;             // the network runs only above this many density iterations
+    float qscale, qmax;               // candidate filter: 512 / h, largest coordinate it holds for
+    uint32_t qthr;                    // its threshold on (d/h)^2 as a pair of halves
     double err_scale;                 // 1 / (nf rho0): a solve's error sum to its mean per rho0
 };
 
@@ -161,7 +163,9 @@ enum KernelId : uint32_t {
     KID_CG_BETA = 36,
     KID_BTOUCH = 37,
     KID_RANK_LARGE_F = 38,
-    KID_RANK_LARGE_B = 39
+    KID_RANK_LARGE_B = 39,
+    KID_BNEAR = 40,
+    KID_DENSITY_SUM = 41
 };
 
 static_assert(KID_STEP_BEGIN == SPH_KID_STEP_BEGIN, "trace id");
@@ -203,6 +207,8 @@ static_assert(KID_CG_BETA == SPH_KID_CG_BETA, "trace id");
 static_assert(KID_BTOUCH == SPH_KID_BTOUCH, "trace id");
 static_assert(KID_RANK_LARGE_F == SPH_KID_RANK_LARGE_F, "trace id");
 static_assert(KID_RANK_LARGE_B == SPH_KID_RANK_LARGE_B, "trace id");
+static_assert(KID_BNEAR == SPH_KID_BNEAR, "trace id");
+static_assert(KID_DENSITY_SUM == SPH_KID_DENSITY_SUM, "trace id");
 
 // First thread of every kernel: count the launch and, when tracing, stamp its start.
 __device__ __forceinline__ void kernel_enter(Control *ctl, uint32_t id)
@@ -240,6 +246,8 @@ struct Ptrs {
     int32_t *id_c, *id_s;
     int32_t *nnf, *nnb;               // neighbour counts (capped at the list capacity)
     int32_t *nbr, *bnbr;
+    uint4 *qpos;                      // [NF / 2 + 8] sorted positions, negated, in 16-bit steps
+                                      // of h/512, two particles a word: (x x', y y', z z', -)
     float *feat;                      // [NF][4]
     // grid scratch (fluid)
     uint32_t *cell_count, *cell_start;
@@ -252,6 +260,7 @@ struct Ptrs {
     int32_t *bid_s;
     int32_t *bbody_s;
     uint32_t *bcell_count, *bcell_start;
+    uint8_t *bnear;                   // [NC] whether the cell's stencil holds a boundary particle
     uint32_t *bkey_tmp, *bslot_tmp, *bsid_tmp, *bsrc_tmp, *bcell_tmp;
     uint32_t *large_f, *large_b;      // crowded cells of the fluid / boundary sort (lists)
     // reductions
@@ -318,24 +327,12 @@ __device__ __forceinline__ float pred_d2(float4 a, float4 b, float &dx, float &d
     return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// The same d2 with the x and y differences and squares as packed FP32 pairs (axy holds a.x in
-// its low half, a.y in its high half): each half rounds like the scalar operation, and the
-// sums keep the order above, so the value is identical, in fewer instructions.
+// Two floats in one register pair, for the packed FP32 instructions.
 __device__ __forceinline__ unsigned long long pack_xy(float x, float y)
 {
     unsigned long long r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
     return r;
-}
-__device__ __forceinline__ float pred_d2_xy2(unsigned long long axy, float az, float4 b)
-{
-    unsigned long long d, q;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(axy), "l"(pack_xy(b.x, b.y)));
-    asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(q) : "l"(d));
-    float qx, qy;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(qx), "=f"(qy) : "l"(q));
-    const float dz = __fsub_rn(az, b.z);
-    return __fadd_rn(__fadd_rn(qx, qy), __fmul_rn(dz, dz));
 }
 
 enum SortWhat { SORT_FLUID = 0, SORT_BOUNDARY = 1 };
@@ -387,6 +384,7 @@ cudaError_t post_height_map(const float4 *pos, int64_t n, const float lo[2], con
 
 // ------------------------------------------------------------------ rigid (sph_rigid.cu)
 void launch_boundary_update(const Ptrs &P, cudaStream_t s);
+void launch_boundary_near(const Ptrs &P, cudaStream_t s);
 void launch_boundary_psi(const Ptrs &P, cudaStream_t s);
 void launch_body_force(const Ptrs &P, cudaStream_t s);
 void launch_body_reduce(const Ptrs &P, cudaStream_t s);

@@ -9,6 +9,8 @@
 //    per body with its torque in FP64 and reduced in a fixed order.
 #include "sph_sweep.cuh"
 
+#include <algorithm>
+
 namespace sph {
 
 namespace {
@@ -73,6 +75,29 @@ __global__ void __launch_bounds__(kBlock) k_boundary_psi(Ptrs P)
         }
     }
     reinterpret_cast<float *>(P.bpos_s + b)[3] = sc.rho0 / (sc.sigma * (1.0f + ws));
+}
+
+// Which cells' stencils hold a boundary particle: the density sweep of the others, most of the
+// fluid, looks up no boundary rows (18 loads a particle).
+__global__ void __launch_bounds__(256) k_boundary_near(Ptrs P)
+{
+    kernel_enter(P.ctl, KID_BNEAR);
+    for (int64_t cell = (int64_t)blockIdx.x * 256 + threadIdx.x; cell < P.NC; cell += (int64_t)gridDim.x * 256) {
+        int32_t s = 0;
+        while (s + 1 < P.nscenes && cell >= P.scenes[s + 1].c_off) ++s;
+        const SceneDev &sc = P.scenes[s];
+        const uint32_t k = (uint32_t)(cell - sc.c_off), row = k / (uint32_t)sc.dims[0];
+        const int32_t x = (int32_t)(k - row * (uint32_t)sc.dims[0]), z = (int32_t)(row / (uint32_t)sc.dims[1]),
+                      y = (int32_t)(row - (uint32_t)z * (uint32_t)sc.dims[1]), R = sc.R;
+        const int32_t x0 = max(x - R, 0), x1 = min(x + R, sc.dims[0] - 1);
+        bool any = false;
+        for (int32_t w = max(z - R, 0); w <= min(z + R, sc.dims[2] - 1); ++w)
+            for (int32_t v = max(y - R, 0); v <= min(y + R, sc.dims[1] - 1); ++v) {
+                const uint32_t *c = P.bcell_start + sc.c_off + (int64_t)sc.dims[0] * (v + (int64_t)sc.dims[1] * w);
+                any |= c[x0] != c[x1 + 1];
+            }
+        P.bnear[cell] = any ? 1 : 0;
+    }
 }
 
 // Force and torque of the fluid on each body of the scene (the T lanes of a particle share
@@ -331,6 +356,10 @@ void launch_strong_update(const Ptrs &P, int phase, cudaStream_t s)
 void launch_boundary_update(const Ptrs &P, cudaStream_t s)
 {
     if (P.nbblk) k_boundary_update<<<P.nbblk, kBlock, 0, s>>>(P);
+}
+void launch_boundary_near(const Ptrs &P, cudaStream_t s)
+{
+    if (P.nbblk) k_boundary_near<<<(int)std::min<int64_t>((P.NC + 255) / 256, 152 * 8), 256, 0, s>>>(P);
 }
 void launch_boundary_psi(const Ptrs &P, cudaStream_t s)
 {

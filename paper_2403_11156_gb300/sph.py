@@ -46,7 +46,8 @@ KERNEL_IDS = {i + 1: n for i, n in enumerate([
     "advect", "step_end", "set_dt", "boundary_update", "boundary_psi", "body_force", "body_reduce",
     "cg_init", "cg_ap", "cg_xr", "cg_p", "mlp_warm", "body_force_inc", "body_apply",
     "boundary_vel", "div_check", "dens_check", "cg_alpha", "cg_beta", "body_touch",
-    "rank_large_fluid", "rank_large_boundary"])}
+    "rank_large_fluid", "rank_large_boundary", "boundary_near",
+    "density_sum"])}
 
 
 class SphError(RuntimeError):
