@@ -399,6 +399,8 @@ sph_status sph_mlp_train(const float *features, const float *labels, int64_t n, 
 #define SPH_KID_RANK_LARGE_B 39   /* crowded cells of the boundary sort, block-sorted */
 #define SPH_KID_BNEAR 40          /* cells whose stencil holds a boundary particle */
 #define SPH_KID_DENSITY_SUM 41    /* density sums over finished lists, two or four lanes */
+#define SPH_KID_SOLVE0 42         /* a whole divergence solve in one launch */
+#define SPH_KID_SOLVE1 43         /* a whole density solve in one launch */
 
 /* Device trace for profiling graph replays: with capacity > 0 every kernel's first thread
  * records (globaltimer_ns << 8 | kernel id) in a device ring of that many entries (the

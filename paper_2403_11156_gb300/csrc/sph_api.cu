@@ -87,8 +87,10 @@ struct sph_ctx {
     std::vector<int32_t> nbody_scene;
     int max_bodies = 0;
     int64_t nbr_entries = 0;             // of the fluid neighbour lists
+    int solve_grid = 0;                  // blocks of the one-launch solves, 0: separate kernels
     bool any_moving = false, any_div = false, any_warm_div = false, any_warm = false,
-         any_learned = false, any_bodies = false, any_implicit = false, any_wcsph = false, any_strong = false;
+         any_learned = false, any_bodies = false, any_implicit = false, any_wcsph = false, any_strong = false,
+         any_dens = false;
     Ptrs P{};
     SceneDev *d_scenes = nullptr;
 
@@ -545,6 +547,12 @@ sph_status enqueue_step(sph_ctx *c, cudaStream_t s, bool capture)
         const char *na = solver == 0 ? "div_pass_a" : "dens_pass_a";
         const char *nb = solver == 0 ? "div_pass_b" : "dens_pass_b";
         const char *nc = solver == 0 ? "div_check" : "dens_check";
+        if (c->solve_grid > 0) {
+            cudaError_t e = cudaSuccess;
+            run(c, s, solver == 0 ? "div_solve" : "dens_solve", [&] { e = launch_solve(P, solver, c->solve_grid, s); });
+            CK(e);
+            return SPH_OK;
+        }
         return device_loop([&](cudaStream_t q, cudaGraphConditionalHandle h, int use) {
             run(c, q, na, [&] { launch_pass_a(P, solver, c->batch, q); });
             run(c, q, nb, [&] { launch_pass_b(P, solver, 0, c->batch, q); });
@@ -583,7 +591,7 @@ sph_status enqueue_step(sph_ctx *c, cudaStream_t s, bool capture)
         run(c, s, "dens_warm_pass_b", [&] { launch_pass_b(P, 1, 1, c->batch, s); });
         if (c->any_strong) run(c, s, "strong_coupling", [&] { launch_strong_update(P, 3, s); });
     }
-    if ((st = loop(1)) != SPH_OK) return st;
+    if (c->any_dens && (st = loop(1)) != SPH_OK) return st;
     if (c->any_bodies) {
         run(c, s, "body_force", [&] { launch_body_force(P, s); });
         run(c, s, "body_reduce", [&] { launch_body_reduce(P, s); });
@@ -787,6 +795,7 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
         c->any_learned |= q.warm == 2;
         c->any_wcsph |= q.solver == SPH_SOLVER_WCSPH;
         c->any_strong |= q.strong != 0;
+        c->any_dens |= q.max_it[1] > 0;   // (not WCSPH, which takes its pressure in one pass)
         c->any_implicit |= d.viscosity_mode == 3;
     }
     if (NC >= ((int64_t)1 << 32) - 1 || NF >= ((int64_t)1 << 31) || (double)NF * cap_f > 4.0e10)
@@ -1008,6 +1017,8 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
     if (c->any_learned && mlp_prepare_kernels() != cudaSuccess)
         return bail(fail(c, SPH_ECUDA, "network kernel attributes could not be set"));
     if (cudaStreamSynchronize(s) != cudaSuccess) return bail(fail(c, SPH_ECUDA, "create: %s", cudaGetErrorString(cudaGetLastError())));
+    // strongly coupled bodies are updated inside the solves' iterations, by their own kernels
+    c->solve_grid = c->any_strong ? 0 : solve_grid(P, c->batch);
     sph_status gs = build_graph(c);
     if (gs != SPH_OK) return bail(gs);
     *out = c;

@@ -13,7 +13,7 @@
 #include <cuda_fp16.h>
 #include <math_constants.h>
 
-#include <type_traits>
+#include <algorithm>
 
 #include "sph_sweep.cuh"
 
@@ -559,16 +559,16 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
 // Sec. 3.5); group_sum of the shares is the full sum.
 constexpr int kBatch = 4;
 
-template <int B, int T>
+template <int B, int T, bool NC = true>
 __device__ __forceinline__ float drho_dt_lane(const Ptrs &P, const SceneDev &sc, int64_t i, int s, float4 pi,
-                                              float4 vi, const float4 *__restrict__ V)
+                                              float4 vi, const float4 *V)
 {
     const int64_t NF = P.NF;
     const Spline sp(sc);
     float acc = 0.0f;
     for_list<B, T>(P.nbr, NF, i, s, P.nnf[i], [&](int32_t j) {
-        const float4 pj = __ldg(P.pos_s + j);
-        const float4 vj = __ldg(V + j);
+        const float4 pj = ld4<NC>(P.pos_s + j);
+        const float4 vj = ld4<NC>(V + j);
         const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
         const float f = grad_factor(sp, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
         acc = fmaf(f, (vi.x - vj.x) * dx + (vi.y - vj.y) * dy + (vi.z - vj.z) * dz, acc);
@@ -592,12 +592,10 @@ __device__ __forceinline__ float drho_dt_lane(const Ptrs &P, const SceneDev &sc,
 // Pass A of a Jacobi iteration (Alg. ppe_solver "refine p"): the source term of
 // Eq. velocity_source (solver 0) or Eq. density_source with rho* (solver 1), the
 // stiffness kappa_i = alpha_i e_i / dt^(1 or 2), and the block's FP64 error partial.
-template <int S, int B, int T>
-__global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
+template <int S, int B, int T, bool NC>
+__device__ __forceinline__ void pass_a(const Ptrs &P, int32_t block, double *sh)
 {
-    __shared__ double sh[kBlock / 32];
-    kernel_enter(P.ctl, (KID_PASS_A0 + S));
-    const Lane<T> c = lane_ctx<T>(P);
+    const Lane<T> c = lane_ctx<T>(P, block);
     const SceneDev &sc = *c.sc;
     SceneState &st = *c.st;
     if (!solver_active(sc, st, S)) return;  // uniform per block
@@ -609,7 +607,7 @@ __global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
     if (c.valid) {
         pi = P.pos_s[i];
         vi = V[i];
-        D = drho_dt_lane<B, T>(P, sc, i, c.s, pi, vi, V);
+        D = drho_dt_lane<B, T, NC>(P, sc, i, c.s, pi, vi, V);
     }
     D = group_sum<T>(D);
     double e = 0.0;
@@ -640,7 +638,15 @@ __global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
     // the block's FP64 error partial; pass B folds the partials and the check kernel sums
     // the folds in a fixed order (no last-block step here: pass A only has to finish)
     const double bsum = block_sum(e, sh);
-    if (threadIdx.x == 0) P.partial[blockIdx.x] = bsum;
+    if (threadIdx.x == 0) P.partial[block] = bsum;
+}
+
+template <int S, int B, int T>
+__global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
+{
+    __shared__ double sh[kBlock / 32];
+    kernel_enter(P.ctl, (KID_PASS_A0 + S));
+    pass_a<S, B, T, true>(P, (int32_t)blockIdx.x, sh);
 }
 
 // Pass B (Alg. ppe_solver "update v*"): pressure acceleration of Sec. 3.3 Eq.
@@ -653,11 +659,10 @@ __global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
 // (measured on the 1.2M scene: 84 -> 80 us per density launch, 90 -> 81 per divergence
 // launch).  Every other variant keeps the compiler's choice (a minimum of 0 blocks): the warm
 // pass already fits in 40 registers, and batch 8 would spill 152 bytes.
-template <int S, int WARM, int B, int T>
-__global__ void __launch_bounds__(kBlock, (T == 1 && WARM == 0 && B == 4) ? 11 : 0) k_pass_b(Ptrs P)
+template <int S, int WARM, int B, int T, bool NC>
+__device__ __forceinline__ void pass_b(const Ptrs &P, int32_t block)
 {
-    kernel_enter(P.ctl, (WARM ? KID_PASS_B0W + S : KID_PASS_B0 + S));
-    const Lane<T> c = lane_ctx<T>(P);
+    const Lane<T> c = lane_ctx<T>(P, block);
     const SceneDev &sc = *c.sc;
     SceneState &st = *c.st;
     // uniform per block; WCSPH scenes apply their equation-of-state pressure here.  In the
@@ -673,7 +678,7 @@ __global__ void __launch_bounds__(kBlock, (T == 1 && WARM == 0 && B == 4) ? 11 :
             const float ki = pi.w;
             const Spline sp(sc);
             for_list<B, T>(P.nbr, NF, i, s, P.nnf[i], [&](int32_t j) {
-                const float4 pj = __ldg(P.pos_s + j);
+                const float4 pj = ld4<NC>(P.pos_s + j);
                 const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
                 const float f = grad_factor(sp, fmaf(dx, dx, fmaf(dy, dy, dz * dz))) * (ki + pj.w);
                 ax = fmaf(f, dx, ax); ay = fmaf(f, dy, ay); az = fmaf(f, dz, az);
@@ -703,15 +708,22 @@ __global__ void __launch_bounds__(kBlock, (T == 1 && WARM == 0 && B == 4) ? 11 :
     // fold pass A's error partials: the scene's first ceil(count / F) blocks each sum F
     // consecutive ones in block order (the check kernel, a later launch, sums the folds)
     if (run && threadIdx.x == 0) {
-        const int32_t lb = (int32_t)blockIdx.x - sc.tblk_first;
+        const int32_t lb = block - sc.tblk_first;
         const int32_t F = fold_size(sc.tblk_count);
         if (lb < (sc.tblk_count + F - 1) / F) {
             const int32_t k0 = lb * F, k1 = min(k0 + F, sc.tblk_count);
             double t = 0.0;
             for (int32_t k = k0; k < k1; ++k) t += __ldcg(P.partial + sc.tblk_first + k);
-            P.partial2[blockIdx.x] = t;
+            P.partial2[block] = t;
         }
     }
+}
+
+template <int S, int WARM, int B, int T>
+__global__ void __launch_bounds__(kBlock, (T == 1 && WARM == 0 && B == 4) ? 11 : 0) k_pass_b(Ptrs P)
+{
+    kernel_enter(P.ctl, (WARM ? KID_PASS_B0W + S : KID_PASS_B0 + S));
+    pass_b<S, WARM, B, T, true>(P, (int32_t)blockIdx.x);
 }
 
 // Convergence test of one Jacobi iteration (Alg. ppe_solver's loop condition), one block
@@ -722,15 +734,12 @@ __global__ void __launch_bounds__(kBlock, (T == 1 && WARM == 0 && B == 4) ? 11 :
 constexpr int kCheckThreads = 1024;
 
 template <int S>
-__global__ void __launch_bounds__(kCheckThreads) k_solver_check(Ptrs P, cudaGraphConditionalHandle handle,
-                                                               int use_handle)
+__device__ __forceinline__ uint32_t solver_check(const Ptrs &P, int *s_any)
 {
-    __shared__ int s_any;
-    kernel_enter(P.ctl, KID_CHECK0 + S);
-    if (threadIdx.x == 0) s_any = 0;
+    if (threadIdx.x == 0) *s_any = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = warp; q < P.nscenes; q += kCheckThreads / 32) {
+    for (int q = warp; q < P.nscenes; q += (int)(blockDim.x / 32)) {
         const SceneDev &qd = P.scenes[q];
         SceneState &qs = P.st[q];
         if (!solver_active(qd, qs, S)) continue;   // its pass A and B did not run
@@ -748,12 +757,12 @@ __global__ void __launch_bounds__(kCheckThreads) k_solver_check(Ptrs P, cudaGrap
             qs.it[S] += 1;
             qs.total_it[S] += 1;
             if (!solver_active(qd, qs, S) && qs.err[S] > (double)qd.eta[S]) qs.flags |= 2;
-            if (solver_active(qd, qs, S)) atomicOr(&s_any, 1);
+            if (solver_active(qd, qs, S)) atomicOr(s_any, 1);
         }
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    uint32_t any = s_any;
+    if (threadIdx.x != 0) return 0u;
+    uint32_t any = *s_any;
     uint32_t guard = ++P.ctl->loop_guard;
     if (guard > 100000u) {
         any = 0;
@@ -761,7 +770,41 @@ __global__ void __launch_bounds__(kCheckThreads) k_solver_check(Ptrs P, cudaGrap
     }
     if (!any) P.ctl->loop_guard = 0;
     P.ctl->loop_flag = any;
-    if (use_handle) cudaGraphSetConditional(handle, any);
+    return any;
+}
+
+template <int S>
+__global__ void __launch_bounds__(kCheckThreads) k_solver_check(Ptrs P, cudaGraphConditionalHandle handle,
+                                                               int use_handle)
+{
+    __shared__ int s_any;
+    kernel_enter(P.ctl, KID_CHECK0 + S);
+    const uint32_t any = solver_check<S>(P, &s_any);
+    if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, any);
+}
+
+// A whole Jacobi solve in one cooperative launch: pass A, barrier, pass B, barrier with the
+// convergence test in the block that arrives last, until no scene goes on.  The arithmetic and
+// every order of summation are those of the separate kernels.  For contexts whose sweep blocks
+// are all resident at once: there an iteration's launches, one-block check and while node
+// (14 us) outweigh its passes; 8k particles: 4 steps 533 -> 480 us.  With more blocks a block's
+// second round waits for nothing else to fill the SM and the separate kernels win (20k
+// particles in two rounds 257 us a step against 236, 100k 447 against 433, 1.2M 2472 against 2376).
+constexpr int kSolveBlocksPerSm = 8;
+template <int S, int T>
+__global__ void __launch_bounds__(kBlock, kSolveBlocksPerSm) k_solve(const __grid_constant__ Ptrs P)
+{
+    __shared__ double sh[kBlock / 32];
+    __shared__ int s_any;
+    kernel_enter(P.ctl, KID_SOLVE0 + S);
+    uint32_t phase = *reinterpret_cast<volatile uint32_t *>(&P.ctl->bar.gen);
+    for (;;) {
+        for (int32_t b = (int32_t)blockIdx.x; b < P.ntblk; b += (int32_t)gridDim.x) pass_a<S, kBatch, T, false>(P, b, sh);
+        if (!grid_barrier(&P.ctl->bar, &P.ctl->error, phase)) return;
+        for (int32_t b = (int32_t)blockIdx.x; b < P.ntblk; b += (int32_t)gridDim.x) pass_b<S, 0, kBatch, T, false>(P, b);
+        if (!grid_barrier(&P.ctl->bar, &P.ctl->error, phase, [&] { solver_check<S>(P, &s_any); })) return;
+        if (*reinterpret_cast<volatile uint32_t *>(&P.ctl->loop_flag) == 0u) return;
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -1084,6 +1127,38 @@ void launch_solver_check(const Ptrs &P, int solver, cudaGraphConditionalHandle h
 {
     if (solver == 0) k_solver_check<0><<<1, kCheckThreads, 0, s>>>(P, h, use_handle);
     else k_solver_check<1><<<1, kCheckThreads, 0, s>>>(P, h, use_handle);
+}
+template <int T>
+static const void *solve_kernel(int solver)
+{
+    return solver == 0 ? reinterpret_cast<const void *>(&k_solve<0, T>) : reinterpret_cast<const void *>(&k_solve<1, T>);
+}
+static const void *solve_kernel(const Ptrs &P, int solver)
+{
+    return P.lanes == 8 ? solve_kernel<8>(solver) : (P.lanes == 4 ? solve_kernel<4>(solver)
+                                                                  : (P.lanes == 2 ? solve_kernel<2>(solver) : solve_kernel<1>(solver)));
+}
+int solve_grid(const Ptrs &P, int batch)
+{
+    // the check walks the scenes with four warps; the passes with eight gathers in flight keep
+    // their own kernels
+    if (batch != kBatch || P.nscenes > kLoopScenes || P.ntblk < 1) return 0;
+    int dev = 0, nsm = 0, coop = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+        return 0;
+    int resident = 0;
+    for (int solver = 0; solver < 2; ++solver) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, solve_kernel(P, solver), kBlock, 0) != cudaSuccess) return 0;
+        resident = solver == 0 ? per * nsm : std::min(resident, per * nsm);
+    }
+    if (resident < 1 || P.ntblk > resident) return 0;
+    return std::min(P.ntblk, resident);
+}
+cudaError_t launch_solve(const Ptrs &P, int solver, int grid, cudaStream_t s)
+{
+    void *args[] = {const_cast<Ptrs *>(&P)};
+    return cudaLaunchCooperativeKernel(solve_kernel(P, solver), dim3((unsigned)grid), dim3(kBlock), args, 0, s);
 }
 void launch_nonpressure(const Ptrs &P, cudaStream_t s)
 {

@@ -104,6 +104,11 @@ struct ScanCtl {
     int32_t pad;
 };
 
+// Barrier over the blocks of one cooperative launch: blocks arrived, completed barriers.
+struct GridBar {
+    uint32_t count, gen;
+};
+
 // Context-wide control words (device).
 struct Control {
     uint32_t probe_flag;              // never set: the wait of sph_probe_wait_timeout
@@ -121,6 +126,7 @@ struct Control {
     int32_t mlp_n;                    // rows the warm-start network runs on this step
     int32_t pad1;
     int32_t nlarge[2];                // crowded cells of the fluid (0) / boundary (1) sort
+    GridBar bar;                      // barrier of the cooperative solve kernels
 };
 
 // Kernel identifiers of the device trace.
@@ -165,7 +171,9 @@ enum KernelId : uint32_t {
     KID_RANK_LARGE_F = 38,
     KID_RANK_LARGE_B = 39,
     KID_BNEAR = 40,
-    KID_DENSITY_SUM = 41
+    KID_DENSITY_SUM = 41,
+    KID_SOLVE0 = 42,
+    KID_SOLVE1 = 43
 };
 
 static_assert(KID_STEP_BEGIN == SPH_KID_STEP_BEGIN, "trace id");
@@ -209,6 +217,8 @@ static_assert(KID_RANK_LARGE_F == SPH_KID_RANK_LARGE_F, "trace id");
 static_assert(KID_RANK_LARGE_B == SPH_KID_RANK_LARGE_B, "trace id");
 static_assert(KID_BNEAR == SPH_KID_BNEAR, "trace id");
 static_assert(KID_DENSITY_SUM == SPH_KID_DENSITY_SUM, "trace id");
+static_assert(KID_SOLVE0 == SPH_KID_SOLVE0, "trace id");
+static_assert(KID_SOLVE1 == SPH_KID_SOLVE1, "trace id");
 
 // First thread of every kernel: count the launch and, when tracing, stamp its start.
 __device__ __forceinline__ void kernel_enter(Control *ctl, uint32_t id)
@@ -358,6 +368,8 @@ void launch_density_alpha(const Ptrs &P, cudaStream_t s);
 void launch_pass_a(const Ptrs &P, int solver, int batch, cudaStream_t s);
 void launch_pass_b(const Ptrs &P, int solver, int warm, int batch, cudaStream_t s);
 void launch_solver_check(const Ptrs &P, int solver, cudaGraphConditionalHandle h, int use_handle, cudaStream_t s);
+int solve_grid(const Ptrs &P, int batch);   // blocks of launch_solve, 0: use the separate kernels
+cudaError_t launch_solve(const Ptrs &P, int solver, int grid, cudaStream_t s);
 void launch_nonpressure(const Ptrs &P, cudaStream_t s);
 void launch_warm_density(const Ptrs &P, cudaStream_t s);
 void launch_advect(const Ptrs &P, cudaStream_t s);

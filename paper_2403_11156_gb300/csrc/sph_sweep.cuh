@@ -53,17 +53,78 @@ struct Lane {
 
 // Particle and lane of this thread in a sweep launched over the sweep-block table.
 template <int T>
-__device__ __forceinline__ Lane<T> lane_ctx(const Ptrs &P)
+__device__ __forceinline__ Lane<T> lane_ctx(const Ptrs &P, int32_t block)
 {
     Lane<T> c;
-    const int32_t sidx = P.tblk_scene[blockIdx.x];
+    const int32_t sidx = P.tblk_scene[block];
     c.sc = &P.scenes[sidx];
     c.st = &P.st[sidx];
-    const int64_t local = (int64_t)(blockIdx.x - c.sc->tblk_first) * (kBlock / T) + threadIdx.x / T;
+    const int64_t local = (int64_t)(block - c.sc->tblk_first) * (kBlock / T) + threadIdx.x / T;
     c.s = (int)(threadIdx.x % T);
     c.valid = local < c.sc->nf;
     c.i = c.sc->f_off + local;
     return c;
+}
+
+template <int T>
+__device__ __forceinline__ Lane<T> lane_ctx(const Ptrs &P) { return lane_ctx<T>(P, (int32_t)blockIdx.x); }
+
+// Gathered particle data: through the read-only path where the kernel does not write it (NC),
+// plain where other blocks of the same launch have.
+template <bool NC>
+__device__ __forceinline__ float4 ld4(const float4 *p)
+{
+    return NC ? __ldg(p) : *p;
+}
+
+// Barrier over all blocks of a cooperative launch, in two halves.  grid_arrive: thread 0 of the
+// block that arrives last gets true.  grid_leave: that thread lets the others go, the others
+// wait; phase is the barrier's generation, kept by the caller (bar->gen before the first).
+// Bounded: a block that waits in vain records it and returns false, and the others follow.
+constexpr int kLoopScenes = 16;   // scenes one block's four warps test between two phases
+constexpr uint32_t kBarrierSpins = 1u << 21;
+__device__ __forceinline__ bool grid_arrive(GridBar *bar)
+{
+    __syncthreads();
+    if (threadIdx.x != 0) return false;
+    uint32_t n;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(n) : "l"(&bar->count) : "memory");
+    return n == gridDim.x - 1u;
+}
+__device__ __forceinline__ bool grid_leave(GridBar *bar, int32_t *error, uint32_t &phase, bool last)
+{
+    bool ok = true;
+    ++phase;
+    if (threadIdx.x == 0) {
+        if (last) {
+            bar->count = 0u;
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&bar->gen), "r"(phase) : "memory");
+        } else {
+            uint32_t g, spins = 0;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&bar->gen) : "memory");
+            } while (g != phase && ++spins < kBarrierSpins);
+            if (g != phase) {
+                atomicExch(error, 5);
+                ok = false;
+            }
+        }
+    }
+    return __syncthreads_and(ok);
+}
+__device__ __forceinline__ bool grid_barrier(GridBar *bar, int32_t *error, uint32_t &phase)
+{
+    const bool last = grid_arrive(bar);
+    return grid_leave(bar, error, phase, last);
+}
+// The same with between(), run by the whole block that arrives last before it lets the others go.
+template <typename F>
+__device__ __forceinline__ bool grid_barrier(GridBar *bar, int32_t *error, uint32_t &phase, F &&between)
+{
+    const bool last = grid_arrive(bar);
+    if (__syncthreads_or(last)) between();
+    __syncthreads();
+    return grid_leave(bar, error, phase, last);
 }
 
 // Sum over the T lanes of a particle; every thread of the warp must call it.

@@ -47,7 +47,7 @@ KERNEL_IDS = {i + 1: n for i, n in enumerate([
     "cg_init", "cg_ap", "cg_xr", "cg_p", "mlp_warm", "body_force_inc", "body_apply",
     "boundary_vel", "div_check", "dens_check", "cg_alpha", "cg_beta", "body_touch",
     "rank_large_fluid", "rank_large_boundary", "boundary_near",
-    "density_sum"])}
+    "density_sum", "div_solve", "dens_solve"])}
 
 
 class SphError(RuntimeError):
