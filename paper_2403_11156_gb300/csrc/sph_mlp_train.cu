@@ -16,6 +16,7 @@
 #include "sph.h"
 #include "sph_gelu.cuh"
 #include "sph_internal.cuh"
+#include "sph_sweep.cuh"
 #include "sph_tc.cuh"
 
 namespace sph {
@@ -144,21 +145,47 @@ __device__ __forceinline__ void gelu_grad_erff(float h0, float h1, gelu::f2 &g, 
 // of the output: Adam divides by the gradient's own size, so that over hundreds of steps a
 // last-bit change of an activation, where it moves a BF16 operand's rounding, grows a
 // thousandfold (small batches are bound by latency, not by the formula).
-template <bool ONCE>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
-    k_mlp_grad(const float *__restrict__ w, const float4 *__restrict__ F, const float *__restrict__ T, int64_t n,
-               int64_t batch_begin, int64_t batch_size, uint64_t pa, uint64_t pc, float *grad, double *loss, int *err)
+//
+// grad_tiles is the walk of one CTA over its tiles of one batch (every thread calls it); the
+// kernels around it own the tensor memory and the mbarrier, whose phase and state a walk carries
+// on.  next: the first tile's sample of this thread, loaded by the caller ahead of time.
+struct Walk {
+    uint32_t phase = 0;   // of the mbarrier
+    bool good = true;     // no wait gave up
+};
+struct Sample {
+    float4 f;
+    float target;
+    bool valid;
+};
+__device__ __forceinline__ Sample load_sample(const float4 *__restrict__ F, const float *__restrict__ T, int64_t n,
+                                              int64_t batch_begin, int64_t batch_size, uint64_t pa, uint64_t pc,
+                                              int64_t tile)
 {
-    extern __shared__ __align__(1024) unsigned char sm[];
+    const int64_t pos = tile * 128 + (threadIdx.x & 127);
+    Sample s{make_float4(0.f, 0.f, 0.f, 0.f), 0.0f, pos < batch_size && batch_begin + pos < n};
+    if (s.valid) {
+        const int64_t i = permute(batch_begin + pos, n, pa, pc);
+        if (threadIdx.x < 128) s.f = F[i];
+        s.target = T[i];
+    }
+    return s;
+}
+
+template <bool ONCE>
+__device__ __forceinline__ void grad_tiles(unsigned char *sm, Walk &walk, const float *w, const float4 *__restrict__ F,
+                                           const float *__restrict__ T, int64_t n, int64_t batch_begin,
+                                           int64_t batch_size, uint64_t pa, uint64_t pc, Sample next, float *grad,
+                                           double *loss)
+{
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int half = warp >> 2, row = t & 127, c0 = 32 * half;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kSmBar);
     uint32_t *slot = reinterpret_cast<uint32_t *>(sm + kSmTmem);
     float *vb1 = reinterpret_cast<float *>(sm + kSmVec), *vb2 = vb1 + kH, *vw3 = vb2 + kH;
     float *ypart = reinterpret_cast<float *>(sm + kSmY);
-
-    if (warp == 0) tc::tmem_alloc(slot, kCols);
-    if (t == 0) tc::mbar_init(bar, 1);
+    const int64_t ntiles = (batch_size + 127) / 128;
+    if ((int64_t)blockIdx.x >= ntiles) return;   // uniform per block
     const float z8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (t < 128) store8(sm + kSmA, t, kH + 8, kColsA, z8);
     if (t < kH) {
@@ -184,30 +211,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     constexpr uint32_t id_grad = tc::idesc_bf16_f32(128, kColsA) | tc::kIdescAMajorM | tc::kIdescBMajorN;
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
     const float b3 = w[kOffB3], inv_b = 1.0f / (float)batch_size;
-    uint32_t tmem = 0, phase = 0;
-    bool good = true;
+    uint32_t tmem = 0;
     auto wait_mma = [&]() {
-        good = tc::mbar_wait_bounded(bar, phase & 1u, kWaitLimit) && good;
-        ++phase;
+        walk.good = tc::mbar_wait_bounded(bar, walk.phase & 1u, kWaitLimit) && walk.good;
+        ++walk.phase;
         tc::fence_after_sync();
     };
     float s_w3 = 0.0f, s_b2 = 0.0f, s_b1 = 0.0f, s_b3 = 0.0f;   // of column c0 + lane; s_b3 of this row
     double s_loss = 0.0;
-    const int64_t ntiles = (batch_size + 127) / 128;
     bool first = true;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t pos = tile * 128 + row;
-        const bool valid = pos < batch_size && batch_begin + pos < n;
-        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float target = 0.0f;
-        if (valid) {
-            const int64_t s = permute(batch_begin + pos, n, pa, pc);
-            if (half == 0) {
-                const float4 q = F[s];
-                f[0] = q.x; f[1] = q.y; f[2] = q.z; f[3] = q.w;
-            }
-            target = T[s];
-        }
+        const bool valid = next.valid;
+        const float f[8] = {next.f.x, next.f.y, next.f.z, next.f.w, 0.f, 0.f, 0.f, 0.f};
+        const float target = next.target;
+        if (tile + gridDim.x < ntiles) next = load_sample(F, T, n, batch_begin, batch_size, pa, pc, tile + gridDim.x);
         if (!first) wait_mma();   // the previous tile's gradient MMAs have read both tiles
         if (half == 0) store8(sm + kSmA, row, kH, kColsA, f);
         sync_for_mma();
@@ -332,9 +349,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         }
         first = false;
     }
-    if (!first) wait_mma();
+    wait_mma();
     const bool vec = (reinterpret_cast<uintptr_t>(grad) & 15u) == 0;
-    if (!first) {
+    {
         const int lrow = (warp & 3) * 32 + lane;      // gradient row of this thread
         if (lrow < kH) {
 #pragma unroll
@@ -385,28 +402,80 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         atomicAdd(&grad[kOffB3], v);
         atomicAdd(loss, l);
     }
-    if (!good && t == 0) {
-        tc::mbar_wait_bounded(bar, (phase - 1) & 1u, kWaitLimit);
-        atomicExch(err, 1);
-    }
-    __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(*slot, kCols);
+    __syncthreads();   // the sums above have been read: the next walk may write
 }
 
-// Adam (Kingma & Ba) on the FP32 master weights; clears the gradient.
-__global__ void k_mlp_adam(float *w, float *m, float *v, float *grad, int64_t step, float lr, float b1, float b2,
-                           float eps)
+// Tensor memory and mbarrier of a CTA, around its walks.
+__device__ __forceinline__ void walk_begin(unsigned char *sm)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= kNW) return;
-    const float g = grad[k];
-    grad[k] = 0.0f;
-    const float mk = b1 * m[k] + (1.0f - b1) * g;
-    const float vk = b2 * v[k] + (1.0f - b2) * g * g;
-    m[k] = mk;
-    v[k] = vk;
-    const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
-    w[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+    if (threadIdx.x < 32) tc::tmem_alloc(reinterpret_cast<uint32_t *>(sm + kSmTmem), kCols);
+    if (threadIdx.x == 0) tc::mbar_init(reinterpret_cast<uint64_t *>(sm + kSmBar), 1);
+    __syncthreads();
+}
+__device__ __forceinline__ void walk_end(unsigned char *sm, const Walk &walk, int *err)
+{
+    if (!walk.good && threadIdx.x == 0) {
+        // an MMA did not report completion: one more bounded wait before the memory is released
+        tc::mbar_wait_bounded(reinterpret_cast<uint64_t *>(sm + kSmBar), (walk.phase - 1) & 1u, kWaitLimit);
+        atomicExch(err, 1);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (threadIdx.x < 32) tc::tmem_dealloc(*reinterpret_cast<uint32_t *>(sm + kSmTmem), kCols);
+}
+
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+    k_mlp_grad(const float *__restrict__ w, const float4 *__restrict__ F, const float *__restrict__ T, int64_t n,
+               float *grad, double *loss, int *err)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    Walk walk;
+    walk_begin(sm);
+    grad_tiles<true>(sm, walk, w, F, T, n, 0, n, 1, 0, load_sample(F, T, n, 0, n, 1, 0, blockIdx.x), grad, loss);
+    walk_end(sm, walk, err);
+}
+
+// One epoch of training in one cooperative launch: per mini-batch the gradient, a barrier, Adam
+// (Kingma & Ba) on the FP32 master weights by all CTAs, which also clears the gradient, and a
+// barrier; the next batch's samples are loaded across the barriers.  As a gradient and an Adam launch a
+// batch, 4,096 samples took 21 us, 12 of them in the gradient; 17 us here.
+struct AdamArgs {
+    float lr, b1, b2, eps;
+};
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+    k_mlp_epoch(float *w, float *m, float *v, float *grad, const float4 *__restrict__ F, const float *__restrict__ T,
+                int64_t n, int64_t batch, uint64_t pa, uint64_t pc, int64_t step, AdamArgs h, double *acc,
+                float *history, GridBar *gbar, int *err)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    Walk walk;
+    uint32_t gen = *reinterpret_cast<volatile uint32_t *>(&gbar->gen);
+    walk_begin(sm);
+    Sample next = load_sample(F, T, n, 0, min(batch, n), pa, pc, blockIdx.x);
+    for (int64_t b0 = 0; b0 < n; b0 += batch) {
+        grad_tiles<false>(sm, walk, w, F, T, n, b0, min(batch, n - b0), pa, pc, next, grad, acc);
+        const int64_t b1 = b0 + batch;
+        if (b1 < n) next = load_sample(F, T, n, b1, min(batch, n - b1), pa, pc, blockIdx.x);
+        if (!grid_barrier(gbar, err, gen)) break;
+        ++step;
+        const float c1 = 1.0f - powf(h.b1, (float)step), c2 = 1.0f - powf(h.b2, (float)step);
+        for (int k = blockIdx.x * kThreads + threadIdx.x; k < kNW; k += gridDim.x * kThreads) {
+            const float g = __ldcg(grad + k);
+            grad[k] = 0.0f;
+            const float mk = h.b1 * m[k] + (1.0f - h.b1) * g;
+            const float vk = h.b2 * v[k] + (1.0f - h.b2) * g * g;
+            m[k] = mk;
+            v[k] = vk;
+            w[k] -= h.lr * (mk / c1) / (sqrtf(vk / c2) + h.eps);
+        }
+        if (b1 >= n && blockIdx.x == 0 && threadIdx.x == 0) {   // the epoch's mean loss
+            if (history) *history = (float)(__ldcg(acc) / (double)n);
+            *acc = 0.0;
+        }
+        if (!grid_barrier(gbar, err, gen)) break;
+    }
+    walk_end(sm, walk, err);
 }
 
 // Mean and standard deviation of the raw features and labels (FP64 sums).
@@ -421,11 +490,20 @@ __global__ void k_mlp_moments(const float4 *__restrict__ F, const float *__restr
             s[5 + a] += x[a] * x[a];
         }
     }
+    // one atomic a block and sum (one a warp, 24,000 on ten words, took 32 us)
+    __shared__ double sh[8][10];
+#pragma unroll
     for (int a = 0; a < 10; ++a) {
         double r = s[a];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&acc[a], r);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][a] = r;
+    }
+    __syncthreads();
+    if (threadIdx.x < 10) {
+        double r = 0.0;
+        for (int k = 0; k < 8; ++k) r += sh[k][threadIdx.x];
+        atomicAdd(&acc[threadIdx.x], r);
     }
 }
 
@@ -458,12 +536,6 @@ __global__ void k_mlp_standardise(const float4 *__restrict__ F, const float *__r
     }
 }
 
-__global__ void k_epoch_loss(double *acc, float *out, int64_t n)
-{
-    *out = (float)(*acc / (double)n);
-    *acc = 0.0;
-}
-
 uint64_t mix64(uint64_t x)
 {
     x += 0x9E3779B97F4A7C15ull;
@@ -483,9 +555,9 @@ uint64_t gcd64(uint64_t a, uint64_t b)
 
 cudaError_t set_attr()
 {
-    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_mlp_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    return cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
 // CTAs of the gradient kernel over a batch: one per tile, at most two per SM.
@@ -513,8 +585,8 @@ extern "C" sph_status sph_mlp_grad(const float *params, const float *features, c
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaMemsetAsync(grad, 0, sizeof(float) * kNW, s) != cudaSuccess) return SPH_ECUDA;
     if (cudaMemsetAsync(loss, 0, sizeof(double), s) != cudaSuccess) return SPH_ECUDA;
-    k_mlp_grad<true><<<grad_grid(n), kThreads, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features), labels, n, 0, n,
-                                                     1, 0, grad, loss, reinterpret_cast<int *>(error));
+    k_mlp_grad<<<grad_grid(n), kThreads, kSmem, s>>>(params, reinterpret_cast<const float4 *>(features), labels, n, grad,
+                                                     loss, reinterpret_cast<int *>(error));
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
 }
 
@@ -538,17 +610,18 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
     };
     if (cudaMallocAsync(&Fs, sizeof(float4) * n, s) != cudaSuccess || cudaMallocAsync(&Ts, sizeof(float) * n, s) != cudaSuccess ||
         cudaMallocAsync(&grad, sizeof(float) * kNW, s) != cudaSuccess ||
-        cudaMallocAsync(&acc, sizeof(double) * 12, s) != cudaSuccess) {
+        cudaMallocAsync(&acc, sizeof(double) * 13, s) != cudaSuccess) {
         cleanup();
         return SPH_ENOMEM;
     }
-    bool ok = cudaMemsetAsync(acc, 0, sizeof(double) * 12, s) == cudaSuccess &&
+    bool ok = cudaMemsetAsync(acc, 0, sizeof(double) * 13, s) == cudaSuccess &&
               cudaMemsetAsync(grad, 0, sizeof(float) * kNW, s) == cudaSuccess;
     const float4 *F = reinterpret_cast<const float4 *>(features);
     k_mlp_moments<<<304, 256, 0, s>>>(F, labels, n, acc);
     k_mlp_standardise<<<304, 256, 0, s>>>(F, labels, n, acc, params, Fs, Ts);
-    cudaMemsetAsync(acc, 0, sizeof(double) * 12, s);
+    cudaMemsetAsync(acc, 0, sizeof(double) * 13, s);
     float *m = adam_state, *v = adam_state + kNW;
+    GridBar *gbar = reinterpret_cast<GridBar *>(acc + 12);
     int64_t step = 0;
     const int64_t B = batch;
     for (int32_t e = 0; e < epochs && ok; ++e) {
@@ -556,16 +629,18 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
         uint64_t a = mix64(seed * 0x100000001B3ull + (uint64_t)e) % (uint64_t)(n - 1) + 1;
         while (gcd64(a, (uint64_t)n) != 1) a = a % (uint64_t)(n - 1) + 1;
         const uint64_t c = mix64(seed ^ (0xA5A5A5A5ull + (uint64_t)e)) % (uint64_t)n;
-        for (int64_t b0 = 0; b0 < n; b0 += B) {
-            const int64_t bs = std::min<int64_t>(B, n - b0);
-            k_mlp_grad<false><<<grad_grid(bs), kThreads, kSmem, s>>>(params, Fs, Ts, n, b0, bs, a, c, grad, acc,
-                                                              reinterpret_cast<int *>(error));
-            ++step;
-            k_mlp_adam<<<(kNW + 255) / 256, 256, 0, s>>>(params, m, v, grad, step, lr, 0.9f, 0.999f, 1e-8f);
-        }
-        if (loss_history) k_epoch_loss<<<1, 1, 0, s>>>(acc, loss_history + e, n);
-        ok = cudaGetLastError() == cudaSuccess;
+        float *hist = loss_history ? loss_history + e : nullptr;
+        int *err = reinterpret_cast<int *>(error);
+        AdamArgs h{lr, 0.9f, 0.999f, 1e-8f};
+        const float4 *Fe = Fs;
+        const float *Te = Ts;
+        void *args[] = {&params, &m, &v, &grad, &Fe, &Te, (void *)&n, (void *)&B, (void *)&a, (void *)&c, &step, &h, &acc,
+                        &hist, &gbar, &err};
+        ok = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_mlp_epoch), dim3(grad_grid(std::min(B, n))),
+                                         dim3(kThreads), args, kSmem, s) == cudaSuccess;
+        step += (n + B - 1) / B;
     }
+    ok = ok && cudaGetLastError() == cudaSuccess;
     cleanup();
     return ok && cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
 }

@@ -62,3 +62,26 @@ def test_forward_non_finite_rows(n):
     keep[bad] = False
     assert bool(torch.isnan(y[1][~keep]).all())
     assert torch.equal(y[0][keep], y[1][keep])
+
+
+@pytest.mark.parametrize("n,batch", [(2, 1), (129, 128), (300, 127), (1000, 5000), (20_003, 4096), (128 * 310 + 1, 128 * 305)])
+def test_epochs_cover_every_sample_once(n, batch):
+    """With a vanishing learning rate every epoch's mean loss is that of the initial network
+    over all (standardised) samples, whatever the batches."""
+    import torch
+    rng = np.random.default_rng(n)
+    p = np.zeros(sph.MLP_PARAMS, np.float32)
+    p[:sph.MLP_WEIGHTS] = rng.normal(scale=0.3, size=sph.MLP_WEIGHTS)
+    f = (rng.normal(size=(n, 4)) * [1.0, 3.0, 0.5, 2.0] + 1.0).astype(np.float32)
+    t = (rng.normal(size=n) * 2.0 + 5.0).astype(np.float32)
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    dp, adam = dev(p), torch.zeros(2 * sph.MLP_WEIGHTS, device="cuda")
+    hist, err = torch.zeros(3, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert sph.sph_mlp_train(dev(f), dev(t), n, dp, adam, 3, batch, 1e-20, 5, hist, err) == sph.SPH_OK
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    std = lambda a: (a - a.mean(0)) / a.std(0)  # noqa: E731
+    ref, _ = oracle.mlp_loss_grad(p.astype(np.float64), std(f.astype(np.float64)), std(t.astype(np.float64)))
+    # BF16 operands: 2e-2, as for the gradient's loss
+    np.testing.assert_allclose(hist.cpu().numpy(), ref, rtol=2e-2)
+    np.testing.assert_array_equal(dp.cpu().numpy()[:sph.MLP_WEIGHTS], p[:sph.MLP_WEIGHTS])
