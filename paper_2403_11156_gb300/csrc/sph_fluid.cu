@@ -65,18 +65,18 @@ __device__ __forceinline__ int warp_max(int v)
 // a scene reduces the same way alone and in any batch.
 __device__ __forceinline__ int32_t fold_size(int32_t count) { return max(8, (count + 255) / 256); }
 
-// Fixed-order block sum of one double per thread (deterministic).
+// Fixed-order block sum of one double per thread (deterministic; valid in thread 0; sh holds
+// one double a thread).  FP64 additions are a few per cycle and SM on this GPU: through shared
+// memory one warp does all 8 x 32 of them, where butterflies in every warp did 20 x 32.
 __device__ double block_sum(double v, double *sh)
 {
-    v = warp_sum(v);
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     __syncthreads();
-    if (lane == 0) sh[w] = v;
+    sh[threadIdx.x] = v;
     __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int k = 0; k < kBlock / 32; ++k) t += sh[k];
-    return t;  // valid in thread 0
+    if (threadIdx.x >= 32) return 0.0;
+    static_assert(kBlock == 128, "four values a lane");
+    const double t = (sh[threadIdx.x] + sh[threadIdx.x + 32]) + (sh[threadIdx.x + 64] + sh[threadIdx.x + 96]);
+    return warp_sum(t);
 }
 
 // ------------------------------------------------------------------------------------
@@ -644,7 +644,7 @@ __device__ __forceinline__ void pass_a(const Ptrs &P, int32_t block, double *sh)
 template <int S, int B, int T>
 __global__ void __launch_bounds__(kBlock) k_pass_a(Ptrs P)
 {
-    __shared__ double sh[kBlock / 32];
+    __shared__ double sh[kBlock];
     kernel_enter(P.ctl, (KID_PASS_A0 + S));
     pass_a<S, B, T, true>(P, (int32_t)blockIdx.x, sh);
 }
@@ -794,7 +794,7 @@ constexpr int kSolveBlocksPerSm = 8;
 template <int S, int T>
 __global__ void __launch_bounds__(kBlock, kSolveBlocksPerSm) k_solve(const __grid_constant__ Ptrs P)
 {
-    __shared__ double sh[kBlock / 32];
+    __shared__ double sh[kBlock];
     __shared__ int s_any;
     kernel_enter(P.ctl, KID_SOLVE0 + S);
     uint32_t phase = *reinterpret_cast<volatile uint32_t *>(&P.ctl->bar.gen);

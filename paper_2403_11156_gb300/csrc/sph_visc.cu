@@ -131,14 +131,19 @@ __device__ __forceinline__ bool cg_active(const SceneDev &sc, const SceneState &
     return sc.visc_mode == 3 && st.cg_active != 0;
 }
 
-// Per-block partial sums of two doubles, written for a later one-block reduction.
-__device__ __forceinline__ void block_partials2(const Ptrs &P, double a, double b, double *sh)
+// The block's sum of one double per thread, written for a later one-block reduction (sh: one
+// double a thread).  FP64 additions are a few per cycle and SM on this GPU, so one warp does
+// the sum through shared memory: 8 x 32 of them, where butterflies in every warp, over a second
+// unused sum too, did 40 x 32.
+__device__ __forceinline__ void block_partial(const Ptrs &P, double a, double *sh)
 {
-    block_sum2(a, b, sh);
-    if (threadIdx.x == 0) {
-        P.cg_dots[2 * blockIdx.x] = a;
-        P.cg_dots[2 * blockIdx.x + 1] = b;
-    }
+    static_assert(kBlock == 128, "four values a lane");
+    __syncthreads();
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    a = warp_sum((sh[threadIdx.x] + sh[threadIdx.x + 32]) + (sh[threadIdx.x + 64] + sh[threadIdx.x + 96]));
+    if (threadIdx.x == 0) P.cg_dots[blockIdx.x] = a;
 }
 
 constexpr int kReduceThreads = 1024;
@@ -147,35 +152,29 @@ constexpr int kReduceThreads = 1024;
 // of the preceding launch over the scene's sweep blocks (SWEEP) or fluid blocks, in a fixed
 // order that depends only on the scene (thread t takes partials t, t + 1024, ..., then a
 // fixed tree), so a scene reduces the same way alone and in any batch; the scenes go in
-// turn.  done(scene, a, b) runs in one thread per scene.
+// turn.  done(scene, a) runs in one thread per scene.  sh: one double a thread.
 template <bool SWEEP, typename F>
 __device__ void reduce_scenes(const Ptrs &P, double *sh, F &&done)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double2 *d = reinterpret_cast<const double2 *>(P.cg_dots);
+    const int t = threadIdx.x;
     for (int q = 0; q < P.nscenes; ++q) {
         const SceneDev &qd = P.scenes[q];
         if (!cg_active(qd, P.st[q])) continue;   // uniform: nothing wrote the state yet
-        const int32_t first = SWEEP ? qd.tblk_first : qd.fblk_first;
+        const double *d = P.cg_dots + (SWEEP ? qd.tblk_first : qd.fblk_first);
         const int32_t count = SWEEP ? qd.tblk_count : qd.fblk_count;
-        double a = 0.0, b = 0.0;
-        for (int k = threadIdx.x; k < count; k += kReduceThreads) {
-            const double2 v = __ldcg(d + first + k);
-            a += v.x;
-            b += v.y;
-        }
-        a = warp_sum(a);
-        b = warp_sum(b);
-        if (lane == 0) {
-            sh[2 * warp] = a;
-            sh[2 * warp + 1] = b;
+        double a = 0.0;
+        for (int k = t; k < count; k += kReduceThreads) a += __ldcg(d + k);
+        sh[t] = a;
+        __syncthreads();
+        if (t < 128) {
+#pragma unroll
+            for (int o = 1; o < kReduceThreads / 128; ++o) a += sh[t + 128 * o];
+            sh[t] = a;
         }
         __syncthreads();
-        if (warp == 0) {
-            double u = sh[2 * lane], w = sh[2 * lane + 1];
-            u = warp_sum(u);
-            w = warp_sum(w);
-            if (lane == 0) done(q, u, w);
+        if (t < 32) {
+            a = warp_sum((sh[t] + sh[t + 32]) + (sh[t + 64] + sh[t + 96]));
+            if (t == 0) done(q, a);
         }
         __syncthreads();
     }
@@ -218,13 +217,13 @@ __global__ void __launch_bounds__(kBlock) k_cg_init(Ptrs P)
 template <int T>
 __global__ void __launch_bounds__(kBlock) k_cg_ap(Ptrs P)
 {
-    __shared__ double sh[2 * kBlock / 32];
+    __shared__ double sh[kBlock];
     kernel_enter(P.ctl, KID_CG_AP);
     const Lane<T> c = lane_ctx<T>(P);
     const SceneDev &sc = *c.sc;
     SceneState &st = *c.st;
     if (!cg_active(sc, st)) return;  // uniform per block
-    double pap = 0.0, unused = 0.0;
+    double pap = 0.0;
     const int64_t i = c.i;
     const float4 pi = c.valid ? P.pos_s[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 p = c.valid ? P.cg_p[i] : make_float4(0.f, 0.f, 0.f, 1.f);
@@ -233,15 +232,15 @@ __global__ void __launch_bounds__(kBlock) k_cg_ap(Ptrs P)
         P.cg_ap[i] = make_float4(ap.x, ap.y, ap.z, 0.0f);
         pap = (double)p.x * ap.x + (double)p.y * ap.y + (double)p.z * ap.z;
     }
-    block_partials2(P, pap, unused, sh);
+    block_partial(P, pap, sh);
 }
 
 // alpha = |r|^2 / p.Ap per scene (one block).
 __global__ void __launch_bounds__(kReduceThreads) k_cg_alpha(Ptrs P)
 {
-    __shared__ double sh[2 * kReduceThreads / 32];
+    __shared__ double sh[kReduceThreads];
     kernel_enter(P.ctl, KID_CG_ALPHA);
-    reduce_scenes<true>(P, sh, [&](int q, double pap, double) {
+    reduce_scenes<true>(P, sh, [&](int q, double pap) {
         SceneState &qs = P.st[q];
         qs.cg_alpha = pap > 0.0 ? qs.cg_rr / pap : 0.0;
     });
@@ -250,13 +249,13 @@ __global__ void __launch_bounds__(kReduceThreads) k_cg_alpha(Ptrs P)
 // x += alpha p, r -= alpha Ap and the block partials of |r_new|^2.
 __global__ void __launch_bounds__(kBlock) k_cg_xr(Ptrs P)
 {
-    __shared__ double sh[2 * kBlock / 32];
+    __shared__ double sh[kBlock];
     kernel_enter(P.ctl, KID_CG_XR);
     Ctx c = ctx(P);
     const SceneDev &sc = *c.sc;
     SceneState &st = *c.st;
     if (!cg_active(sc, st)) return;
-    double rr = 0.0, unused = 0.0;
+    double rr = 0.0;
     if (c.valid) {
         const int64_t i = c.i;
         const float a = (float)st.cg_alpha;
@@ -270,7 +269,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_xr(Ptrs P)
         P.cg_r[i] = r;
         rr = (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
     }
-    block_partials2(P, rr, unused, sh);
+    block_partial(P, rr, sh);
 }
 
 // beta = |r_new|^2 / |r|^2 per scene, the iteration count and the residual; a scene stops
@@ -279,12 +278,12 @@ __global__ void __launch_bounds__(kBlock) k_cg_xr(Ptrs P)
 __global__ void __launch_bounds__(kReduceThreads) k_cg_beta(Ptrs P, cudaGraphConditionalHandle handle,
                                                            int use_handle)
 {
-    __shared__ double sh[2 * kReduceThreads / 32];
+    __shared__ double sh[kReduceThreads];
     __shared__ int s_any;
     kernel_enter(P.ctl, KID_CG_BETA);
     if (threadIdx.x == 0) s_any = 0;
     __syncthreads();
-    reduce_scenes<false>(P, sh, [&](int q, double rr, double) {
+    reduce_scenes<false>(P, sh, [&](int q, double rr) {
         const SceneDev &qd = P.scenes[q];
         SceneState &qs = P.st[q];
         qs.cg_beta = qs.cg_rr > 0.0 ? rr / qs.cg_rr : 0.0;
