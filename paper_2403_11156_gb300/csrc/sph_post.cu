@@ -12,8 +12,7 @@
 //    iso-level are cut off by one triangle (one or three corners above) or two (two
 //    above), vertices interpolated linearly along the cut edges from the corner above to
 //    the corner below (the same arithmetic in every cube sharing an edge), each triangle oriented
-//    so its normal points from the corners above to those below.  One kernel counts a tile
-//    of cubes, finds its place in cube order by decoupled look-back and writes its triangles.
+//    so its normal points from the corners above to those below, in cube order.
 //  * height map: per particle, the pixels of its disk receive z + sqrt(R^2 - d^2) through
 //    an atomic maximum on an order-preserving integer image of the float.
 #include "sph.h"
@@ -363,15 +362,13 @@ __device__ __forceinline__ void emit_tet(const Cube &c, uint32_t above, int t, f
     }
 }
 
-// The whole surface in one pass over the field: a block takes the next tile of consecutive
-// cubes, counts each cube's triangles from its corner bits, adds the counts of all earlier
-// tiles by decoupled look-back (a warp looks at 32 tiles at a time), and its threads then
-// write the tile's crossed tetrahedra, one each, from a shared list.  16M cubes of the 1.2M
-// scene: 640 us before, in three kernels (a 64 MB count array written, scanned and read, the field
-// read twice, and a crossed cube's thread writing all its triangles alone).
+// The surface in three launches: a block counts the triangles of a tile of consecutive cubes from
+// their corner bits; one block makes the tiles' places out of the counts; the blocks of crossed
+// tiles place their cubes and write the crossed tetrahedra, one a thread, from a shared list.
+// 16M cubes of the 1.2M scene: about 250 us; 640 us with a count a cube in memory (64 MB written,
+// scanned and read) and a crossed cube's thread writing all its triangles alone; 276 us as one
+// launch with look-back between the tiles, which it spent waiting.
 constexpr int kMeshThreads = 256, kMeshItems = 8, kMeshTile = kMeshThreads * kMeshItems;
-constexpr uint32_t kMeshSpin = 1u << 22;
-constexpr uint64_t kMeshAgg = 1ull << 62, kMeshIncl = 2ull << 62;   // a tile's own / inclusive count
 // Division of n < 2^31 by d >= 1: n m >> (31 + l), l = ceil(log2 d), m = ceil(2^(31+l) / d).
 struct Divisor {
     uint32_t d, l;
@@ -383,53 +380,108 @@ struct Divisor {
     }
     __device__ __forceinline__ uint32_t quotient(uint32_t n) const { return (uint32_t)(((uint64_t)n * (uint32_t)m) >> (31 + l)); }
 };
-struct MeshCtl {
-    uint32_t total;    // triangles
-    int32_t error;     // a look-back wait gave up
-    int32_t ticket;    // next tile
-    int32_t pad;
+
+struct MeshGrid {
+    const float *f;
+    int32_t nx, ny;
+    Divisor by_x, by_y;   // cubes along x, along y
+    uint32_t cubes;       // fewer than 2^31
+    float iso;
 };
 
-__global__ void __launch_bounds__(kMeshThreads)
-    k_mt_mesh(const float *__restrict__ f, int32_t nx, int32_t ny, int32_t nz, float ox, float oy, float oz, float sp,
-              float iso, Divisor by_x, Divisor by_y, uint32_t cubes, MeshCtl *ctl, uint64_t *status, float *tris, int64_t cap)
+// Triangles by corner bits, for the block.
+__device__ __forceinline__ void mesh_counts(uint8_t *s_count)
 {
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) n += tet_count((uint32_t)threadIdx.x, q);
+    s_count[threadIdx.x] = (uint8_t)n;
+    __syncthreads();
+}
+
+// Corner bits of this thread's cubes of a tile: base + t, base + t + 256, ...: a warp reads 33
+// consecutive values of each of four rows.
+__device__ __forceinline__ void mesh_corners(const MeshGrid &g, uint32_t tile, uint32_t (&above)[kMeshItems])
+{
+    const int64_t dz = (int64_t)g.nx * g.ny;
+#pragma unroll
+    for (int q = 0; q < kMeshItems; ++q) {
+        const uint32_t cube = tile * kMeshTile + (uint32_t)(q * kMeshThreads) + threadIdx.x;
+        above[q] = 0u;
+        if (cube < g.cubes) {
+            const uint32_t row = g.by_x.quotient(cube), i = cube - row * g.by_x.d, k = g.by_y.quotient(row), j = row - k * g.by_y.d;
+            const float *p = g.f + (int64_t)i + (int64_t)g.nx * (j + (int64_t)g.ny * k);
+            const float iso = g.iso;
+            above[q] = (p[0] > iso ? 1u : 0u) | (p[1] > iso ? 2u : 0u) | (p[g.nx] > iso ? 4u : 0u) |
+                       (p[g.nx + 1] > iso ? 8u : 0u) | (p[dz] > iso ? 16u : 0u) | (p[dz + 1] > iso ? 32u : 0u) |
+                       (p[dz + g.nx] > iso ? 64u : 0u) | (p[dz + g.nx + 1] > iso ? 128u : 0u);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kMeshThreads) k_mt_count(MeshGrid g, uint32_t *tile_count)
+{
+    __shared__ uint8_t s_count[256];
+    __shared__ uint32_t s_warp[kMeshThreads / 32];
+    mesh_counts(s_count);
+    uint32_t above[kMeshItems], n = 0u;
+    mesh_corners(g, blockIdx.x, above);
+#pragma unroll
+    for (int q = 0; q < kMeshItems; ++q) n += s_count[above[q]];
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = n;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kMeshThreads / 32; ++w) n += s_warp[w];
+        tile_count[blockIdx.x] = n;
+    }
+}
+
+// Exclusive sums of the tiles' counts in place, the total behind them (one block).
+__global__ void __launch_bounds__(1024) k_mt_places(uint32_t *tile_count, int32_t ntiles)
+{
+    __shared__ uint32_t s_warp[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t run = 0u;
+    for (int32_t k0 = 0; k0 < ntiles; k0 += 1024) {
+        const int32_t k = k0 + (int32_t)threadIdx.x;
+        const uint32_t v = k < ntiles ? tile_count[k] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        const uint32_t w = s_warp[lane];
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+        if (k < ntiles) tile_count[k] = run + before + x - v;
+        run += __reduce_add_sync(0xffffffffu, w);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) tile_count[ntiles] = run;
+}
+
+__global__ void __launch_bounds__(kMeshThreads)
+    k_mt_emit(MeshGrid g, float ox, float oy, float oz, float sp, const uint32_t *__restrict__ place, float *tris, int64_t cap)
+{
+    const uint32_t tile = blockIdx.x;
+    const int64_t first = (int64_t)place[tile];
+    if ((int64_t)place[tile + 1] == first || first >= cap) return;
     constexpr int kWarps = kMeshThreads / 32;
     static_assert(kMeshItems * kWarps == 64, "one warp scans the sums of all items, two a lane");
     __shared__ uint8_t s_count[256];                 // triangles by corner bits
     __shared__ uint32_t s_list[kMeshTile];           // crossed cubes: index in the tile, corner bits
     __shared__ uint16_t s_first[kMeshTile];          // their first triangle in the tile (at most 24,576)
     __shared__ uint32_t s_sum[kMeshItems * kWarps];  // per item and warp, then their exclusive sums
-    __shared__ uint32_t s_all, s_prefix;
-    __shared__ int32_t s_tile;
+    __shared__ uint32_t s_crossed;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (t == 0) s_tile = atomicAdd(&ctl->ticket, 1);
-    {
-        int n = 0;
-        for (int q = 0; q < 6; ++q) n += tet_count((uint32_t)t, q);
-        s_count[t] = (uint8_t)n;
-    }
-    __syncthreads();
-    const int32_t tile = s_tile;
-    // fewer than 2^31 cubes: 32-bit indices, divided by multiplication
-    const uint32_t base = (uint32_t)tile * kMeshTile;
-    // cubes base + t, base + t + 256, ...: a warp reads 33 consecutive values of each of four
-    // rows.  Per item, places in cube order from sums over the warp of the triangles (low 16
-    // bits) and the crossed cubes (high 16 bits).
+    mesh_counts(s_count);
+    // per item, places in cube order from sums over the warp of the triangles (low 16 bits)
+    // and the crossed cubes (high 16 bits)
     uint32_t above[kMeshItems], sum[kMeshItems];
-#pragma unroll
-    for (int q = 0; q < kMeshItems; ++q) {
-        const uint32_t cube = base + (uint32_t)(q * kMeshThreads + t);
-        above[q] = 0u;
-        if (cube < cubes) {
-            const uint32_t row = by_x.quotient(cube), i = cube - row * by_x.d, k = by_y.quotient(row), j = row - k * by_y.d;
-            const float *p = f + (int64_t)i + (int64_t)nx * (j + (int64_t)ny * k);
-            const int64_t dz = (int64_t)nx * ny;
-            above[q] = (p[0] > iso ? 1u : 0u) | (p[1] > iso ? 2u : 0u) | (p[nx] > iso ? 4u : 0u) | (p[nx + 1] > iso ? 8u : 0u) |
-                       (p[dz] > iso ? 16u : 0u) | (p[dz + 1] > iso ? 32u : 0u) | (p[dz + nx] > iso ? 64u : 0u) |
-                       (p[dz + nx + 1] > iso ? 128u : 0u);
-        }
-    }
+    mesh_corners(g, tile, above);
 #pragma unroll
     for (int q = 0; q < kMeshItems; ++q) {
         const uint32_t n = s_count[above[q]], v = n | (n ? 0x10000u : 0u);
@@ -453,57 +505,20 @@ __global__ void __launch_bounds__(kMeshThreads)
             const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) s_all = x;
+        if (lane == 31) s_crossed = x >> 16;
         s_sum[2 * lane] = x - a - b;
         s_sum[2 * lane + 1] = x - b;
     }
     __syncthreads();
-    const uint32_t mine = s_all & 0xffffu, crossed = s_all >> 16;
-    if (crossed != 0u) {
+    const uint32_t crossed = s_crossed;
 #pragma unroll
-        for (int q = 0; q < kMeshItems; ++q) {
-            if (s_count[above[q]] == 0u) continue;
-            const uint32_t at = s_sum[q * kWarps + warp] + sum[q];
-            s_list[at >> 16] = (uint32_t)(q * kMeshThreads + t) | (above[q] << 16);
-            s_first[at >> 16] = (uint16_t)(at & 0xffffu);
-        }
-    }
-    if (warp == 0) {
-        uint32_t prefix = 0u;
-        volatile uint64_t *st = status;
-        if (lane == 0) atomicExch((unsigned long long *)&status[tile], (tile == 0 ? kMeshIncl : kMeshAgg) | mine);
-        for (int32_t last = tile - 1; last >= 0;) {
-            // lane l looks at tile last - l; the nearest inclusive count ends the walk
-            const int32_t at = last - lane;
-            uint64_t w = kMeshIncl;                   // before the first tile: nothing
-            if (at >= 0) {
-                uint32_t spins = 0;
-                while (((w = st[at]) >> 62) == 0ull) {
-                    if (++spins > kMeshSpin) {
-                        atomicExch(&ctl->error, 1);
-                        w = kMeshIncl;
-                        break;
-                    }
-                    __nanosleep(32);
-                }
-            }
-            const unsigned incl = __ballot_sync(0xffffffffu, (w >> 63) != 0ull);
-            const int stop = incl ? __ffs(incl) - 1 : 31;
-            uint32_t c = lane <= stop ? (uint32_t)w : 0u;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            prefix += c;
-            if (incl) break;
-            last -= 32;
-        }
-        if (lane == 0) {
-            if (tile > 0) atomicExch((unsigned long long *)&status[tile], kMeshIncl | (uint64_t)(prefix + mine));
-            s_prefix = prefix;
-            if ((uint64_t)base + kMeshTile >= cubes) ctl->total = prefix + mine;
-        }
+    for (int q = 0; q < kMeshItems; ++q) {
+        if (s_count[above[q]] == 0u) continue;
+        const uint32_t at = s_sum[q * kWarps + warp] + sum[q];
+        s_list[at >> 16] = (uint32_t)(q * kMeshThreads + t) | (above[q] << 16);
+        s_first[at >> 16] = (uint16_t)(at & 0xffffu);
     }
     __syncthreads();
-    const int64_t first = (int64_t)s_prefix;
     for (uint32_t u = (uint32_t)t; u < crossed * 6u; u += kMeshThreads) {
         const uint32_t c = u / 6u;
         const int tet = (int)(u - 6u * c);
@@ -512,9 +527,9 @@ __global__ void __launch_bounds__(kMeshThreads)
         int64_t o = first + s_first[c];
         for (int q = 0; q < tet; ++q) o += tet_count(a, q);
         if (o >= cap) continue;
-        const uint32_t cube = base + (e & 0xffffu), row = by_x.quotient(cube), k = by_y.quotient(row);
-        const Cube cb{f, nx, ny, (int32_t)(cube - row * by_x.d), (int32_t)(row - k * by_y.d), (int32_t)k, ox, oy, oz, sp};
-        emit_tet(cb, a, tet, iso, o, tris, cap);
+        const uint32_t cube = tile * kMeshTile + (e & 0xffffu), row = g.by_x.quotient(cube), k = g.by_y.quotient(row);
+        const Cube cb{g.f, g.nx, g.ny, (int32_t)(cube - row * g.by_x.d), (int32_t)(row - k * g.by_y.d), (int32_t)k, ox, oy, oz, sp};
+        emit_tet(cb, a, tet, g.iso, o, tris, cap);
     }
 }
 
@@ -635,26 +650,20 @@ extern "C" sph_status sph_surface_mesh(const float *field, const int32_t dims[3]
     if ((int64_t)dims[0] * dims[1] * dims[2] > ((int64_t)1 << 31)) return SPH_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t ntiles = (cubes + kMeshTile - 1) / kMeshTile;
-    // result and ticket first, then a look-back word a tile
-    MeshCtl *ctl = nullptr;
-    const size_t bytes = sizeof(MeshCtl) + sizeof(uint64_t) * (size_t)ntiles;
-    cudaError_t e = cudaMallocAsync((void **)&ctl, bytes, s);
-    MeshCtl r{};
+    uint32_t *place = nullptr, total = 0;
+    cudaError_t e = cudaMallocAsync((void **)&place, sizeof(uint32_t) * (size_t)(ntiles + 1), s);
     if (e == cudaSuccess) {
-        e = cudaMemsetAsync(ctl, 0, bytes, s);
-        if (e == cudaSuccess) {
-            k_mt_mesh<<<(unsigned)ntiles, kMeshThreads, 0, s>>>(field, dims[0], dims[1], dims[2], origin[0], origin[1],
-                                                               origin[2], spacing, iso, Divisor((uint32_t)dims[0] - 1u),
-                                                               Divisor((uint32_t)dims[1] - 1u), (uint32_t)cubes, ctl,
-                                                               reinterpret_cast<uint64_t *>(ctl + 1), tris, cap);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&r, ctl, sizeof r, cudaMemcpyDeviceToHost, s);
-        cudaFreeAsync(ctl, s);
+        const MeshGrid g{field, dims[0], dims[1], Divisor((uint32_t)dims[0] - 1u), Divisor((uint32_t)dims[1] - 1u),
+                         (uint32_t)cubes, iso};
+        k_mt_count<<<(unsigned)ntiles, kMeshThreads, 0, s>>>(g, place);
+        k_mt_places<<<1, 1024, 0, s>>>(place, (int32_t)ntiles);
+        if (cap > 0) k_mt_emit<<<(unsigned)ntiles, kMeshThreads, 0, s>>>(g, origin[0], origin[1], origin[2], spacing, place, tris, cap);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&total, place + ntiles, sizeof total, cudaMemcpyDeviceToHost, s);
+        cudaFreeAsync(place, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return SPH_ECUDA;
-    if (r.error) return SPH_ETIMEOUT;
-    *n_tris = (int64_t)r.total;
-    return (int64_t)r.total > cap ? SPH_EOVERFLOW : SPH_OK;
+    *n_tris = (int64_t)total;
+    return (int64_t)total > cap ? SPH_EOVERFLOW : SPH_OK;
 }
