@@ -229,6 +229,7 @@ __device__ __forceinline__ void grad_tiles(unsigned char *sm, Walk &walk, const 
         if (half == 0) store8(sm + kSmA, row, kH, kColsA, f);
         sync_for_mma();
         tmem = *slot;
+        float g1[ONCE ? 1 : 32];   // gelu'(z1), kept to the backward pass (ONCE: taken again there)
         // layer 1: z1 -> columns [0, 64)
         if (t == 0) {
             tc::mma_bf16(tmem, tc::smem_desc(sb + kSmA + (kH / 8) * 128, 128, kColsA * 16),
@@ -247,8 +248,10 @@ __device__ __forceinline__ void grad_tiles(unsigned char *sm, Walk &walk, const 
                 if (ONCE) {
                     gelu::upk(gelu::gelu_pair(h0, h1), v[k], v[k + 1]);
                 } else {
-                    v[k] = h0 * (1.0f + erff(2.0f * h0 * 0.70710678118654752f));
-                    v[k + 1] = h1 * (1.0f + erff(2.0f * h1 * 0.70710678118654752f));
+                    gelu::f2 a, d;
+                    gelu_grad_erff(h0, h1, a, d);
+                    gelu::upk(a, v[k], v[k + 1]);
+                    gelu::upk(d, g1[c * 16 + k], g1[c * 16 + k + 1]);
                 }
             }
             store8(sm + kSmA, row, c0 + c * 16, kColsA, v);
@@ -325,15 +328,18 @@ __device__ __forceinline__ void grad_tiles(unsigned char *sm, Walk &walk, const 
         for (int c = 0; c < 2; ++c) {
             float g[16], z[16];
             tc::tmem_ld16(tmem + lanes + kColZ2 + c0 + c * 16, g);
-            tc::tmem_ld16(tmem + lanes + c0 + c * 16, z);
+            if (ONCE) tc::tmem_ld16(tmem + lanes + c0 + c * 16, z);
 #pragma unroll
             for (int k = 0; k < 16; k += 2) {
                 const int o = c0 + c * 16 + k, q = c * 16 + k;
-                gelu::f2 a, d;
-                const float h0 = fmaf(0.5f, z[k], vb1[o]), h1 = fmaf(0.5f, z[k + 1], vb1[o + 1]);
-                if (ONCE) gelu::gelu_grad_pair(h0, h1, a, d);
-                else gelu_grad_erff(h0, h1, a, d);
-                gelu::upk(gelu::mul2(d, gelu::pk(g[k], g[k + 1])), d1[q], d1[q + 1]);
+                if constexpr (ONCE) {
+                    gelu::f2 a, d;
+                    gelu::gelu_grad_pair(fmaf(0.5f, z[k], vb1[o]), fmaf(0.5f, z[k + 1], vb1[o + 1]), a, d);
+                    gelu::upk(gelu::mul2(d, gelu::pk(g[k], g[k + 1])), d1[q], d1[q + 1]);
+                } else {
+                    d1[q] = g[k] * g1[q];
+                    d1[q + 1] = g[k + 1] * g1[q + 1];
+                }
             }
         }
 #pragma unroll
@@ -439,11 +445,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 // One epoch of training in one cooperative launch: per mini-batch the gradient, a barrier, Adam
 // (Kingma & Ba) on the FP32 master weights by all CTAs, which also clears the gradient, and a
 // barrier; the next batch's samples are loaded across the barriers.  As a gradient and an Adam launch a
-// batch, 4,096 samples took 21 us, 12 of them in the gradient; 17 us here.
+// batch, 4,096 samples took 21 us, 12 of them in the gradient; 17 us here with two CTAs an SM,
+// 15 with one that keeps gelu'(z1) in registers from the forward to the backward pass.
 struct AdamArgs {
     float lr, b1, b2, eps;
 };
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+__global__ void __launch_bounds__(kThreads, 1)
     k_mlp_epoch(float *w, float *m, float *v, float *grad, const float4 *__restrict__ F, const float *__restrict__ T,
                 int64_t n, int64_t batch, uint64_t pa, uint64_t pc, int64_t step, AdamArgs h, double *acc,
                 float *history, GridBar *gbar, int *err)
@@ -560,14 +567,15 @@ cudaError_t set_attr()
     return cudaFuncSetAttribute(k_mlp_epoch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
-// CTAs of the gradient kernel over a batch: one per tile, at most two per SM.
-unsigned grad_grid(int64_t batch)
+// CTAs over a batch: one per tile, at most two per SM (training, which keeps more in registers:
+// one).
+unsigned grad_grid(int64_t batch, int per_sm = kCtasPerSm)
 {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         nsm = 1;
-    return (unsigned)std::min<int64_t>((batch + 127) / 128, (int64_t)nsm * kCtasPerSm);
+    return (unsigned)std::min<int64_t>((batch + 127) / 128, (int64_t)nsm * per_sm);
 }
 
 }  // namespace
@@ -636,7 +644,7 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
         const float *Te = Ts;
         void *args[] = {&params, &m, &v, &grad, &Fe, &Te, (void *)&n, (void *)&B, (void *)&a, (void *)&c, &step, &h, &acc,
                         &hist, &gbar, &err};
-        ok = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_mlp_epoch), dim3(grad_grid(std::min(B, n))),
+        ok = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_mlp_epoch), dim3(grad_grid(std::min(B, n), 1)),
                                          dim3(kThreads), args, kSmem, s) == cudaSuccess;
         step += (n + B - 1) / B;
     }
