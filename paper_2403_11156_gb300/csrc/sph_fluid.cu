@@ -427,28 +427,38 @@ __global__ void __launch_bounds__(kBlock) k_density_sum(Ptrs P)
     density_sums<T, false>(P, c, pi, c.valid ? P.nnf[c.i] : 0, c.valid ? P.nnb[c.i] : 0);
 }
 
-// The same sweep by T threads a particle, for contexts too small to fill the GPU otherwise: the
-// T lanes test T consecutive candidates at a time with the exact predicate and append the hits
-// in candidate order (ballot over the group), so the list is the same.  Eight blocks per SM (64
-// registers for the batched cooperative append).
-template <int T>
+// The same sweep by G threads a particle, for contexts too small to fill the GPU otherwise: lane
+// r of the group loads the range of stencil row r, all in one memory latency, and for row after
+// row the lanes test G consecutive candidates at a time with the exact predicate and append the
+// hits in candidate order (ballot over the group), so the list is the same.  T of the G lanes
+// then sum, T as in the context's other sweeps, whatever G.  G is the most of 32, 16 and 8 whose
+// threads still fit the GPU: four steps of 8k particles 475 -> 467 us with 32, a step of 20k 236 ->
+// 224 with 16 (both against 8 that loaded their ranges row by row).  Eight blocks per SM (64 registers for the batched cooperative append).
+template <int T, int G>
 __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
 {
     kernel_enter(P.ctl, KID_DENSITY);
-    const Lane<T> c = lane_ctx<T>(P);
-    const SceneDev &sc = *c.sc;
-    const int64_t i = c.i, NF = P.NF;
-    const int s = c.s;
-    int nn_f = 0, nn_b = 0;  // this lane's neighbours (may exceed its capacity)
+    // a block takes 1 / (G / T) of the particles of a sweep block
+    constexpr int kSplit = G / T;
+    const int32_t block = (int32_t)blockIdx.x / kSplit;
+    const int32_t sidx = P.tblk_scene[block];
+    const SceneDev &sc = P.scenes[sidx];
+    SceneState &st = P.st[sidx];
+    const int64_t local = (int64_t)(block - sc.tblk_first) * (kBlock / T) + ((int32_t)blockIdx.x % kSplit) * (kBlock / G) +
+                          threadIdx.x / G;
+    const bool valid = local < sc.nf;
+    const int64_t i = sc.f_off + local, NF = P.NF;
+    const int s = (int)(threadIdx.x % G);
+    int nn_f = 0, nn_b = 0;  // the particle's neighbours (may exceed the capacity)
     float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (c.valid) {
+    if (valid) {
         pi = P.pos_s[i];
         const int32_t cx = cell_coord(pi.x, sc.origin[0], sc.cell, sc.dims[0]);
         const int32_t cy = cell_coord(pi.y, sc.origin[1], sc.cell, sc.dims[1]);
         const int32_t cz = cell_coord(pi.z, sc.origin[2], sc.cell, sc.dims[2]);
-        const int32_t R = sc.R;
         // a boundary particle in the stencil
         const bool walls = P.bnear[sc.c_off + cx + (int64_t)sc.dims[0] * (cy + (int64_t)sc.dims[1] * cz)] != 0;
+        const int32_t R = sc.R, side = 2 * R + 1, rows = side * side;
         const float h2 = sc.h2, cull2 = sc.cull2, cs = sc.cell;
         // offset of the particle inside its cell, per axis: the distance from the particle
         // to a stencil cell d cells away is at least gap(d) (zero for d = 0)
@@ -461,55 +471,55 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
         };
         const int cap_f = sc.cap_f, cap_b = sc.cap_b;
         const uint32_t self = (uint32_t)i;
-        // the group's lanes relative to this one (cooperative append)
-        const unsigned gmask = group_mask<T>();
-        const int gshift = (int)(threadIdx.x & 31u) & ~(T - 1);
+        const unsigned gmask = group_mask<G>();
+        const int gshift = (int)(threadIdx.x & 31u) & ~(G - 1);
         const unsigned below = (1u << s) - 1u;
-        // phase 1: the float predicate over the stencil's index ranges only records
-        // neighbours; keeping the per-pair work out of this loop keeps the warp converged
-        // while most candidates are rejected.  Rows and end cells whose nearest point is
-        // farther than h (plus a margin above the rounding of these bounds) are skipped:
-        // they hold no particle that passes the predicate, so the lists are unchanged.
-        for (int32_t dz = -R; dz <= R; ++dz) {
-            const int32_t z = cz + dz;
-            if (z < 0 || z >= sc.dims[2]) continue;
-            const float gz = gap(oz, dz);
-            for (int32_t dy = -R; dy <= R; ++dy) {
-                const int32_t y = cy + dy;
-                if (y < 0 || y >= sc.dims[1]) continue;
-                int32_t x0 = cx - R, x1 = cx + R;
-                const float gy = gap(oy, dy);
-                const float g2 = fmaf(gy, gy, gz * gz);
-                if (g2 > cull2) continue;
-                while (x0 < cx && fmaf(gap(ox, x0 - cx), gap(ox, x0 - cx), g2) > cull2) ++x0;
-                while (x1 > cx && fmaf(gap(ox, x1 - cx), gap(ox, x1 - cx), g2) > cull2) --x1;
-                x0 = max(x0, 0);
-                x1 = min(x1, sc.dims[0] - 1);
-                const int64_t row = sc.c_off + (int64_t)sc.dims[0] * (y + (int64_t)sc.dims[1] * z);
-                const uint32_t jb = P.cell_start[row + x0], je = P.cell_start[row + x1 + 1];
-                // the group's lanes test T consecutive candidates at a time and append the
-                // hits in candidate order; full batches of kCand groups load all their
-                // candidates before the first test (one memory latency per batch)
+        // The float predicate over the stencil's index ranges only records neighbours.  Rows and
+        // end cells whose nearest point is farther than h (plus a margin above the rounding of
+        // these bounds) are skipped: they hold no particle that passes the predicate.
+        for (int32_t r0 = 0; r0 < rows; r0 += G) {
+            uint32_t jb_r = 0, je_r = 0, bb_r = 0, be_r = 0;
+            if (r0 + s < rows) {
+                const int32_t dz = (r0 + s) / side - R, dy = (r0 + s) % side - R, z = cz + dz, y = cy + dy;
+                const float gz = gap(oz, dz), gy = gap(oy, dy), g2 = fmaf(gy, gy, gz * gz);
+                if (z >= 0 && z < sc.dims[2] && y >= 0 && y < sc.dims[1] && !(g2 > cull2)) {
+                    int32_t x0 = cx - R, x1 = cx + R;
+                    while (x0 < cx && fmaf(gap(ox, x0 - cx), gap(ox, x0 - cx), g2) > cull2) ++x0;
+                    while (x1 > cx && fmaf(gap(ox, x1 - cx), gap(ox, x1 - cx), g2) > cull2) --x1;
+                    x0 = max(x0, 0);
+                    x1 = min(x1, sc.dims[0] - 1);
+                    const int64_t row = sc.c_off + (int64_t)sc.dims[0] * (y + (int64_t)sc.dims[1] * z);
+                    jb_r = P.cell_start[row + x0];
+                    je_r = P.cell_start[row + x1 + 1];
+                    if (walls) {
+                        bb_r = P.bcell_start[row + x0];
+                        be_r = P.bcell_start[row + x1 + 1];
+                    }
+                }
+            }
+            for (int32_t r = 0; r < min(G, rows - r0); ++r) {
+                const uint32_t jb = __shfl_sync(gmask, jb_r, r, G), je = __shfl_sync(gmask, je_r, r, G);
+                // full batches of kCand groups load all their candidates before the first test
                 auto append = [&](uint32_t j, bool hit) {
-                    const unsigned bits = __ballot_sync(gmask, hit) >> gshift;
+                    const unsigned bits = G == 32 ? __ballot_sync(gmask, hit) : (__ballot_sync(gmask, hit) >> gshift);
                     const int slot = nn_f + __popc(bits & below);
                     if (hit && slot < cap_f) P.nbr[(int64_t)slot * NF + i] = (int32_t)j;
                     nn_f += __popc(bits);
                 };
                 constexpr int kCand = 4;
                 uint32_t j0 = jb;
-                for (; j0 + (uint32_t)(kCand * T) <= je; j0 += (uint32_t)(kCand * T)) {   // uniform in the group
+                for (; j0 + (uint32_t)(kCand * G) <= je; j0 += (uint32_t)(kCand * G)) {   // uniform in the group
                     float4 pc[kCand];
 #pragma unroll
-                    for (int u = 0; u < kCand; ++u) pc[u] = __ldg(P.pos_s + j0 + (uint32_t)(u * T + s));
+                    for (int u = 0; u < kCand; ++u) pc[u] = __ldg(P.pos_s + j0 + (uint32_t)(u * G + s));
 #pragma unroll
                     for (int u = 0; u < kCand; ++u) {
-                        const uint32_t j = j0 + (uint32_t)(u * T + s);
+                        const uint32_t j = j0 + (uint32_t)(u * G + s);
                         float dx, dy2, dz2;
                         append(j, pred_d2(pi, pc[u], dx, dy2, dz2) < h2 && j != self);
                     }
                 }
-                for (; j0 < je; j0 += (uint32_t)T) {   // uniform in the group
+                for (; j0 < je; j0 += (uint32_t)G) {   // uniform in the group
                     const uint32_t j = j0 + (uint32_t)s;
                     bool hit = false;
                     if (j < je) {
@@ -519,15 +529,15 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
                     append(j, hit);
                 }
                 if (walls) {
-                    const uint32_t bb = P.bcell_start[row + x0], be = P.bcell_start[row + x1 + 1];
-                    for (uint32_t b0 = bb; b0 < be; b0 += (uint32_t)T) {
+                    const uint32_t bb = __shfl_sync(gmask, bb_r, r, G), be = __shfl_sync(gmask, be_r, r, G);
+                    for (uint32_t b0 = bb; b0 < be; b0 += (uint32_t)G) {
                         const uint32_t b = b0 + (uint32_t)s;
                         bool hit = false;
                         if (b < be) {
                             float dx, dy2, dz2;
                             hit = pred_d2(pi, __ldg(P.bpos_s + b), dx, dy2, dz2) < h2;
                         }
-                        const unsigned bits = __ballot_sync(gmask, hit) >> gshift;
+                        const unsigned bits = G == 32 ? __ballot_sync(gmask, hit) : (__ballot_sync(gmask, hit) >> gshift);
                         const int slot = nn_b + __popc(bits & below);
                         if (hit && slot < cap_b) P.bnbr[(int64_t)slot * NF + i] = (int32_t)b;
                         nn_b += __popc(bits);
@@ -538,8 +548,9 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
         // the lists were written by the group's lanes: order them before the reads below
         __syncwarp(gmask);
     }
+    const Lane<T> c{&sc, &st, i, s % T, valid && s < T};
     density_sums<T, true>(P, c, pi, min(nn_f, sc.cap_f), min(nn_b, sc.cap_b));
-    if (c.valid && s == 0) {
+    if (valid && s == 0) {
         P.nnf[i] = min(nn_f, sc.cap_f);
         P.nnb[i] = min(nn_b, sc.cap_b);
     }
@@ -547,9 +558,9 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
     // this long sweep they cost less than a block barrier would)
     const int mf = warp_max(nn_f), mb = warp_max(nn_b);
     if ((threadIdx.x & 31) == 0) {
-        if (mf > 0) atomicMax(&c.st->max_nn_f, mf);
-        if (mb > 0) atomicMax(&c.st->max_nn_b, mb);
-        if (mf > sc.cap_f || mb > sc.cap_b) atomicOr(&c.st->flags, 1);
+        if (mf > 0) atomicMax(&st.max_nn_f, mf);
+        if (mb > 0) atomicMax(&st.max_nn_b, mb);
+        if (mf > sc.cap_f || mb > sc.cap_b) atomicOr(&st.flags, 1);
     }
 }
 
@@ -1088,7 +1099,11 @@ void launch_density_alpha(const Ptrs &P, cudaStream_t s)
     // eight: 8k particles 43 and 28 us, 38k about even); four or two lanes never did (100k: 160 us
     // with two, 55 with one).  Both write the same lists.
     if (P.lanes == 8) {
-        k_density_lanes<8><<<P.ntblk, kBlock, 0, s>>>(P);
+        // resident threads of a full GPU, as for the choice of the lanes
+        constexpr int64_t kThreads = 152 * 2048;
+        if (P.NF * 32 <= kThreads) k_density_lanes<8, 32><<<P.ntblk * 4, kBlock, 0, s>>>(P);
+        else if (P.NF * 16 <= kThreads) k_density_lanes<8, 16><<<P.ntblk * 2, kBlock, 0, s>>>(P);
+        else k_density_lanes<8, 8><<<P.ntblk, kBlock, 0, s>>>(P);
     } else if (P.lanes == 1) {
         k_density<true><<<P.nfblk, kBlock, 0, s>>>(P);
     } else {
