@@ -367,14 +367,13 @@ __global__ void k_read_boundary(Ptrs P, int scene, int field, void *out)
     }
 }
 
-// A state written by the caller replaces the canonical arrays in original particle order.
-// First launch: the present state goes to that order through the sorted arrays (what the
-// caller does not give keeps its value), and the next step's size starts from its maximum.
+// A state written by the caller replaces the canonical arrays in original particle order.  The
+// present state goes to that order through the sorted arrays (whose fields stay readable, and
+// which keep the value of what the caller does not give).
 __global__ void k_unpermute_to_sorted(Ptrs P, int scene)
 {
     const SceneDev &sc = P.scenes[scene];
     int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (local == 0) P.st[scene].dt_next = sc.dt_max;
     if (local >= sc.nf) return;
     int64_t i = sc.f_off + local;
     int64_t d = sc.f_off + P.id_c[i];
@@ -384,39 +383,50 @@ __global__ void k_unpermute_to_sorted(Ptrs P, int scene)
     P.kvprev_s[d] = P.kvprev_c[i];
 }
 
-// Second launch: the canonical arrays in original order from the caller's packed [n][3] and
-// [n] device arrays (null: the present value) and the CFL step of the new velocities,
-// min(dt_max, cfl 2r / max|v|).  Each block takes the step of its own largest speed and the
-// scene's is the minimum over the blocks: division and square root round monotonically, so
-// that is the step of the largest speed.  (As seven launches with a one-block maximum, which
-// read 1.2M velocities in 382 us, writing and reading back that state made a one-step pass
-// 2827 us; with this and the one-launch read it is 2401 us.)
+// The canonical arrays in original order from the caller's packed [n][3] and [n] device arrays
+// (null: the present value, from the sorted arrays), and the CFL step of the new velocities,
+// min(dt_max, cfl 2r / max|v|), in the block that finishes last.  ALL: every array is given, so
+// nothing is taken from the sorted arrays and this launch unpermutes the present state into them
+// itself (each thread reads its canonical slot before it overwrites it).  As seven launches with a
+// one-block maximum, which read 1.2M velocities in 382 us, writing and reading back that state
+// made a one-step pass 2827 us; 2401 with two launches and the one-launch read.
 constexpr int kWriteThreads = 256;
+template <bool ALL>
 __global__ void __launch_bounds__(kWriteThreads)
     k_write_canonical(Ptrs P, int scene, const float *__restrict__ x, const float *__restrict__ vel,
                       const float *__restrict__ kp, const float *__restrict__ kvp)
 {
     __shared__ float sh[kWriteThreads / 32];
     const SceneDev &sc = P.scenes[scene];
+    SceneState &st = P.st[scene];
     const int64_t local = (int64_t)blockIdx.x * kWriteThreads + threadIdx.x;
     float m = 0.0f;
     if (local < sc.nf) {
         const int64_t i = sc.f_off + local;
-        float4 p = P.pos_s[i], v = P.vel_s[i];
-        if (x) p = make_float4(x[3 * local], x[3 * local + 1], x[3 * local + 2], 0.0f);
-        if (vel) v = make_float4(vel[3 * local], vel[3 * local + 1], vel[3 * local + 2], 0.0f);
+        float4 p, v;
+        if (ALL) {
+            const int64_t d = sc.f_off + P.id_c[i];
+            P.pos_s[d] = P.pos_c[i];
+            P.vel_s[d] = P.vel_c[i];
+            P.kprev_s[d] = P.kprev_c[i];
+            P.kvprev_s[d] = P.kvprev_c[i];
+        } else {
+            p = P.pos_s[i];
+            v = P.vel_s[i];
+        }
+        if (ALL || x) p = make_float4(x[3 * local], x[3 * local + 1], x[3 * local + 2], 0.0f);
+        if (ALL || vel) v = make_float4(vel[3 * local], vel[3 * local + 1], vel[3 * local + 2], 0.0f);
         v.w = 0.0f;
         P.pos_c[i] = p;
         P.vel_c[i] = v;
-        P.kprev_c[i] = kp ? kp[local] : P.kprev_s[i];
-        P.kvprev_c[i] = kvp ? kvp[local] : P.kvprev_s[i];
+        P.kprev_c[i] = ALL || kp ? kp[local] : P.kprev_s[i];
+        P.kvprev_c[i] = ALL || kvp ? kvp[local] : P.kvprev_s[i];
         P.id_c[i] = (int32_t)local;
         P.id_s[i] = (int32_t)local;
         P.ksum[i] = 0.0f;
         P.kvsum[i] = 0.0f;
         m = v.x * v.x + v.y * v.y + v.z * v.z;
     }
-    if (!(sc.cfl > 0.0f)) return;
     m = fmaxf(m, 0.0f);   // a NaN counts as no speed
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -424,12 +434,16 @@ __global__ void __launch_bounds__(kWriteThreads)
     __syncthreads();
     if (threadIdx.x != 0) return;
     for (int w = 1; w < kWriteThreads / 32; ++w) m = fmaxf(m, sh[w]);
-    const float vm = sqrtf(m);
-    if (vm > 0.0f) {
-        // steps are not negative: their order is that of their bit patterns
-        const float dt = sc.cfl * sc.two_r / vm;
-        if (dt < sc.dt_max) atomicMin(reinterpret_cast<int *>(&P.st[scene].dt_next), __float_as_int(dt));
-    }
+    // squared speeds are not negative: their order is that of their bit patterns
+    atomicMax(&st.write_maxv2, __float_as_int(m));
+    __threadfence();
+    if (atomicAdd(&st.write_count, 1u) != gridDim.x - 1u) return;
+    __threadfence();
+    const float vm = sqrtf(__int_as_float(atomicExch(&st.write_maxv2, 0)));
+    st.write_count = 0u;
+    float dt = sc.dt_max;
+    if (sc.cfl > 0.0f && vm > 0.0f) dt = fminf(dt, sc.cfl * sc.two_r / vm);
+    st.dt_next = dt;
 }
 
 // ------------------------------------------------------------------ launch plumbing
@@ -1513,9 +1527,13 @@ sph_status sph_write_state(sph_ctx *c, int32_t scene, const float *x, const floa
             dv = stage.p + 3 * nf;
         }
     }
-    k_unpermute_to_sorted<<<blocks, kWriteThreads, 0, s>>>(c->P, scene);
-    k_write_canonical<<<blocks, kWriteThreads, 0, s>>>(c->P, scene, dx, dv, on_device ? kappa_prev : nullptr,
-                                                       on_device ? kappa_v_prev : nullptr);
+    if (on_device && x && v && kappa_prev && kappa_v_prev) {
+        k_write_canonical<true><<<blocks, kWriteThreads, 0, s>>>(c->P, scene, x, v, kappa_prev, kappa_v_prev);
+    } else {
+        k_unpermute_to_sorted<<<blocks, kWriteThreads, 0, s>>>(c->P, scene);
+        k_write_canonical<false><<<blocks, kWriteThreads, 0, s>>>(c->P, scene, dx, dv, on_device ? kappa_prev : nullptr,
+                                                                  on_device ? kappa_v_prev : nullptr);
+    }
     if ((st = check_async(c)) != SPH_OK) return st;
     if (!on_device && kappa_prev)
         CK(cudaMemcpyAsync(c->P.kprev_c + q.f_off, kappa_prev, 4 * nf, cudaMemcpyHostToDevice, s));

@@ -80,7 +80,8 @@ struct SceneState {
     int64_t steps;
     int64_t total_it[2];
     int32_t last_it[2];               // iterations of the previous step
-    int32_t pad_s[2];
+    uint32_t write_count;             // sph_write_state: blocks done, and the largest |v|^2 bits
+    int32_t write_maxv2;
 };
 
 // Rigid body state (device, FP64).
