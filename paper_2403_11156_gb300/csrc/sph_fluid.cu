@@ -133,10 +133,16 @@ __global__ void k_step_begin(Ptrs P)
 // A particle whose passed candidates exceed the list, or that has left the range the filter
 // holds for (SceneDev::qmax), takes the exact predicate over its rows instead.
 //
-// Bound by instruction issue and gather latency in turn: at 500k particles 154 us (167 with the
-// exact predicate on every candidate and boundary rows looked up by all), of which the filter
-// takes about 50, the list writes 38 and phase 2 53; 1.2M with bodies 357 us (396).  With two and
-// four lanes the lists are built here and the lanes only sum: 100k particles 160 -> 58 us.
+// Between the phases a thread keeps its first kStage passed candidates in shared memory: written
+// straight to the list, whose entries the lanes of a warp reach at different times, each store
+// touched its own line, and phase 2 read them back from memory.  Phase 2 writes the list entry by
+// entry with the warp in step.
+//
+// Bound by instruction issue and gather latency in turn: at 500k particles 146 us (167 with the
+// exact predicate on every candidate and boundary rows looked up by all, 154 without the stage),
+// 1.2M with bodies 343 us (396, 356).  24 staged candidates, which 28 neighbours overrun, take 153
+// and 355.  With two and four lanes the lists are built here and the lanes only sum: 100k particles
+// 160 -> 59 us.
 __device__ __forceinline__ uint32_t query_pair(uint32_t word, uint32_t odd)
 {
     return ((0x6600u - (odd ? word >> 16 : word)) & 0xffffu) * 0x10001u;
@@ -168,9 +174,11 @@ __device__ __noinline__ int exact_list(const Ptrs &P, const Stencil &st, int64_t
     return n;
 }
 
+constexpr int kStage = 32;   // candidates a thread keeps in shared memory between the phases
 template <bool SUM>
 __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ Ptrs P)
 {
+    __shared__ int32_t s_list[kStage][kBlock];
     kernel_enter(P.ctl, KID_DENSITY);
     const BlockCtx c = fluid_ctx(P);
     const SceneDev &sc = *c.sc;
@@ -207,7 +215,6 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
             const uint32_t qx = query_pair(own.x, self & 1u), qy = query_pair(own.y, self & 1u),
                            qz = query_pair(own.z, self & 1u);
             const __half2 thr = as_half2(sc.qthr), unit = __float2half2_rn(1.0f / 512.0f), bias = __float2half2_rn(-3.0f);
-            int32_t *slot = P.nbr + i;
             const int32_t rows = st.ny * st.nz;
             uint32_t row = st.row;
             for (int32_t k = 0, y = 0; k < rows; ++k) {
@@ -238,11 +245,13 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
                     uint32_t near = ~far & (0xffffffffu >> (32u - n));
                     if (c0 < jb) near &= ~1u;
                     if (k == st.centre && self - c0 < 32u) near &= ~(1u << (self - c0));
+                    int q = passed;
                     passed += __popc(near);
                     if (passed > cap_f) near = 0u;   // the exact predicate builds the list instead
-                    for (; near != 0u; near &= near - 1u) {
-                        *slot = (int32_t)(c0 + (uint32_t)__ffs((int)near) - 1u);
-                        slot += NF;
+                    for (; near != 0u; near &= near - 1u, ++q) {
+                        const int32_t j = (int32_t)(c0 + (uint32_t)__ffs((int)near) - 1u);
+                        if (q < kStage) s_list[q][threadIdx.x] = j;
+                        else P.nbr[(int64_t)q * NF + i] = j;
                     }
                 }
             }
@@ -271,28 +280,38 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
         const float4 vi = P.vel_s[i];
         const Spline sp(sc);
         float w_sum = 0.0f, s1x = 0.0f, s1y = 0.0f, s1z = 0.0f, s2 = 0.0f, div_l = 0.0f;
-        int k = 0;
-        for_list<2, 1, false>(P.nbr, NF, i, 0, passed, [&](int32_t j) {
-            const float4 pj = __ldg(P.pos_s + j);
+        // the passed candidates are in shared memory (the rest, and a list built by the exact
+        // predicate, in the list itself, which is read ahead of where it is written)
+        const int staged = total < 0 ? kStage : 0;
+        auto candidate = [&](int k) { return k < staged ? s_list[k][threadIdx.x] : P.nbr[(int64_t)k * NF + i]; };
+        auto visit = [&](int32_t j, float4 pj) {
             float dx, dy2, dz2;
             const float d2 = pred_d2(pi, pj, dx, dy2, dz2);
-            if (d2 < h2) {
-                if (nn_f != k) P.nbr[(int64_t)nn_f * NF + i] = j;
-                ++nn_f;
+            if (!(d2 < h2)) return;
+            P.nbr[(int64_t)nn_f * NF + i] = j;
+            ++nn_f;
+            if (!SUM) return;
+            w_sum += spline_w(sqrtf(d2) * sp.inv_h);
+            const float f = grad_factor(sp, d2);
+            const float gx = f * dx, gy = f * dy2, gz = f * dz2;
+            s1x += gx; s1y += gy; s1z += gz;
+            s2 = fmaf(gx, gx, fmaf(gy, gy, fmaf(gz, gz, s2)));
+            if (gate) {
+                const float4 vj = __ldg(P.vel_s + j);
+                div_l += (vi.x - vj.x) * gx + (vi.y - vj.y) * gy + (vi.z - vj.z) * gz;
             }
-            ++k;
-            if (SUM && d2 < h2) {
-                w_sum += spline_w(sqrtf(d2) * sp.inv_h);
-                const float f = grad_factor(sp, d2);
-                const float gx = f * dx, gy = f * dy2, gz = f * dz2;
-                s1x += gx; s1y += gy; s1z += gz;
-                s2 = fmaf(gx, gx, fmaf(gy, gy, fmaf(gz, gz, s2)));
-                if (gate) {
-                    const float4 vj = __ldg(P.vel_s + j);
-                    div_l += (vi.x - vj.x) * gx + (vi.y - vj.y) * gy + (vi.z - vj.z) * gz;
-                }
-            }
-        });
+        };
+        int k = 0;
+        for (; k + 2 <= passed; k += 2) {
+            const int32_t j0 = candidate(k), j1 = candidate(k + 1);
+            const float4 p0 = __ldg(P.pos_s + j0), p1 = __ldg(P.pos_s + j1);
+            visit(j0, p0);
+            visit(j1, p1);
+        }
+        if (k < passed) {
+            const int32_t j0 = candidate(k);
+            visit(j0, __ldg(P.pos_s + j0));
+        }
         const int nb = min(nn_b, cap_b);
         P.nnf[i] = nn_f;
         P.nnb[i] = nb;
