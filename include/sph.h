@@ -453,7 +453,8 @@ sph_status sph_grid_order_noalloc(const float *x, int64_t n, const float *domain
 /* Outcome of the last sph_grid_order_noalloc call on the current device: synchronises
  * stream (the one that call used), then reads the scratch array's error word into host
  * memory with a copy from the symbol (no allocation).  SPH_ETIMEOUT: a bounded wait of the
- * call's look-back prefix scan ran out, so its order is not valid (the GPU stays usable);
+ * call ran out, or a call that overlapped disturbed its histogram, so its order is not
+ * valid (the GPU stays usable);
  * SPH_OK: it completed; SPH_ECUDA: the synchronisation or the copy failed.  The word is
  * cleared by every call, so a later or overlapping call replaces it.  Not for use inside a
  * stream capture (it synchronises). */

@@ -121,7 +121,7 @@ __device__ void sort_cell(const View &v, uint32_t b, uint32_t e, int32_t *order)
 // The whole order in one cooperative launch: keys and histogram, prefix sum (each block sums its
 // share of the cells, then adds the shares before it), scatter, rank inside the cell by index or,
 // for the crowded cells, which the prefix sum queues, block sort; four barriers.  The histogram
-// is zero between calls: the prefix sum clears what it has read.  As six launches it was bound
+// is zero between calls: the prefix sum clears what it has read, and its total has to be n.  As six launches it was bound
 // by them: 262,143 points 39.0 -> 24.6 us.
 __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, const float *__restrict__ x, int64_t n,
                                                             int64_t ncell, uint32_t *keys_out, int32_t *order, int slot)
@@ -154,8 +154,18 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
     }
     if (!grid_barrier(bar, &ctl->error, phase)) return;
     {
-        uint32_t run = 0u;
-        block_scan(threadIdx.x < blockIdx.x ? v.sums[threadIdx.x] : 0u, run);   // shares before this one
+        __shared__ uint32_t s_run;
+        const uint32_t before_me = block_scan(threadIdx.x < gridDim.x ? v.sums[threadIdx.x] : 0u, total);
+        if (threadIdx.x == blockIdx.x) s_run = before_me;   // shares before this one
+        __syncthreads();
+        uint32_t run = s_run;
+        if (total != (uint32_t)n) {
+            // the histogram was not this call's alone (a call that overlapped, now or earlier):
+            // clear it for the next one and say so instead of scattering by it (every block alike)
+            for (int64_t c = c0 + threadIdx.x; c < c1; c += kLargeThreads) v.count[c] = 0u;
+            if (threadIdx.x == 0) atomicExch(&ctl->error, 7);
+            return;
+        }
         for (int64_t c = c0; c < c1; c += kLargeThreads) {
             const int64_t at = c + threadIdx.x;
             const uint32_t k = at < c1 ? v.count[at] : 0u;
