@@ -54,22 +54,23 @@ BOUNDARY_BYTES = 16                             # x_b, Psi_b per boundary partic
 # now (the roofline's `traffic`; null for any other kernel or configuration).  Filled from
 # the committed captures (profiles/*_dam_break_1.2M.md); a kernel changed since its capture
 # has no entry.
-TRAFFIC = {("density_alpha", 1, 4, 27): 82.70e6 + 169.47e6,
+TRAFFIC = {("density_alpha", 1, 4, 27): 68.49e6 + 157.95e6,
            ("dens_pass_a", 1, 4, 27): 211.59e6 + 4.72e6,
            ("dens_pass_b", 1, 4, 27): 199.69e6 + 4.33e6}
 # L1 data-pipe (LSU) wavefronts per launch measured by ncu in the same captures
 # (l1tex__data_pipe_lsu_wavefronts, per-SM average x 152 SMs).  The pipe takes one wavefront per
 # SM per cycle, so over the live launch time this is the fraction of the roof that binds the
 # neighbour gathers.
-L1_WAVEFRONTS = {("density_alpha", 1, 4, 27): 617053.83 * 152,
+L1_WAVEFRONTS = {("density_alpha", 1, 4, 27): 442185.92 * 152,
                  ("dens_pass_a", 1, 4, 27): 203077.14 * 152,
                  ("dens_pass_b", 1, 4, 27): 124865.32 * 152}
 # FP32 operations per neighbour pair in the list sweeps (distance, spline gradient, dot)
 FLOPS_PER_PAIR = {"dens_pass_a": 26, "div_pass_a": 24, "dens_pass_b": 22, "div_pass_b": 22,
                   "dens_warm_pass_b": 22, "div_warm_pass_b": 22, "nonpressure": 30,
                   "warm_density": 26, "density_alpha": 40}
-# extra FP32 operations per fluid particle outside the pair sums: the density sweep's
-# candidate tests (about 216 per particle at 8 flop each: 3 differences, 3 products, 2 sums)
+# extra operations per fluid particle outside the pair sums: the density sweep's candidate
+# tests (about 216 per particle at 8 flop each: 3 differences, 3 products, 2 sums; in half
+# precision, two at a time)
 FLOPS_PER_PARTICLE = {"density_alpha": 216 * 8}
 # the kernels reported with a roofline of their own (the step's three largest)
 ROOFLINE_KERNELS = ("density_alpha", "dens_pass_a", "dens_pass_b")

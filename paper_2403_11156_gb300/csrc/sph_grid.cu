@@ -141,9 +141,8 @@ __global__ void __launch_bounds__(kLargeThreads) k_rank_large(Ptrs P)
         const uint32_t cell = large[q];
         const uint32_t b = start[cell], e = start[cell + 1];
         block_sort_segment(sid, src, sid2, src2, b, e);
-        int32_t s0 = 0;   // the cell's scene: cells of a context are numbered scene after scene
-        while (s0 + 1 < P.nscenes && (int64_t)cell >= P.scenes[s0 + 1].c_off) ++s0;
-        for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) gather_one<WHAT>(P, P.scenes[s0], d, src[d], sid[d]);
+        const SceneDev &sc = P.scenes[scene_of_cell(P, (int64_t)cell)];
+        for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) gather_one<WHAT>(P, sc, d, src[d], sid[d]);
         __syncthreads();
     }
 }

@@ -292,6 +292,18 @@ struct Ptrs {
 };
 
 // ------------------------------------------------------------------ grid (sph_grid.cu)
+// Scene of a global cell: cells of a context are numbered scene after scene.
+__device__ __forceinline__ int32_t scene_of_cell(const Ptrs &P, int64_t cell)
+{
+    int32_t lo = 0, hi = P.nscenes - 1;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi + 1) / 2;
+        if (P.scenes[mid].c_off <= cell) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
 // Cell coordinate under the float contract: clamp(floor((x - o)/c), 0, n-1).
 __device__ __forceinline__ int32_t cell_coord(float x, float o, float c, int32_t n)
 {

@@ -83,9 +83,7 @@ __global__ void __launch_bounds__(256) k_boundary_near(Ptrs P)
 {
     kernel_enter(P.ctl, KID_BNEAR);
     for (int64_t cell = (int64_t)blockIdx.x * 256 + threadIdx.x; cell < P.NC; cell += (int64_t)gridDim.x * 256) {
-        int32_t s = 0;
-        while (s + 1 < P.nscenes && cell >= P.scenes[s + 1].c_off) ++s;
-        const SceneDev &sc = P.scenes[s];
+        const SceneDev &sc = P.scenes[scene_of_cell(P, cell)];
         const uint32_t k = (uint32_t)(cell - sc.c_off), row = k / (uint32_t)sc.dims[0];
         const int32_t x = (int32_t)(k - row * (uint32_t)sc.dims[0]), z = (int32_t)(row / (uint32_t)sc.dims[1]),
                       y = (int32_t)(row - (uint32_t)z * (uint32_t)sc.dims[1]), R = sc.R;

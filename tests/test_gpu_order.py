@@ -34,3 +34,29 @@ def test_order(n, cells, crowd):
         np.testing.assert_array_equal(order.cpu().numpy(), order_o)
         if keys_too:
             np.testing.assert_array_equal(keys.cpu().numpy().view(np.uint32), keys_o)
+
+
+@pytest.mark.parametrize("n,cells", [(3001, 20), (50_000, 40)])
+def test_order_under_capture(n, cells):
+    """Enqueued into another component's graph capture, and replayed on other points."""
+    import torch
+    rng = np.random.default_rng(n)
+    extent = 0.04 * cells
+    lo, hi = np.zeros(3, np.float32), np.full(3, extent, np.float32)
+    x = torch.zeros((n, 3), device="cuda")
+    order = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        assert sph.sph_grid_order_noalloc(x, n, lo, hi, np.float32(0.04), order, None, stream) == sph.SPH_OK
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        assert sph.sph_grid_order_noalloc(x, n, lo, hi, np.float32(0.04), order, None, stream) == sph.SPH_OK
+    for _ in range(3):
+        pts = rng.uniform(0, extent, (n, 3)).astype(np.float32)
+        x.copy_(torch.from_numpy(pts))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        want = oracle.sort_order(oracle.cell_keys(pts, lo, hi, np.float32(0.04)))
+        np.testing.assert_array_equal(order.cpu().numpy(), want)
