@@ -587,11 +587,15 @@ sph_status enqueue_step(sph_ctx *c, cudaStream_t s, bool capture)
     if (c->any_implicit) {
         run(c, s, "cg_init", [&] { launch_cg_init(P, s); });
         st = device_loop([&](cudaStream_t q, cudaGraphConditionalHandle h, int use) {
-            run(c, q, "cg_ap", [&] { launch_cg_ap(P, q); });
-            run(c, q, "cg_alpha", [&] { launch_cg_alpha(P, q); });
-            run(c, q, "cg_xr", [&] { launch_cg_xr(P, q); });
-            run(c, q, "cg_beta", [&] { launch_cg_beta(P, h, use, q); });
-            run(c, q, "cg_p", [&] { launch_cg_p(P, q); });
+            // two iterations a turn of the while node (20 to 40 are usual); the second's kernels
+            // find no active scene where the first was the last
+            for (int turn = 0; turn < 2; ++turn) {
+                run(c, q, "cg_ap", [&] { launch_cg_ap(P, q); });
+                run(c, q, "cg_alpha", [&] { launch_cg_alpha(P, q); });
+                run(c, q, "cg_xr", [&] { launch_cg_xr(P, q); });
+                run(c, q, "cg_beta", [&] { launch_cg_beta(P, h, use, q); });
+                run(c, q, "cg_p", [&] { launch_cg_p(P, q); });
+            }
         });
         if (st != SPH_OK) return st;
     }
