@@ -36,7 +36,7 @@ struct BlockCtx {
 __device__ __forceinline__ BlockCtx fluid_ctx(const Ptrs &P)
 {
     BlockCtx c;
-    int32_t s = P.fblk_scene[blockIdx.x];
+    int32_t s = scene_of_block(P, P.fblk_scene, (int32_t)blockIdx.x);
     c.sc = &P.scenes[s];
     c.st = &P.st[s];
     int64_t local = (int64_t)(blockIdx.x - c.sc->fblk_first) * kBlock + threadIdx.x;
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
     // a block takes 1 / (G / T) of the particles of a sweep block
     constexpr int kSplit = G / T;
     const int32_t block = (int32_t)blockIdx.x / kSplit;
-    const int32_t sidx = P.tblk_scene[block];
+    const int32_t sidx = scene_of_block(P, P.tblk_scene, block);
     const SceneDev &sc = P.scenes[sidx];
     SceneState &st = P.st[sidx];
     const int64_t local = (int64_t)(block - sc.tblk_first) * (kBlock / T) + ((int32_t)blockIdx.x % kSplit) * (kBlock / G) +
@@ -586,17 +586,18 @@ __global__ void __launch_bounds__(kBlock, 8) k_density_lanes(Ptrs P)
 // ------------------------------------------------------------------------------------
 // This lane's share of D rho_i/Dt = sum_j m (v_i - v_j).grad W_ij + sum_b Psi_b (v_i -
 // v_b).grad W_ib (SPH divergence of Sec. 3.2 in the continuity equation, boundary per
-// Sec. 3.5); group_sum of the shares is the full sum.
+// Sec. 3.5); group_sum of the shares is the full sum.  nf, nb: the list lengths (nb < 0: loaded
+// where it is needed, which saves a register over the fluid list).
 constexpr int kBatch = 4;
 
 template <int B, int T, bool NC = true>
 __device__ __forceinline__ float drho_dt_lane(const Ptrs &P, const SceneDev &sc, int64_t i, int s, float4 pi,
-                                              float4 vi, const float4 *V)
+                                              float4 vi, const float4 *V, int nf, int nb)
 {
     const int64_t NF = P.NF;
     const Spline sp(sc);
     float acc = 0.0f;
-    for_list<B, T>(P.nbr, NF, i, s, P.nnf[i], [&](int32_t j) {
+    for_list<B, T>(P.nbr, NF, i, s, nf, [&](int32_t j) {
         const float4 pj = ld4<NC>(P.pos_s + j);
         const float4 vj = ld4<NC>(V + j);
         const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
@@ -605,7 +606,7 @@ __device__ __forceinline__ float drho_dt_lane(const Ptrs &P, const SceneDev &sc,
     });
     float accb = 0.0f;
     const bool moving = sc.has_moving != 0;
-    for_list<4, T>(P.bnbr, NF, i, s, P.nnb[i], [&](int32_t b) {
+    for_list<4, T>(P.bnbr, NF, i, s, nb < 0 ? P.nnb[i] : nb, [&](int32_t b) {
         const float4 pb = __ldg(P.bpos_s + b);
         const float dx = pi.x - pb.x, dy = pi.y - pb.y, dz = pi.z - pb.z;
         const float f = pb.w * grad_factor(sp, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
@@ -628,39 +629,59 @@ __device__ __forceinline__ void pass_a(const Ptrs &P, int32_t block, double *sh)
     const Lane<T> c = lane_ctx<T>(P, block);
     const SceneDev &sc = *c.sc;
     SceneState &st = *c.st;
-    if (!solver_active(sc, st, S)) return;  // uniform per block
-    const float dt = st.dt;
     const float4 *V = S == 0 ? P.vel_s : P.vel_c;
     const int64_t i = c.i;
+    // with several lanes, where latency is what a pass consists of, the particle's own loads, also
+    // those the pass's end needs, go with those of the scene's state
     float4 pi = make_float4(0.f, 0.f, 0.f, 0.f), vi = pi;
-    float D = 0.0f;
-    if (c.valid) {
+    int nf = 0, nb = T > 1 ? 0 : -1;
+    float alpha = 0.0f, ks = 0.0f;
+    float *sum = S == 0 ? P.kvsum : P.ksum;
+    if (T > 1 && c.valid) {
         pi = P.pos_s[i];
         vi = V[i];
-        D = drho_dt_lane<B, T, NC>(P, sc, i, c.s, pi, vi, V);
+        nf = P.nnf[i];
+        nb = P.nnb[i];
+        alpha = P.alpha[i];
+        ks = sum[i];
+    }
+    if (!solver_active(sc, st, S)) return;  // uniform per block
+    const float dt = st.dt;
+    float D = 0.0f;
+    if (c.valid) {
+        if (T == 1) {
+            pi = P.pos_s[i];
+            vi = V[i];
+            nf = P.nnf[i];
+        }
+        D = drho_dt_lane<B, T, NC>(P, sc, i, c.s, pi, vi, V, nf, nb);
     }
     D = group_sum<T>(D);
     double e = 0.0;
     if (c.valid && c.s == 0) {
         const float rho = vi.w;
+        if (T == 1) {
+            alpha = P.alpha[i];
+            ks = sum[i];
+        }
         float ei, kappa;
         if (S == 0) {
             ei = fmaxf(D, 0.0f);
-            kappa = P.alpha[i] * ei / dt;
-            P.kvsum[i] += kappa;
+            kappa = alpha * ei / dt;
+            sum[i] = ks + kappa;
         } else if (sc.solver == 2) {
             // PCISPH: refine the total pressure p <- max(p + delta (rho* - rho0), 0) with
             // the prototype's delta; the pass B applies the change (kept as p/rho)
             const float dev = fmaf(dt, D, rho - sc.rho0);
             ei = fmaxf(dev, 0.0f);
-            const float p_old = P.ksum[i] * rho;
+            const float p_old = ks * rho;
             const float p_new = fmaxf(fmaf(sc.pci_c / (dt * dt), dev, p_old), 0.0f);
             kappa = (p_new - p_old) / rho;
-            P.ksum[i] = p_new / rho;
+            sum[i] = p_new / rho;
         } else {
             ei = fmaxf(fmaf(dt, D, rho - sc.rho0), 0.0f);
-            kappa = P.alpha[i] * ei / (dt * dt);
-            P.ksum[i] += kappa;
+            kappa = alpha * ei / (dt * dt);
+            sum[i] = ks + kappa;
         }
         set_w(P.pos_s, i, kappa / rho);
         e = (double)ei;
@@ -698,16 +719,26 @@ __device__ __forceinline__ void pass_b(const Ptrs &P, int32_t block)
     // uniform per block; WCSPH scenes apply their equation-of-state pressure here.  In the
     // loop, a scene's pass B runs exactly when its pass A did: the solver state only
     // changes in the check kernel that follows.
+    // (With several lanes the particle's own loads go first, as in pass A.)
+    float4 *V = S == 0 ? P.vel_s : P.vel_c;
+    float4 own = make_float4(0.f, 0.f, 0.f, 0.f), v = own;
+    int nf = 0, nb = 0;
+    if (T > 1 && c.valid) {
+        own = P.pos_s[c.i];
+        nf = P.nnf[c.i];
+        nb = P.nnb[c.i];
+        if (c.s == 0) v = V[c.i];
+    }
     const bool run = WARM ? warm_pass_runs(sc, S) : solver_active(sc, st, S);
     if (run) {
         const int64_t i = c.i, NF = P.NF;
         const int s = c.s;
         float ax = 0.0f, ay = 0.0f, az = 0.0f;
         if (c.valid) {
-            const float4 pi = P.pos_s[i];
+            const float4 pi = T > 1 ? own : P.pos_s[i];
             const float ki = pi.w;
             const Spline sp(sc);
-            for_list<B, T>(P.nbr, NF, i, s, P.nnf[i], [&](int32_t j) {
+            for_list<B, T>(P.nbr, NF, i, s, T > 1 ? nf : P.nnf[i], [&](int32_t j) {
                 const float4 pj = ld4<NC>(P.pos_s + j);
                 const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
                 const float f = grad_factor(sp, fmaf(dx, dx, fmaf(dy, dy, dz * dz))) * (ki + pj.w);
@@ -716,7 +747,7 @@ __device__ __forceinline__ void pass_b(const Ptrs &P, int32_t block)
             ax *= sc.m; ay *= sc.m; az *= sc.m;
             if (ki != 0.0f) {
                 float bx = 0.0f, by = 0.0f, bz = 0.0f;
-                for_list<4, T>(P.bnbr, NF, i, s, P.nnb[i], [&](int32_t b) {
+                for_list<4, T>(P.bnbr, NF, i, s, T > 1 ? nb : P.nnb[i], [&](int32_t b) {
                     const float4 pb = __ldg(P.bpos_s + b);
                     const float dx = pi.x - pb.x, dy = pi.y - pb.y, dz = pi.z - pb.z;
                     const float f = pb.w * grad_factor(sp, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
@@ -727,9 +758,8 @@ __device__ __forceinline__ void pass_b(const Ptrs &P, int32_t block)
         }
         ax = group_sum<T>(ax); ay = group_sum<T>(ay); az = group_sum<T>(az);
         if (c.valid && s == 0) {
-            float4 *V = S == 0 ? P.vel_s : P.vel_c;
             const float dt = st.dt;
-            float4 v = V[i];
+            if (T == 1) v = V[i];
             v.x -= dt * ax; v.y -= dt * ay; v.z -= dt * az;
             V[i] = v;
         }
@@ -772,12 +802,12 @@ __device__ __forceinline__ uint32_t solver_check(const Ptrs &P, int *s_any)
     for (int q = warp; q < P.nscenes; q += (int)(blockDim.x / 32)) {
         const SceneDev &qd = P.scenes[q];
         SceneState &qs = P.st[q];
-        if (!solver_active(qd, qs, S)) continue;   // its pass A and B did not run
         const int32_t F = fold_size(qd.tblk_count);
         const int32_t nfold = (qd.tblk_count + F - 1) / F;
         double t = 0.0;
 #pragma unroll 8
         for (int k = lane; k < nfold; k += 32) t += __ldcg(P.partial2 + qd.tblk_first + k);
+        if (!solver_active(qd, qs, S)) continue;   // its pass A and B did not run
         t = warp_sum(t);
         if (lane == 0) {
             double err = t * qd.err_scale;   // FP64 division is a long sequence here
@@ -933,7 +963,7 @@ __global__ void __launch_bounds__(kBlock) k_warm_density(Ptrs P)
     if (c.valid) {
         pi = P.pos_s[i];
         vi = P.vel_c[i];
-        D = drho_dt_lane<kBatch, T>(P, sc, i, c.s, pi, vi, P.vel_c);
+        D = drho_dt_lane<kBatch, T>(P, sc, i, c.s, pi, vi, P.vel_c, P.nnf[i], T > 1 ? P.nnb[i] : -1);
     }
     D = group_sum<T>(D);
     const bool own = c.valid && c.s == 0;
@@ -954,7 +984,7 @@ __global__ void __launch_bounds__(kBlock) k_warm_density(Ptrs P)
             if (lane == lead) base = atomicAdd(&P.ctl->mlp_n, __popc(m));
             base = __shfl_sync(0xffffffffu, base, lead);
         }
-        if (gated) P.mlp_rows[base + __popc(m & ((1u << lane) - 1u))] = make_int2((int)i, P.tblk_scene[blockIdx.x]);
+        if (gated) P.mlp_rows[base + __popc(m & ((1u << lane) - 1u))] = make_int2((int)i, scene_of_block(P, P.tblk_scene, (int32_t)blockIdx.x));
     }
     if (!own) return;
     // the network's inputs are recorded in both warm-start modes (the previous-step mode

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(kBlock) k_key_hist(Ptrs P)
 {
     kernel_enter(P.ctl, (WHAT == SORT_FLUID ? KID_KEY_HIST_F : KID_KEY_HIST_B));
     const int32_t *tab = WHAT == SORT_FLUID ? P.fblk_scene : P.bblk_scene;
-    const SceneDev &sc = P.scenes[tab[blockIdx.x]];
+    const SceneDev &sc = P.scenes[scene_of_block(P, tab, (int32_t)blockIdx.x)];
     const int32_t first = WHAT == SORT_FLUID ? sc.fblk_first : sc.bblk_first;
     const int64_t off = WHAT == SORT_FLUID ? sc.f_off : sc.b_off;
     const int64_t n = WHAT == SORT_FLUID ? sc.nf : sc.nb;
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kBlock) k_scatter(Ptrs P)
 {
     kernel_enter(P.ctl, (WHAT == SORT_FLUID ? KID_SCATTER_F : KID_SCATTER_B));
     const int32_t *tab = WHAT == SORT_FLUID ? P.fblk_scene : P.bblk_scene;
-    const SceneDev &sc = P.scenes[tab[blockIdx.x]];
+    const SceneDev &sc = P.scenes[scene_of_block(P, tab, (int32_t)blockIdx.x)];
     const int32_t first = WHAT == SORT_FLUID ? sc.fblk_first : sc.bblk_first;
     const int64_t off = WHAT == SORT_FLUID ? sc.f_off : sc.b_off;
     const int64_t n = WHAT == SORT_FLUID ? sc.nf : sc.nb;
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kBlock) k_rank_gather(Ptrs P)
 {
     kernel_enter(P.ctl, (WHAT == SORT_FLUID ? KID_RANK_F : KID_RANK_B));
     const int32_t *tab = WHAT == SORT_FLUID ? P.fblk_scene : P.bblk_scene;
-    const SceneDev &sc = P.scenes[tab[blockIdx.x]];
+    const SceneDev &sc = P.scenes[scene_of_block(P, tab, (int32_t)blockIdx.x)];
     const int32_t first = WHAT == SORT_FLUID ? sc.fblk_first : sc.bblk_first;
     const int64_t off = WHAT == SORT_FLUID ? sc.f_off : sc.b_off;
     const int64_t n = WHAT == SORT_FLUID ? sc.nf : sc.nb;

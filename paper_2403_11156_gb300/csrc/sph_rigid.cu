@@ -19,7 +19,7 @@ namespace {
 __global__ void __launch_bounds__(kBlock) k_boundary_update(Ptrs P)
 {
     kernel_enter(P.ctl, KID_BUPDATE);
-    const SceneDev &sc = P.scenes[P.bblk_scene[blockIdx.x]];
+    const SceneDev &sc = P.scenes[scene_of_block(P, P.bblk_scene, (int32_t)blockIdx.x)];
     if (!sc.has_moving) return;
     int64_t local = (int64_t)(blockIdx.x - sc.bblk_first) * kBlock + threadIdx.x;
     if (local >= sc.nb) return;
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(kBlock) k_boundary_update(Ptrs P)
 __global__ void __launch_bounds__(kBlock) k_boundary_psi(Ptrs P)
 {
     kernel_enter(P.ctl, KID_PSI);
-    const SceneDev &sc = P.scenes[P.bblk_scene[blockIdx.x]];
+    const SceneDev &sc = P.scenes[scene_of_block(P, P.bblk_scene, (int32_t)blockIdx.x)];
     int64_t local = (int64_t)(blockIdx.x - sc.bblk_first) * kBlock + threadIdx.x;
     if (local >= sc.nb) return;
     int64_t b = sc.b_off + local;

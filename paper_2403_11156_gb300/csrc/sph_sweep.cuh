@@ -56,7 +56,7 @@ template <int T>
 __device__ __forceinline__ Lane<T> lane_ctx(const Ptrs &P, int32_t block)
 {
     Lane<T> c;
-    const int32_t sidx = P.tblk_scene[block];
+    const int32_t sidx = scene_of_block(P, P.tblk_scene, block);
     c.sc = &P.scenes[sidx];
     c.st = &P.st[sidx];
     const int64_t local = (int64_t)(block - c.sc->tblk_first) * (kBlock / T) + threadIdx.x / T;

@@ -27,7 +27,7 @@ struct Ctx {
 __device__ __forceinline__ Ctx ctx(const Ptrs &P)
 {
     Ctx c;
-    int32_t s = P.fblk_scene[blockIdx.x];
+    int32_t s = scene_of_block(P, P.fblk_scene, (int32_t)blockIdx.x);
     c.sc = &P.scenes[s];
     c.st = &P.st[s];
     int64_t local = (int64_t)(blockIdx.x - c.sc->fblk_first) * kBlock + threadIdx.x;
