@@ -233,7 +233,9 @@ __global__ void __launch_bounds__(32 * kTileWarps, 8)
                     // distance to the box: no larger than to any node, operation by operation
                     const float dx = fmaxf(fmaxf(lox - p.x, p.x - hix), 0.0f), dy = fmaxf(fmaxf(loy - p.y, p.y - hiy), 0.0f),
                                 dz = fmaxf(fmaxf(loz - p.z, p.z - hiz), 0.0f);
-                    keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < h2;
+                    // (a NaN coordinate, which the maxima here and in add() pass over, is near no node)
+                    const float any = p.x + p.y + p.z;
+                    keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < h2 && any == any;
                 }
                 const unsigned kept = __ballot_sync(0xffffffffu, keep);
                 if (keep) buf[cnt + __popc(kept & ((1u << lane) - 1u))] = p;
