@@ -85,7 +85,9 @@ __device__ __forceinline__ f2 gelu_pair(float h0, float h1)
 __device__ __forceinline__ uint32_t tie_key(uint32_t m, float a, float b)
 {
     uint32_t x = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x5410);
-    x += 0x80108010u;   // (a carry moves the second by one)
+    // without a carry between the halves: what is found here has to be all that at_tie replaces,
+    // or a row's output would depend on the rows beside it
+    asm("add.u16x2 %0, %0, %1;" : "+r"(x) : "r"(0x80108010u));
     asm("min.u16x2 %0, %0, %1;" : "+r"(m) : "r"(x));
     return m;
 }
