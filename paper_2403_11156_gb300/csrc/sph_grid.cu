@@ -166,13 +166,14 @@ __device__ __forceinline__ void st_release(uint64_t *p, uint64_t v)
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t *count, uint32_t *start, int64_t n,
-                                                       uint64_t *status, int32_t tiles, ScanCtl *sc, Control *ctl)
+                                                       uint64_t *status, int32_t tiles, ScanCtl *sc, Control *ctl,
+                                                       bool of_step)
 {
     __shared__ int32_t s_tile;
     __shared__ uint32_t s_epoch;
     __shared__ uint32_t s_warp[kScanThreads / 32];
     __shared__ uint32_t s_prefix;
-    kernel_enter(ctl, KID_SCAN);
+    if (of_step) kernel_enter(ctl, KID_SCAN);   // counted and traced
     if (threadIdx.x == 0) {
         s_tile = atomicAdd(&sc->tile_counter, 1);
         s_epoch = *reinterpret_cast<volatile uint32_t *>(&sc->epoch);
@@ -296,10 +297,10 @@ int32_t scan_tiles_for(int64_t n) { return (int32_t)((n + kScanTile - 1) / kScan
 int64_t large_capacity(int64_t n) { return n / (kRankSmall + 1) + 1; }
 
 void launch_scan(uint32_t *count, uint32_t *start, int64_t n, uint64_t *status, int32_t tiles,
-                 ScanCtl *sc, Control *ctl, cudaStream_t s)
+                 ScanCtl *sc, Control *ctl, bool of_step, cudaStream_t s)
 {
     if (n <= 0 || tiles <= 0) return;
-    k_scan<<<tiles, kScanThreads, 0, s>>>(count, start, n, status, tiles, sc, ctl);
+    k_scan<<<tiles, kScanThreads, 0, s>>>(count, start, n, status, tiles, sc, ctl, of_step);
 }
 
 void launch_key_hist(const Ptrs &P, SortWhat what, cudaStream_t s)
@@ -315,10 +316,10 @@ void launch_scan_cells(const Ptrs &P, SortWhat what, cudaStream_t s)
     if (what == SORT_FLUID) {
         if (P.nfblk)
             launch_scan(P.cell_count, P.cell_start, P.NC, P.scan_status, scan_tiles_for(P.NC), &P.ctl->scan[0],
-                        P.ctl, s);
+                        P.ctl, true, s);
     } else if (P.nbblk) {
         launch_scan(P.bcell_count, P.bcell_start, P.NC, P.bscan_status, scan_tiles_for(P.NC), &P.ctl->scan[1],
-                    P.ctl, s);
+                    P.ctl, true, s);
     }
 }
 void launch_scatter(const Ptrs &P, SortWhat what, cudaStream_t s)

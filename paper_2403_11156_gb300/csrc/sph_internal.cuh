@@ -375,8 +375,9 @@ void launch_key_hist(const Ptrs &P, SortWhat what, cudaStream_t s);
 void launch_scan_cells(const Ptrs &P, SortWhat what, cudaStream_t s);
 void launch_scatter(const Ptrs &P, SortWhat what, cudaStream_t s);
 void launch_rank_gather(const Ptrs &P, SortWhat what, cudaStream_t s);
+// of_step: the launch counts (and is traced) as one of the step's
 void launch_scan(uint32_t *count, uint32_t *start, int64_t n, uint64_t *status, int32_t tiles,
-                 ScanCtl *sc, Control *ctl, cudaStream_t s);
+                 ScanCtl *sc, Control *ctl, bool of_step, cudaStream_t s);
 int32_t scan_tiles_for(int64_t n);
 
 // In-cell ranking: a cell of at most kRankSmall particles ranks each one by counting the

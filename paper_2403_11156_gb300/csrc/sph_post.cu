@@ -605,7 +605,7 @@ cudaError_t post_surface_field(const Ptrs &P, const SceneDev &sc, int64_t nbr_en
     }
     if (e == cudaSuccess) {
         k_pf_hist<<<blocks_for(n), kPostBlock, 0, s>>>(pos, n, sc, count, key, slot);
-        launch_scan(count, start, ncell, P.scan_status, scan_tiles_for(ncell), &P.ctl->scan[0], P.ctl, s);
+        launch_scan(count, start, ncell, P.scan_status, scan_tiles_for(ncell), &P.ctl->scan[0], P.ctl, false, s);
         k_pf_place<<<blocks_for(n), kPostBlock, 0, s>>>(n, key, slot, start, cellidx);
         k_pf_rank<<<blocks_for(n), kPostBlock, 0, s>>>(pos, vel, n, sc.m, sc.rho0, key, start, cellidx, sorted);
         const int64_t nodes = (int64_t)dims[0] * dims[1] * dims[2];
