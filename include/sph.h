@@ -442,7 +442,9 @@ sph_status sph_launch_count(sph_ctx *ctx, int64_t *out);
  * comes from counting each point's smaller indices; a more crowded cell is sorted by one
  * thread block (a stable radix sort on the index), so the work stays linear in n however
  * the points crowd into cells.
- * SPH_OK means the work was enqueued; whether its prefix scan completed is reported by
+ * Beyond 8,192 points (or 24,576 cells) the call is one cooperative launch of at most one block
+ * per SM: it starts once all its blocks have room beside what runs on other streams.
+ * SPH_OK means the work was enqueued; whether it completed is reported by
  * sph_grid_order_noalloc_status. */
 #define SPH_NOALLOC_MAX_POINTS 262144
 #define SPH_NOALLOC_MAX_CELLS 1048576
@@ -454,7 +456,7 @@ sph_status sph_grid_order_noalloc(const float *x, int64_t n, const float *domain
  * stream (the one that call used), then reads the scratch array's error word into host
  * memory with a copy from the symbol (no allocation).  SPH_ETIMEOUT: a bounded wait of the
  * call ran out, or a call that overlapped disturbed its histogram, so its order is not
- * valid (the GPU stays usable);
+ * valid (the GPU stays usable, and later calls, replays of captured ones too, are not affected);
  * SPH_OK: it completed; SPH_ECUDA: the synchronisation or the copy failed.  The word is
  * cleared by every call, so a later or overlapping call replaces it.  Not for use inside a
  * stream capture (it synchronises). */

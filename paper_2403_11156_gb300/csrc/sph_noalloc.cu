@@ -15,7 +15,6 @@
 #include "sph_sweep.cuh"
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <mutex>
@@ -27,9 +26,6 @@ namespace {
 constexpr int64_t kMaxPoints = SPH_NOALLOC_MAX_POINTS;
 constexpr int64_t kMaxCells = SPH_NOALLOC_MAX_CELLS;
 constexpr int kOrderBlocks = 152;   // at most one block per SM
-// barriers, a call after the other in turn: calls that overlap (which race on the rest of the
-// scratch) do not meet in one, and each call clears the barrier of the fourth after it
-constexpr int kBarSlots = 8;
 
 // Byte offsets of the scratch regions (each a multiple of 256).
 constexpr size_t kOffCount = 0;                                          // u32 [kMaxCells]
@@ -39,7 +35,7 @@ constexpr size_t kOffSlot = kOffKey + 4 * kMaxPoints;                    // u32 
 constexpr size_t kOffSid = kOffSlot + 4 * kMaxPoints;                    // u32 [kMaxPoints]
 constexpr size_t kOffCell = kOffSid + 4 * kMaxPoints;                    // u32 [kMaxPoints]
 constexpr size_t kOffSums = kOffCell + 4 * kMaxPoints;                    // u32 [kOrderBlocks]
-constexpr size_t kOffBar = kOffSums + ((4 * kOrderBlocks + 255) / 256) * 256;  // GridBar [kBarSlots]
+constexpr size_t kOffBar = kOffSums + ((4 * kOrderBlocks + 255) / 256) * 256;  // u64, see OrderBarrier
 constexpr size_t kOffCtl = kOffBar + 256;                                // Control
 constexpr int64_t kMaxLarge = kMaxPoints / (kRankSmall + 1) + 1;
 constexpr size_t kOffLarge = kOffCtl + ((sizeof(Control) + 255) / 256) * 256;  // u32 [kMaxLarge]
@@ -50,7 +46,7 @@ static __device__ __align__(256) unsigned char g_grid_scratch[kScratchBytes];
 struct View {
     uint32_t *count, *start, *key, *slot, *sid, *cell;
     uint32_t *sums;
-    GridBar *bar;
+    uint64_t *bar;
     Control *ctl;
     uint32_t *large;
 };
@@ -65,7 +61,7 @@ View carve(unsigned char *base)
     v.sid = reinterpret_cast<uint32_t *>(base + kOffSid);
     v.cell = reinterpret_cast<uint32_t *>(base + kOffCell);
     v.sums = reinterpret_cast<uint32_t *>(base + kOffSums);
-    v.bar = reinterpret_cast<GridBar *>(base + kOffBar);
+    v.bar = reinterpret_cast<uint64_t *>(base + kOffBar);
     v.ctl = reinterpret_cast<Control *>(base + kOffCtl);
     v.large = reinterpret_cast<uint32_t *>(base + kOffLarge);
     return v;
@@ -118,54 +114,103 @@ __device__ void sort_cell(const View &v, uint32_t b, uint32_t e, int32_t *order)
     __syncthreads();
 }
 
+// The barrier over the blocks of a call, on a word that no call resets: a captured call is replayed
+// with the arguments of its capture and cannot be given a fresh one, and a memset before the
+// launch takes 4 us.  High half: arrivals.  A barrier's sum to kArrivals whatever
+// the grid (block 0 makes up the difference), so that every block knows from the value it met
+// which barrier it is in.  Low half: blocks that gave up a bounded wait; a change since a block's
+// start ends its waits (the blocks of a cooperative launch start together).
+// A block of any call leaves exactly kBarriers barriers' arrivals behind (those that it did not
+// come to are added as it leaves), so the word is whole again after calls that gave up or overlapped.
+struct OrderBarrier {
+    static constexpr uint32_t kArrivals = 1u << 16;
+    static constexpr int kBarriers = 7;   // the most that a call meets
+    uint64_t *word;
+    int32_t *error;
+    uint32_t fails;
+    int left = kBarriers;
+    __device__ OrderBarrier(uint64_t *w, int32_t *e) : word(w), error(e), fails((uint32_t)*reinterpret_cast<volatile uint64_t *>(w)) {}
+    __device__ static uint64_t share() { return blockIdx.x == 0 ? kArrivals - (gridDim.x - 1u) : 1u; }
+    __device__ void leave(bool gave_up)
+    {
+        if (threadIdx.x == 0 && left > 0) atomicAdd(reinterpret_cast<unsigned long long *>(word), (unsigned long long)((share() * left << 32) + (gave_up ? 1u : 0u)));
+        left = 0;
+    }
+    // Whether all blocks came; if not, the block has left.
+    __device__ bool wait()
+    {
+        bool ok = true;
+        __syncthreads();
+        --left;
+        if (threadIdx.x == 0) {
+            const uint64_t add = share() << 32;
+            uint64_t met;
+            asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(met) : "l"(word), "l"(add) : "memory");
+            const uint32_t base = (uint32_t)(met >> 32) & ~(kArrivals - 1u);
+            auto open = [&](uint64_t w) { return (uint32_t)(w >> 32) - base >= kArrivals; };
+            auto whole = [&](uint64_t w) { return (uint32_t)w == fails; };
+            uint64_t now = met + add;
+            for (uint32_t spins = 0; !open(now) && whole(now) && spins < kBarrierSpins; ++spins)
+                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(word) : "memory");
+            ok = open(now) && whole(now);
+            if (!ok) atomicExch(error, 5);
+        }
+        ok = __syncthreads_and(ok);
+        if (!ok) leave(true);
+        return ok;
+    }
+};
+
 // The whole order in one cooperative launch: keys and histogram, prefix sum (each block sums its
 // share of the cells, then adds the shares before it), scatter, rank inside the cell by index or,
 // for the crowded cells, which the prefix sum queues, block sort; four barriers.  The histogram
-// is zero between calls: the prefix sum clears what it has read, and its total has to be n.  As six launches it was bound
-// by them: 262,143 points 39.0 -> 24.6 us.
+// is zero between calls: the prefix sum clears what it has read.  Its total has to be n; where an
+// earlier call left something in it, it is cleared and filled once more.  As six launches it was
+// bound by them: 262,143 points 39.0 -> 21.9 us (24.6 with count and generation in two words,
+// 28.7 with a memset that cleared both and the histogram before every call).
 __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, const float *__restrict__ x, int64_t n,
-                                                            int64_t ncell, uint32_t *keys_out, int32_t *order, int slot)
+                                                            int64_t ncell, uint32_t *keys_out, int32_t *order)
 {
     Control *ctl = v.ctl;
-    GridBar *bar = &v.bar[slot];
-    uint32_t phase = *reinterpret_cast<volatile uint32_t *>(&bar->gen);
+    OrderBarrier bar(v.bar, &ctl->error);
     const int64_t first = (int64_t)blockIdx.x * kLargeThreads + threadIdx.x, stride = (int64_t)gridDim.x * kLargeThreads;
     if (first == 0) {
         ctl->error = 0;   // (no block can have given up yet)
         ctl->nlarge[0] = 0;
-        v.bar[(slot + kBarSlots / 2) % kBarSlots] = GridBar{0u, 0u};
     }
-    for (int64_t i = first; i < n; i += stride) {
-        const uint32_t key = key_of(g, x, i);
-        v.key[i] = key;
-        v.slot[i] = atomicAdd(&v.count[key], 1u);
-        if (keys_out) keys_out[i] = key;
-    }
-    if (!grid_barrier(bar, &ctl->error, phase)) return;
     // cells [c0, c1) are this block's share, a multiple of the block's width
     const int64_t share = ((ncell + gridDim.x - 1) / gridDim.x + kLargeThreads - 1) / kLargeThreads * kLargeThreads;
     const int64_t c0 = (int64_t)blockIdx.x * share, c1 = min(c0 + share, ncell);
-    uint32_t total = 0u;
-    {
+    __shared__ uint32_t s_run;
+    uint32_t total;
+    for (int attempt = 0;; ++attempt) {
+        for (int64_t i = first; i < n; i += stride) {
+            const uint32_t key = key_of(g, x, i);
+            v.key[i] = key;
+            v.slot[i] = atomicAdd(&v.count[key], 1u);
+            if (keys_out) keys_out[i] = key;
+        }
+        if (!bar.wait()) return;
         uint32_t sum = 0u;
         for (int64_t c = c0 + threadIdx.x; c < c1; c += kLargeThreads) sum += v.count[c];
         block_scan(sum, total);
         if (threadIdx.x == 0) v.sums[blockIdx.x] = total;
-    }
-    if (!grid_barrier(bar, &ctl->error, phase)) return;
-    {
-        __shared__ uint32_t s_run;
+        if (!bar.wait()) return;
         const uint32_t before_me = block_scan(threadIdx.x < gridDim.x ? v.sums[threadIdx.x] : 0u, total);
         if (threadIdx.x == blockIdx.x) s_run = before_me;   // shares before this one
-        __syncthreads();
-        uint32_t run = s_run;
-        if (total != (uint32_t)n) {
-            // the histogram was not this call's alone (a call that overlapped, now or earlier):
-            // clear it for the next one and say so instead of scattering by it (every block alike)
-            for (int64_t c = c0 + threadIdx.x; c < c1; c += kLargeThreads) v.count[c] = 0u;
+        if (total == (uint32_t)n) break;
+        // the histogram was not this call's alone (every block alike)
+        for (int64_t c = c0 + threadIdx.x; c < c1; c += kLargeThreads) v.count[c] = 0u;
+        if (attempt > 0) {   // not a leftover: another call writes it now
             if (threadIdx.x == 0) atomicExch(&ctl->error, 7);
+            bar.leave(false);
             return;
         }
+        if (!bar.wait()) return;
+    }
+    {
+        __syncthreads();
+        uint32_t run = s_run;
         for (int64_t c = c0; c < c1; c += kLargeThreads) {
             const int64_t at = c + threadIdx.x;
             const uint32_t k = at < c1 ? v.count[at] : 0u;
@@ -179,13 +224,13 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
         }
         if (c1 == ncell && c0 < c1 && threadIdx.x == 0) v.start[ncell] = run;
     }
-    if (!grid_barrier(bar, &ctl->error, phase)) return;
+    if (!bar.wait()) return;
     for (int64_t i = first; i < n; i += stride) {
         const uint32_t key = v.key[i], s = v.start[key] + v.slot[i];
         v.sid[s] = (uint32_t)i;
         v.cell[s] = key;
     }
-    if (!grid_barrier(bar, &ctl->error, phase)) return;
+    if (!bar.wait()) return;
     for (int64_t s = first; s < n; s += stride) {
         const uint32_t c = v.cell[s], b = v.start[c], e = v.start[c + 1];
         if (e - b > kRankSmall) continue;   // queued
@@ -201,6 +246,7 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
         const uint32_t c = v.large[q];
         sort_cell(v, v.start[c], v.start[c + 1], order);
     }
+    bar.leave(false);
 }
 
 // Few points in few cells: the same in one block, histogram, starts and order in shared memory.
@@ -327,9 +373,7 @@ extern "C" sph_status sph_grid_order_noalloc(const float *x, int64_t n, const fl
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) return SPH_ECUDA;
     const int64_t want = (std::max(n, ncell) + kLargeThreads - 1) / kLargeThreads;
     const int blocks = (int)std::min<int64_t>(want, std::min(nsm, kOrderBlocks));
-    static std::atomic<unsigned> calls{0};
-    int slot = (int)(calls.fetch_add(1u, std::memory_order_relaxed) % (unsigned)kBarSlots);
-    void *args[] = {&v, &g, (void *)&x, &n, &ncell, &keys, &order, &slot};
+    void *args[] = {&v, &g, (void *)&x, &n, &ncell, &keys, &order};
     const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_na_order), dim3((unsigned)blocks),
                                                       dim3(kLargeThreads), args, 0, s);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
@@ -337,9 +381,9 @@ extern "C" sph_status sph_grid_order_noalloc(const float *x, int64_t n, const fl
 
 extern "C" sph_status sph_grid_order_noalloc_status(void *stream)
 {
-    // the scan's bounded waits record a timeout in the scratch's control word, which each
-    // call clears before its scan: read it back once the stream's work is done (a copy
-    // from the symbol into a host integer, nothing allocated)
+    // a call that found its histogram disturbed or gave up a bounded wait records it in the
+    // scratch's error word, which each call clears: read it back once the stream's work is done
+    // (a copy from the symbol into a host integer, nothing allocated)
     if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return SPH_ECUDA;
     int32_t err = 0;
     const size_t off = kOffCtl + offsetof(Control, error);
