@@ -105,12 +105,12 @@ __device__ __forceinline__ uint32_t key_of(const Grid &g, const float *__restric
     return (uint32_t)ix + (uint32_t)g.dims[0] * ((uint32_t)iy + (uint32_t)g.dims[1] * (uint32_t)iz);
 }
 
-// Put the indices v.sid[b..e) of a crowded cell in order and write them out, by the whole block.
-__device__ void sort_cell(const View &v, uint32_t b, uint32_t e, int32_t *order)
+// Put the indices sid[b..e) of a crowded cell in order and write them out, by the whole block, with
+// other[b..e) for the passes (sorted by index alone: an index is its own value).
+__device__ void sort_cell(uint32_t *sid, uint32_t *other, uint32_t b, uint32_t e, int32_t *order)
 {
-    // (sorted by index alone: the second of the pair, in the result's place, is not used)
-    block_sort_segment(v.sid, reinterpret_cast<uint32_t *>(order), v.key, v.slot, b, e);
-    for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) order[d] = (int32_t)v.sid[d];
+    block_sort_segment(sid, sid, other, other, b, e);
+    for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) order[d] = (int32_t)sid[d];
     __syncthreads();
 }
 
@@ -165,8 +165,9 @@ struct OrderBarrier {
 // share of the cells, then adds the shares before it), scatter, rank inside the cell by index or,
 // for the crowded cells, which the prefix sum queues, block sort; four barriers.  The histogram
 // is zero between calls: the prefix sum clears what it has read.  Its total has to be n; where an
-// earlier call left something in it, it is cleared and filled once more.  As six launches it was
-// bound by them: 262,143 points 39.0 -> 21.9 us (24.6 with count and generation in two words,
+// earlier call left something in it, it is cleared and filled once more.
+// Calls that overlap race on the scratch: what is read from it is checked (places below n, the
+// queue's length) before it is used as an index.  As six launches it was bound by them: 262,143 points 39.0 -> 22.1 us (24.6 with count and generation in two words,
 // 28.7 with a memset that cleared both and the histogram before every call).
 __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, const float *__restrict__ x, int64_t n,
                                                             int64_t ncell, uint32_t *keys_out, int32_t *order)
@@ -218,7 +219,10 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
             if (at < c1) {
                 v.start[at] = run + before;
                 v.count[at] = 0u;
-                if (k > kRankSmall) v.large[atomicAdd(&ctl->nlarge[0], 1)] = (uint32_t)at;
+                if (k > kRankSmall) {
+                    const int q = atomicAdd(&ctl->nlarge[0], 1);
+                    if (q < kMaxLarge) v.large[q] = (uint32_t)at;
+                }
             }
             run += total;
         }
@@ -227,24 +231,31 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
     if (!bar.wait()) return;
     for (int64_t i = first; i < n; i += stride) {
         const uint32_t key = v.key[i], s = v.start[key] + v.slot[i];
+        if (s >= (uint32_t)n) continue;
         v.sid[s] = (uint32_t)i;
         v.cell[s] = key;
     }
     if (!bar.wait()) return;
     for (int64_t s = first; s < n; s += stride) {
-        const uint32_t c = v.cell[s], b = v.start[c], e = v.start[c + 1];
+        const uint32_t c = v.cell[s], b = v.start[c], e = min(v.start[c + 1], (uint32_t)n);
         if (e - b > kRankSmall) continue;   // queued
         const uint32_t my = v.sid[s];
         uint32_t rank = 0;
         for (uint32_t t = b; t < e; ++t) rank += (v.sid[t] < my) ? 1u : 0u;
-        order[b + rank] = (int32_t)my;
+        if (b + rank < e) order[b + rank] = (int32_t)my;
     }
     // the queued cells: one block per cell at a time sorts the cell's indices stably and writes
-    // them out (the key and slot regions, free once scattered, are its scratch).
-    const int nq = *reinterpret_cast<volatile int32_t *>(&ctl->nlarge[0]);
+    // them out (the slot region, free once scattered, is its scratch).
+    __shared__ uint32_t s_seg[2];
+    const int nq = min(*reinterpret_cast<volatile int32_t *>(&ctl->nlarge[0]), (int)kMaxLarge);
     for (int q = blockIdx.x; q < nq; q += gridDim.x) {
-        const uint32_t c = v.large[q];
-        sort_cell(v, v.start[c], v.start[c + 1], order);
+        if (threadIdx.x == 0) {
+            const uint32_t c = v.large[q];
+            s_seg[0] = v.start[c];
+            s_seg[1] = min(v.start[c + 1], (uint32_t)n);
+        }
+        __syncthreads();
+        sort_cell(v.sid, v.slot, s_seg[0], s_seg[1], order);
     }
     bar.leave(false);
 }
@@ -253,18 +264,19 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
 // 3,001 points in 10,648 cells: 28.7 us as six launches, 8.2 us here (a barrier over blocks
 // costs more than this range's work).
 constexpr int64_t kOneBlockPoints = 8 * kLargeThreads, kOneBlockCells = 24 * kLargeThreads;
-__global__ void __launch_bounds__(kLargeThreads) k_na_order_one(View v, Grid g, const float *__restrict__ x, int n, int ncell,
+__global__ void __launch_bounds__(kLargeThreads) k_na_order_one(Control *ctl, Grid g, const float *__restrict__ x, int n, int ncell,
                                                                 uint32_t *keys_out, int32_t *order)
 {
     extern __shared__ uint32_t sm[];
-    uint32_t *start = sm, *sid = sm + ncell + 1;
+    uint32_t *start = sm, *sid = sm + ncell + 1, *other = sid + n;
     __shared__ int s_large;
+    __shared__ uint32_t s_cells[kOneBlockPoints / (kRankSmall + 1)];   // the crowded ones
     constexpr int kOwn = (int)(kOneBlockPoints / kLargeThreads);
     const int t = threadIdx.x;
     for (int c = t; c < ncell; c += kLargeThreads) start[c] = 0u;
     if (t == 0) {
         s_large = 0;
-        v.ctl->error = 0;
+        ctl->error = 0;
     }
     __syncthreads();
     uint32_t key[kOwn], at[kOwn];
@@ -303,7 +315,7 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order_one(View v, Grid g, 
         if (i >= n) continue;
         const uint32_t b = start[key[k]], e = start[key[k] + 1];
         if (e - b > kRankSmall) {
-            if (at[k] == 0u) v.large[atomicAdd(&s_large, 1)] = key[k];
+            if (at[k] == 0u) s_cells[atomicAdd(&s_large, 1)] = key[k];
             continue;
         }
         uint32_t rank = 0;
@@ -312,10 +324,8 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order_one(View v, Grid g, 
     }
     __syncthreads();
     for (int q = 0; q < s_large; ++q) {
-        const uint32_t c = v.large[q], b = start[c], e = start[c + 1];
-        for (uint32_t d = b + (uint32_t)t; d < e; d += kLargeThreads) v.sid[d] = sid[d];
-        __syncthreads();
-        sort_cell(v, b, e, order);
+        const uint32_t c = s_cells[q];
+        sort_cell(sid, other, start[c], start[c + 1], order);
     }
 }
 
@@ -361,11 +371,11 @@ extern "C" sph_status sph_grid_order_noalloc(const float *x, int64_t n, const fl
     View v = carve(base);
     cudaStream_t s = (cudaStream_t)stream;
     if (n <= kOneBlockPoints && ncell <= kOneBlockCells && n <= kRankSmall / 2 * ncell) {   // (no crowd of crowded cells)
-        const size_t bytes = sizeof(uint32_t) * (size_t)(ncell + 1 + n);
+        const size_t bytes = sizeof(uint32_t) * (size_t)(ncell + 1 + 2 * n);
         if (cudaFuncSetAttribute(k_na_order_one, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(uint32_t) * (kOneBlockCells + 1 + kOneBlockPoints))) != cudaSuccess)
+                                 (int)(sizeof(uint32_t) * (kOneBlockCells + 1 + 2 * kOneBlockPoints))) != cudaSuccess)
             return SPH_ECUDA;
-        k_na_order_one<<<1, kLargeThreads, bytes, s>>>(v, g, x, (int)n, (int)ncell, keys, order);
+        k_na_order_one<<<1, kLargeThreads, bytes, s>>>(v.ctl, g, x, (int)n, (int)ncell, keys, order);
         return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
     }
     // a block of 1024 threads per 1024 points or cells, at most one per SM

@@ -42,6 +42,16 @@ extern "C" int run_late(uint64_t *word, int32_t *error, int32_t *ok, int blocks,
     void *args[] = {&word, &error, &ok, &late};
     return (int)cudaLaunchCooperativeKernel((const void *)k_late, dim3(blocks), dim3(64), args, 0, 0);
 }
+// The one-block kernel on control words of the caller's: it needs nothing else that calls share.
+extern "C" int run_one(void *ctl, const float *x, int n, int side, float cell, int32_t *order)
+{
+    Grid g{{-cell, -cell, -cell}, cell, {side, side, side}};
+    const int ncell = side * side * side;
+    const size_t bytes = sizeof(uint32_t) * (size_t)(ncell + 1 + 2 * n);
+    if (cudaFuncSetAttribute(k_na_order_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return 1;
+    k_na_order_one<<<1, kLargeThreads, bytes>>>((Control *)ctl, g, x, n, ncell, nullptr, order);
+    return cudaDeviceSynchronize() != cudaSuccess;
+}
 """
 
 
@@ -55,6 +65,7 @@ def lib(tmp_path_factory):
     L.sph_grid_order_noalloc.argtypes = sph.load().sph_grid_order_noalloc.argtypes
     L.sph_grid_order_noalloc_status.argtypes = [ctypes.c_void_p]
     L.fill_scratch.argtypes = [ctypes.c_int, ctypes.c_uint64]
+    L.run_one.argtypes = [ctypes.c_void_p] * 2 + [ctypes.c_int] * 2 + [ctypes.c_float] + [ctypes.c_void_p]
     L.run_late.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int] * 2
     return L
 
@@ -115,3 +126,23 @@ def test_late_block(lib, blocks, late):
         assert int(error.item()) == (0 if late < 0 else 5)
         gave_up = blocks if late >= 0 else 0
         assert int(word.item()) % (1 << 64) == (start + (7 << 48) + gave_up) % (1 << 64)
+
+
+@pytest.mark.parametrize("n,crowds", [(1, 0), (2000, 1), (8192, 126)])
+def test_one_block_shares_nothing(lib, n, crowds):
+    import torch
+    rng = np.random.default_rng(n)
+    side, cell = 28, np.float32(0.04)
+    extent = float(cell) * (side - 2)
+    pts = rng.uniform(0, extent, (n, 3)).astype(np.float32)
+    for k in range(crowds):          # 65 points each, beyond what a cell ranks by counting
+        pts[65 * k:65 * (k + 1)] = rng.uniform(0, extent, 3)
+    pts = pts[rng.permutation(n)]
+    ctl = torch.zeros(512, dtype=torch.uint8, device="cuda")
+    guard = torch.full((n + 64,), -7, dtype=torch.int32, device="cuda")
+    x = torch.from_numpy(pts).cuda()
+    torch.cuda.synchronize()
+    assert lib.run_one(ctl.data_ptr(), x.data_ptr(), n, side, cell, guard.data_ptr()) == 0
+    lo, hi = np.zeros(3, np.float32), np.full(3, extent, np.float32)
+    np.testing.assert_array_equal(guard[:n].cpu().numpy(), oracle.sort_order(oracle.cell_keys(pts, lo, hi, cell)))
+    assert bool((guard[n:] == -7).all())
