@@ -858,10 +858,12 @@ __global__ void __launch_bounds__(kBlock, kSolveBlocksPerSm) k_solve(const __gri
     __shared__ int s_any;
     kernel_enter(P.ctl, KID_SOLVE0 + S);
     uint32_t phase = *reinterpret_cast<volatile uint32_t *>(&P.ctl->bar.gen);
+    // after a wait that gave up the state is lost: the steps still queued must not wait in vain too
+    // (looked at after the first pass A, beside which the load takes no time)
     for (;;) {
-        for (int32_t b = (int32_t)blockIdx.x; b < P.ntblk; b += (int32_t)gridDim.x) pass_a<S, kBatch, T, false>(P, b, sh);
+        pass_a<S, kBatch, T, false>(P, (int32_t)blockIdx.x, sh);
         if (!grid_barrier(&P.ctl->bar, &P.ctl->error, phase)) return;
-        for (int32_t b = (int32_t)blockIdx.x; b < P.ntblk; b += (int32_t)gridDim.x) pass_b<S, 0, kBatch, T, false>(P, b);
+        pass_b<S, 0, kBatch, T, false>(P, (int32_t)blockIdx.x);
         if (!grid_barrier(&P.ctl->bar, &P.ctl->error, phase, [&] { solver_check<S>(P, &s_any); })) return;
         if (*reinterpret_cast<volatile uint32_t *>(&P.ctl->loop_flag) == 0u) return;
     }
@@ -1216,8 +1218,7 @@ int solve_grid(const Ptrs &P, int batch)
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, solve_kernel(P, solver), kBlock, 0) != cudaSuccess) return 0;
         resident = solver == 0 ? per * nsm : std::min(resident, per * nsm);
     }
-    if (resident < 1 || P.ntblk > resident) return 0;
-    return std::min(P.ntblk, resident);
+    return P.ntblk <= resident ? P.ntblk : 0;
 }
 cudaError_t launch_solve(const Ptrs &P, int solver, int grid, cudaStream_t s)
 {

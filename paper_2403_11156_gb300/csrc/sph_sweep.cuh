@@ -195,22 +195,6 @@ __device__ __forceinline__ void for_list(const int32_t *__restrict__ list, int64
         if (k + u < m) visit(j[u]);
 }
 
-// Visit the candidates j0, j0 + T, ... below je of a grid row in batches of U: the U
-// position loads of a batch are issued before any visit, in index order.
-template <int U, int T, typename F>
-__device__ __forceinline__ void for_range(const float4 *__restrict__ pos, uint32_t j0, uint32_t je, F &&visit)
-{
-    uint32_t j = j0;
-    for (; j + (uint32_t)((U - 1) * T) < je; j += (uint32_t)(U * T)) {
-        float4 p[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) p[u] = __ldg(pos + j + u * T);
-#pragma unroll
-        for (int u = 0; u < U; ++u) visit(j + (uint32_t)(u * T), p[u]);
-    }
-    for (; j < je; j += (uint32_t)T) visit(j, __ldg(pos + j));
-}
-
 }  // namespace sph
 
 // Instantiate CALL(T) for the context's threads per particle.
