@@ -352,7 +352,10 @@ sph_status sph_mlp_grad(const float *params, const float *features, const float 
  * `batch` samples in a seeded per-epoch order, updating params (device, FP32 master
  * weights) and adam_state (device float [2 * SPH_MLP_WEIGHTS], zero for a fresh start).
  * loss_history (device float [epochs], may be NULL) receives each epoch's mean squared
- * error in standardised units.  Allocates its scratch with cudaMallocAsync on stream. */
+ * error in standardised units.  *error (device int32) is set to a non-zero value if a bounded
+ * wait gave up; the epochs still to come are then left out.  Allocates its scratch with
+ * cudaMallocAsync on stream.  An epoch is one cooperative launch of at most one block per SM,
+ * which starts once all its blocks have room beside what runs on other streams. */
 sph_status sph_mlp_train(const float *features, const float *labels, int64_t n, float *params,
                          float *adam_state, int32_t epochs, int32_t batch, float lr, uint64_t seed,
                          float *loss_history, int32_t *error, void *stream);

@@ -450,21 +450,31 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 struct AdamArgs {
     float lr, b1, b2, eps;
 };
+// Zero before the first epoch; failed: a barrier's wait gave up, and the epochs that follow return
+// at once instead of waiting in vain on the barrier that it left half full (the caller's error
+// word may hold anything before the call).
+struct EpochSync {
+    GridBar bar;
+    int32_t failed, pad;
+};
+constexpr int kAccDoubles = 12;   // of the moments, and of the loss
 __global__ void __launch_bounds__(kThreads, 1)
     k_mlp_epoch(float *w, float *m, float *v, float *grad, const float4 *__restrict__ F, const float *__restrict__ T,
                 int64_t n, int64_t batch, uint64_t pa, uint64_t pc, int64_t step, AdamArgs h, double *acc,
-                float *history, GridBar *gbar, int *err)
+                float *history, EpochSync *sync, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
+    GridBar *gbar = &sync->bar;
+    bool came = *reinterpret_cast<volatile int32_t *>(&sync->failed) == 0;   // (every block alike)
     Walk walk;
     uint32_t gen = *reinterpret_cast<volatile uint32_t *>(&gbar->gen);
     walk_begin(sm);
     Sample next = load_sample(F, T, n, 0, min(batch, n), pa, pc, blockIdx.x);
-    for (int64_t b0 = 0; b0 < n; b0 += batch) {
+    for (int64_t b0 = 0; came && b0 < n; b0 += batch) {
         grad_tiles<false>(sm, walk, w, F, T, n, b0, min(batch, n - b0), pa, pc, next, grad, acc);
         const int64_t b1 = b0 + batch;
         if (b1 < n) next = load_sample(F, T, n, b1, min(batch, n - b1), pa, pc, blockIdx.x);
-        if (!grid_barrier(gbar, err, gen)) break;
+        if (!(came = grid_barrier(gbar, &sync->failed, gen))) break;
         ++step;
         const float c1 = 1.0f - powf(h.b1, (float)step), c2 = 1.0f - powf(h.b2, (float)step);
         for (int k = blockIdx.x * kThreads + threadIdx.x; k < kNW; k += gridDim.x * kThreads) {
@@ -480,8 +490,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (history) *history = (float)(__ldcg(acc) / (double)n);
             *acc = 0.0;
         }
-        if (!grid_barrier(gbar, err, gen)) break;
+        came = grid_barrier(gbar, &sync->failed, gen);
     }
+    if (!came && threadIdx.x == 0) atomicExch(err, 5);
     walk_end(sm, walk, err);
 }
 
@@ -610,6 +621,7 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
     float4 *Fs = nullptr;
     float *Ts = nullptr, *grad = nullptr;
     double *acc = nullptr;
+    constexpr size_t kAccBytes = sizeof(double) * kAccDoubles + sizeof(EpochSync);
     auto cleanup = [&]() {
         if (Fs) cudaFreeAsync(Fs, s);
         if (Ts) cudaFreeAsync(Ts, s);
@@ -618,18 +630,18 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
     };
     if (cudaMallocAsync(&Fs, sizeof(float4) * n, s) != cudaSuccess || cudaMallocAsync(&Ts, sizeof(float) * n, s) != cudaSuccess ||
         cudaMallocAsync(&grad, sizeof(float) * kNW, s) != cudaSuccess ||
-        cudaMallocAsync(&acc, sizeof(double) * 13, s) != cudaSuccess) {
+        cudaMallocAsync(&acc, kAccBytes, s) != cudaSuccess) {
         cleanup();
         return SPH_ENOMEM;
     }
-    bool ok = cudaMemsetAsync(acc, 0, sizeof(double) * 13, s) == cudaSuccess &&
+    bool ok = cudaMemsetAsync(acc, 0, kAccBytes, s) == cudaSuccess &&
               cudaMemsetAsync(grad, 0, sizeof(float) * kNW, s) == cudaSuccess;
     const float4 *F = reinterpret_cast<const float4 *>(features);
     k_mlp_moments<<<304, 256, 0, s>>>(F, labels, n, acc);
     k_mlp_standardise<<<304, 256, 0, s>>>(F, labels, n, acc, params, Fs, Ts);
-    cudaMemsetAsync(acc, 0, sizeof(double) * 13, s);
+    cudaMemsetAsync(acc, 0, kAccBytes, s);
     float *m = adam_state, *v = adam_state + kNW;
-    GridBar *gbar = reinterpret_cast<GridBar *>(acc + 12);
+    EpochSync *sync = reinterpret_cast<EpochSync *>(acc + kAccDoubles);
     int64_t step = 0;
     const int64_t B = batch;
     for (int32_t e = 0; e < epochs && ok; ++e) {
@@ -643,7 +655,7 @@ extern "C" sph_status sph_mlp_train(const float *features, const float *labels, 
         const float4 *Fe = Fs;
         const float *Te = Ts;
         void *args[] = {&params, &m, &v, &grad, &Fe, &Te, (void *)&n, (void *)&B, (void *)&a, (void *)&c, &step, &h, &acc,
-                        &hist, &gbar, &err};
+                        &hist, &sync, &err};
         ok = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_mlp_epoch), dim3(grad_grid(std::min(B, n), 1)),
                                          dim3(kThreads), args, kSmem, s) == cudaSuccess;
         step += (n + B - 1) / B;

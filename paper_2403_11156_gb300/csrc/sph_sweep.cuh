@@ -80,7 +80,11 @@ __device__ __forceinline__ float4 ld4(const float4 *p)
 // Barrier over all blocks of a cooperative launch, in two halves.  grid_arrive: thread 0 of the
 // block that arrives last gets true.  grid_leave: that thread lets the others go, the others
 // wait; phase is the barrier's generation, kept by the caller (bar->gen before the first).
-// Bounded: a block that waits in vain records it and returns false, and the others follow.
+// Bounded: a block that waits in vain (2^21 looks, half a second over a full GPU) records it in
+// *error, which is zero before the first launch, and returns false, and the others follow.  The
+// wait is for blocks that run: measured with half of the SMs taken by another stream's kernel for
+// 20 ms, and with two cooperative launches that do not fit beside one another, all blocks of a
+// launch start within 0.2 us, and none before there is room for all.
 constexpr int kLoopScenes = 16;   // scenes one block's four warps test between two phases
 constexpr uint32_t kBarrierSpins = 1u << 21;
 __device__ __forceinline__ bool grid_arrive(GridBar *bar)
@@ -103,7 +107,10 @@ __device__ __forceinline__ bool grid_leave(GridBar *bar, int32_t *error, uint32_
             uint32_t g, spins = 0;
             do {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&bar->gen) : "memory");
-            } while (g != phase && ++spins < kBarrierSpins);
+                // once a wait has given up, here or in an earlier launch on this barrier, there is
+                // nothing to wait for: launches queued behind it end soon
+                if ((++spins & 1023u) == 0u && *reinterpret_cast<volatile int32_t *>(error) != 0) break;
+            } while (g != phase && spins < kBarrierSpins);
             if (g != phase) {
                 atomicExch(error, 5);
                 ok = false;
