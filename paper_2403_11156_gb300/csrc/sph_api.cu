@@ -2,6 +2,7 @@
 // the step as a CUDA graph (conditional while-nodes run the Jacobi loops on the device),
 // an eager mode with optional per-kernel CUDA-event timing, and the read/write paths.
 #include "sph.h"
+#include "sph_filter.h"
 #include "sph_internal.cuh"
 
 #include <cmath>
@@ -774,22 +775,11 @@ sph_status create_impl(const sph_scene_desc *descs, int32_t n, const sph_allocat
             const double margin = 1e-3 * h + 1e-6 * mag;
             q.cull2 = (float)((h + margin) * (h + margin));
         }
-        {
-            // candidate filter of the density sweep (steps of h/512): a neighbour's coordinate
-            // differences are off by at most one step of rounding, one of carry and the float
-            // rounding of coordinates up to qmax; the half-precision sum of squares by 2e-3 more
-            double mag = 0.0;
-            for (int a = 0; a < 3; ++a)
-                mag = std::max(mag, std::max(std::fabs((double)d.domain_min[a]), std::fabs((double)d.domain_max[a])));
-            const double qmax = 2.0 * mag + 16.0 * h;
-            const double off = 2.0 / 512.0 + 16.0 * std::ldexp(qmax, -22) / h;
-            const double thr = std::pow(1.0 + 1.7321 * off, 2.0) * 1.002;
-            q.qscale = (float)(512.0 / h);
-            q.qmax = (float)qmax;
-            // steps of 2^-10 from 1 to 2, rounded up; past 2 nothing is filtered out (half infinity)
-            const uint32_t half = thr < 2.0 ? 0x3c00u + (uint32_t)std::ceil((thr - 1.0) * 1024.0) : 0x7c00u;
-            q.qthr = half | half << 16;
-        }
+        const DensityFilter filter =
+            density_filter(h, (double)q.cell * std::max(q.dims[0], std::max(q.dims[1], q.dims[2])));
+        q.qscale = filter.scale;
+        q.qreach = filter.reach;
+        q.qthr = filter.thr;
         q.cg_tol = d.cg_tol > 0.0f ? d.cg_tol : 1e-4f;
         q.cg_max = d.cg_max_iter > 0 ? d.cg_max_iter : 500;
         cap_f = std::max(cap_f, q.cap_f);

@@ -131,7 +131,7 @@ __global__ void k_step_begin(Ptrs P)
 // the exact test on every candidate, in the same order.
 //
 // A particle whose passed candidates exceed the list, or that has left the range the filter
-// holds for (SceneDev::qmax), takes the exact predicate over its rows instead.
+// holds for (SceneDev::qreach), takes the exact predicate over its rows instead.
 //
 // Between the phases a thread keeps its first kStage passed candidates in shared memory: written
 // straight to the list, whose entries the lanes of a warp reach at different times, each store
@@ -272,7 +272,8 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
             }
         }
         int total = -1;   // exact count, where the list was built by the exact predicate
-        if (passed > cap_f || !(fmaxf(fmaxf(fabsf(pi.x), fabsf(pi.y)), fabsf(pi.z)) <= sc.qmax)) {
+        const float away = fmaxf(fmaxf(fabsf(pi.x - sc.origin[0]), fabsf(pi.y - sc.origin[1])), fabsf(pi.z - sc.origin[2]));
+        if (passed > cap_f || !(away <= sc.qreach)) {
             total = exact_list(P, st, i, pi, h2, cap_f);
             passed = min(total, cap_f);
         }

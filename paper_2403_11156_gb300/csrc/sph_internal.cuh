@@ -58,8 +58,8 @@ struct SceneDev {
     int32_t strong;                   // strong rigid coupling: bodies pushed during the solves
     float learned_frac;               // fraction of the network's stiffness warm-starting it
     int32_t learned_gate;             // the network runs only above this many density iterations
-    float qscale, qmax;               // candidate filter: 512 / h, largest coordinate it holds for
-    uint32_t qthr;                    // its threshold on (d/h)^2 as a pair of halves
+    float qscale, qreach;             // candidate filter (sph_filter.h): 512 / h, how far from the
+    uint32_t qthr;                    // origin it holds, its threshold on (d/h)^2 as a pair of halves
     double err_scale;                 // 1 / (nf rho0): a solve's error sum to its mean per rho0
 };
 
