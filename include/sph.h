@@ -442,8 +442,8 @@ sph_status sph_launch_count(sph_ctx *ctx, int64_t *out);
  * device current) and should come before any stream capture.  Calls no allocator.
  * Points outside [domain_min, domain_max] (and NaN coordinates) are clamped into the edge
  * cells of the padded grid, as in sph_step.  Inside a cell of up to 64 points the order
- * comes from counting each point's smaller indices; a more crowded cell is sorted by one
- * thread block (a stable radix sort on the index), so the work stays linear in n however
+ * comes from counting each point's smaller indices; a more crowded cell is put in order by
+ * one warp or block through a bitmap of its indices, so the work stays linear in n however
  * the points crowd into cells.
  * Beyond 8,192 points (or 24,576 cells) the call is one cooperative launch of at most one block
  * per SM: it starts once all its blocks have room beside what runs on other streams.

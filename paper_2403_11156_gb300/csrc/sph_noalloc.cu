@@ -6,8 +6,8 @@
 // GPU's memory budget and forbid libraries from allocating, and real-time loops in which
 // an allocation's latency or a possible out-of-memory failure is not acceptable.  For them
 // sph_grid_order_noalloc runs the same counting sort as the per-step neighbour search
-// (cell keys, histogram, prefix sum, scatter, rank by index, with the crowded cells sorted by one
-// block each) with its scratch in one file-scope static device array of fixed size, which
+// (cell keys, histogram, prefix sum, scatter, rank by index, with the crowded cells in order by a
+// bitmap each) with its scratch in one file-scope static device array of fixed size, which
 // every GPU that loads the library holds until the process exits.
 #include "sph.h"
 #include "sph_blocksort.cuh"
@@ -105,13 +105,72 @@ __device__ __forceinline__ uint32_t key_of(const Grid &g, const float *__restric
     return (uint32_t)ix + (uint32_t)g.dims[0] * ((uint32_t)iy + (uint32_t)g.dims[1] * (uint32_t)iz);
 }
 
-// Put the indices sid[b..e) of a crowded cell in order and write them out, by the whole block, with
-// other[b..e) for the passes (sorted by index alone: an index is its own value).
-__device__ void sort_cell(uint32_t *sid, uint32_t *other, uint32_t b, uint32_t e, int32_t *order)
+// A crowded cell's indices sid[b..e), each below n and there once, in ascending order to order[b..e):
+// an index's place is the number of bits below its own in a bitmap of the members.  Linear in the
+// members and n / 32 words whatever their number; the radix sort of the step's crowded cells takes
+// four passes of several barriers, 5 us for a cell of 65 and 2,110 for one of 262,000.
+// By the whole block (every thread calls it).
+__device__ void order_crowd(const uint32_t *sid, uint32_t b, uint32_t e, uint32_t n, int32_t *order)
 {
-    block_sort_segment(sid, sid, other, other, b, e);
-    for (uint32_t d = b + threadIdx.x; d < e; d += kLargeThreads) order[d] = (int32_t)sid[d];
+    __shared__ __align__(16) uint32_t s_map[kMaxPoints / 32];
+    __shared__ uint32_t s_before[kLargeThreads];   // bits before each 256
+    static_assert(kMaxPoints == 256 * kLargeThreads, "eight words a thread");
+    uint4 *mine = reinterpret_cast<uint4 *>(s_map) + 2 * threadIdx.x;
+    mine[0] = mine[1] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
+    for (uint32_t t = b + threadIdx.x; t < e; t += kLargeThreads) {
+        const uint32_t i = sid[t];
+        if (i < n) atomicOr(&s_map[i >> 5], 1u << (i & 31u));
+    }
+    __syncthreads();
+    const uint4 p = mine[0], q = mine[1];
+    uint32_t total;
+    s_before[threadIdx.x] = block_scan(__popc(p.x) + __popc(p.y) + __popc(p.z) + __popc(p.w) + __popc(q.x) + __popc(q.y) +
+                                           __popc(q.z) + __popc(q.w), total);
+    __syncthreads();
+    for (uint32_t t = b + threadIdx.x; t < e; t += kLargeThreads) {
+        const uint32_t i = sid[t];
+        if (i >= n) continue;
+        uint32_t at = b + s_before[i >> 8] + __popc(s_map[i >> 5] & ((1u << (i & 31u)) - 1u));
+        for (uint32_t w = (i >> 8) * 8u; w < i >> 5; ++w) at += __popc(s_map[w]);
+        if (at < e) order[at] = (int32_t)i;
+    }
+    __syncthreads();
+}
+
+// The same by one warp, for indices below 8,192, with 256 words of its own and as many counts.
+constexpr int kWarpMap = 256;
+__device__ void order_crowd_warp(const uint32_t *sid, uint32_t b, uint32_t e, uint32_t *map, uint16_t *before, int32_t *order)
+{
+    const int lane = threadIdx.x & 31;
+    uint4 *mine = reinterpret_cast<uint4 *>(map) + 2 * lane;
+    mine[0] = mine[1] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    for (uint32_t t = b + lane; t < e; t += 32u) atomicOr(&map[sid[t] >> 5], 1u << (sid[t] & 31u));
+    __syncwarp();
+    const uint4 p = mine[0], q = mine[1];
+    const uint32_t w[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+    uint32_t sum = 0u, x;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sum += __popc(w[k]);
+    x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    x -= sum;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        before[8 * lane + k] = (uint16_t)x;
+        x += __popc(w[k]);
+    }
+    __syncwarp();
+    for (uint32_t t = b + lane; t < e; t += 32u) {
+        const uint32_t i = sid[t];
+        order[b + before[i >> 5] + __popc(map[i >> 5] & ((1u << (i & 31u)) - 1u))] = (int32_t)i;
+    }
+    __syncwarp();
 }
 
 // The barrier over the blocks of a call, on a word that no call resets: a captured call is replayed
@@ -163,12 +222,14 @@ struct OrderBarrier {
 
 // The whole order in one cooperative launch: keys and histogram, prefix sum (each block sums its
 // share of the cells, then adds the shares before it), scatter, rank inside the cell by index or,
-// for the crowded cells, which the prefix sum queues, block sort; four barriers.  The histogram
+// for the crowded cells, which the prefix sum queues, by bitmap; four barriers.  The histogram
 // is zero between calls: the prefix sum clears what it has read.  Its total has to be n; where an
-// earlier call left something in it, it is cleared and filled once more.
-// Calls that overlap race on the scratch: what is read from it is checked (places below n, the
-// queue's length) before it is used as an index.  As six launches it was bound by them: 262,143 points 39.0 -> 22.1 us (24.6 with count and generation in two words,
-// 28.7 with a memset that cleared both and the histogram before every call).
+// earlier call left something in it, it is cleared and filled once more.  Calls that overlap race
+// on the scratch: what is read from it is checked (places below n, the queue's length) before it
+// is used as an index.
+// As six launches it was bound by them: 262,143 points 39.0 -> 22.5 us (24.6 with the barrier's
+// count and generation in two words, 28.7 with a memset that cleared both and the histogram before
+// every call); 100,000 points in 1,000 crowded cells 77 -> 40.
 __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, const float *__restrict__ x, int64_t n,
                                                             int64_t ncell, uint32_t *keys_out, int32_t *order)
 {
@@ -244,8 +305,7 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
         for (uint32_t t = b; t < e; ++t) rank += (v.sid[t] < my) ? 1u : 0u;
         if (b + rank < e) order[b + rank] = (int32_t)my;
     }
-    // the queued cells: one block per cell at a time sorts the cell's indices stably and writes
-    // them out (the slot region, free once scattered, is its scratch).
+    // the queued cells, one block per cell at a time
     __shared__ uint32_t s_seg[2];
     const int nq = min(*reinterpret_cast<volatile int32_t *>(&ctl->nlarge[0]), (int)kMaxLarge);
     for (int q = blockIdx.x; q < nq; q += gridDim.x) {
@@ -255,20 +315,27 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order(View v, Grid g, cons
             s_seg[1] = min(v.start[c + 1], (uint32_t)n);
         }
         __syncthreads();
-        sort_cell(v.sid, v.slot, s_seg[0], s_seg[1], order);
+        order_crowd(v.sid, s_seg[0], s_seg[1], (uint32_t)n, order);
     }
     bar.leave(false);
 }
 
-// Few points in few cells: the same in one block, histogram, starts and order in shared memory.
-// 3,001 points in 10,648 cells: 28.7 us as six launches, 8.2 us here (a barrier over blocks
-// costs more than this range's work).
+// Few points in few cells: the same in one block, histogram, starts and order in shared memory, a
+// warp for each crowded cell.  3,001 points in 10,648 cells: 28.7 us as six launches, 8.2 us here
+// (a barrier over blocks costs more than this range's work); 8,192 in 21,952 cells 15.5 us, as the
+// cooperative kernel's 15.6, in 64 crowded cells 13.0 against 19.5, with 126 cells of 65 17.2 (35.8
+// as six launches, 610 with the block's radix sort for one cell after the other).
 constexpr int64_t kOneBlockPoints = 8 * kLargeThreads, kOneBlockCells = 24 * kLargeThreads;
+static_assert(kOneBlockPoints == 32 * kWarpMap, "a bit for each point");
+constexpr int kOneBlockMaps = kLargeThreads / 32 * (kWarpMap + kWarpMap / 2);   // words
 __global__ void __launch_bounds__(kLargeThreads) k_na_order_one(Control *ctl, Grid g, const float *__restrict__ x, int n, int ncell,
                                                                 uint32_t *keys_out, int32_t *order)
 {
-    extern __shared__ uint32_t sm[];
-    uint32_t *start = sm, *sid = sm + ncell + 1, *other = sid + n;
+    extern __shared__ __align__(16) uint32_t sm[];
+    // a bitmap and its counts for each warp, the cells' starts, the order inside them not yet fixed
+    uint32_t *map = sm + (threadIdx.x >> 5) * kWarpMap;
+    uint16_t *before = reinterpret_cast<uint16_t *>(sm + kLargeThreads / 32 * kWarpMap) + (threadIdx.x >> 5) * kWarpMap;
+    uint32_t *start = sm + kOneBlockMaps, *sid = start + ncell + 1;
     __shared__ int s_large;
     __shared__ uint32_t s_cells[kOneBlockPoints / (kRankSmall + 1)];   // the crowded ones
     constexpr int kOwn = (int)(kOneBlockPoints / kLargeThreads);
@@ -323,9 +390,9 @@ __global__ void __launch_bounds__(kLargeThreads) k_na_order_one(Control *ctl, Gr
         order[b + rank] = i;
     }
     __syncthreads();
-    for (int q = 0; q < s_large; ++q) {
+    for (int q = t >> 5; q < s_large; q += kLargeThreads / 32) {
         const uint32_t c = s_cells[q];
-        sort_cell(sid, other, start[c], start[c + 1], order);
+        order_crowd_warp(sid, start[c], start[c + 1], map, before, order);
     }
 }
 
@@ -370,10 +437,10 @@ extern "C" sph_status sph_grid_order_noalloc(const float *x, int64_t n, const fl
     }
     View v = carve(base);
     cudaStream_t s = (cudaStream_t)stream;
-    if (n <= kOneBlockPoints && ncell <= kOneBlockCells && n <= kRankSmall / 2 * ncell) {   // (no crowd of crowded cells)
-        const size_t bytes = sizeof(uint32_t) * (size_t)(ncell + 1 + 2 * n);
+    if (n <= kOneBlockPoints && ncell <= kOneBlockCells) {
+        const size_t bytes = sizeof(uint32_t) * (size_t)(kOneBlockMaps + ncell + 1 + n);
         if (cudaFuncSetAttribute(k_na_order_one, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(uint32_t) * (kOneBlockCells + 1 + 2 * kOneBlockPoints))) != cudaSuccess)
+                                 (int)(sizeof(uint32_t) * (kOneBlockMaps + kOneBlockCells + 1 + kOneBlockPoints))) != cudaSuccess)
             return SPH_ECUDA;
         k_na_order_one<<<1, kLargeThreads, bytes, s>>>(v.ctl, g, x, (int)n, (int)ncell, keys, order);
         return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;

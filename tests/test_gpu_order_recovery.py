@@ -47,7 +47,7 @@ extern "C" int run_one(void *ctl, const float *x, int n, int side, float cell, i
 {
     Grid g{{-cell, -cell, -cell}, cell, {side, side, side}};
     const int ncell = side * side * side;
-    const size_t bytes = sizeof(uint32_t) * (size_t)(ncell + 1 + 2 * n);
+    const size_t bytes = sizeof(uint32_t) * (size_t)(kOneBlockMaps + ncell + 1 + n);
     if (cudaFuncSetAttribute(k_na_order_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return 1;
     k_na_order_one<<<1, kLargeThreads, bytes>>>((Control *)ctl, g, x, n, ncell, nullptr, order);
     return cudaDeviceSynchronize() != cudaSuccess;
