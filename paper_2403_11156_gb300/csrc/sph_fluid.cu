@@ -851,7 +851,11 @@ __global__ void __launch_bounds__(kCheckThreads) k_solver_check(Ptrs P, cudaGrap
 // (14 us) outweigh its passes; 8k particles: 4 steps 533 -> 480 us.  With more blocks a block's
 // second round waits for nothing else to fill the SM and the separate kernels win (20k
 // particles in two rounds 257 us a step against 236, 100k 447 against 433, 1.2M 2472 against 2376).
+// And with many scenes: the last block's four warps test them four at a time, on the way of every
+// iteration (4 + 12 iterations a step, one launch against separate kernels: 4 scenes of 1,000
+// particles 265 and 343 us, 8 326 and 357, 12 382 and 380, 16 459 and 401).
 constexpr int kSolveBlocksPerSm = 8;
+constexpr int kSolveScenes = 8;
 template <int S, int T>
 __global__ void __launch_bounds__(kBlock, kSolveBlocksPerSm) k_solve(const __grid_constant__ Ptrs P)
 {
@@ -1207,9 +1211,8 @@ static const void *solve_kernel(const Ptrs &P, int solver)
 }
 int solve_grid(const Ptrs &P, int batch)
 {
-    // the check walks the scenes with four warps; the passes with eight gathers in flight keep
-    // their own kernels
-    if (batch != kBatch || P.nscenes > kLoopScenes || P.ntblk < 1) return 0;
+    // the passes with eight gathers in flight keep their own kernels
+    if (batch != kBatch || P.nscenes > kSolveScenes || P.ntblk < 1) return 0;
     int dev = 0, nsm = 0, coop = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)

@@ -85,7 +85,6 @@ __device__ __forceinline__ float4 ld4(const float4 *p)
 // wait is for blocks that run: measured with half of the SMs taken by another stream's kernel for
 // 20 ms, and with two cooperative launches that do not fit beside one another, all blocks of a
 // launch start within 0.2 us, and none before there is room for all.
-constexpr int kLoopScenes = 16;   // scenes one block's four warps test between two phases
 constexpr uint32_t kBarrierSpins = 1u << 21;
 __device__ __forceinline__ bool grid_arrive(GridBar *bar)
 {

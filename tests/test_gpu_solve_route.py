@@ -13,7 +13,7 @@ SEPARATE = {"div_pass_a", "div_pass_b", "div_check", "dens_pass_a", "dens_pass_b
 
 
 @pytest.mark.parametrize("lanes", [1, 2, 4, 8])
-@pytest.mark.parametrize("sizes,one", [([(9, 11, 13)], True), ([(5, 4, 3)] * 16, True), ([(5, 4, 3)] * 17, False),
+@pytest.mark.parametrize("sizes,one", [([(9, 11, 13)], True), ([(5, 4, 3)] * 8, True), ([(5, 4, 3)] * 9, False),
                                        ([(60, 60, 100)], False)])
 def test_route(sizes, one, lanes):
     descs = [scenes.dam_break_small(seed=2 + k, n=n, box=2.2, lanes_per_particle=lanes, warm_start=scenes.WARM_ZERO)
