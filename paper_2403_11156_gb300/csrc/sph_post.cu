@@ -138,6 +138,14 @@ __device__ __forceinline__ f2 sub2(f2 a, f2 b)
 __device__ __forceinline__ f2 dup(float a) { return pack_xy(a, a); }
 __device__ __forceinline__ void unpack(f2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 
+// Largest of three, NaN if one is.
+__device__ __forceinline__ float max_nan(float a, float b, float c)
+{
+    float r;
+    asm("{ .reg .f32 t; max.NaN.f32 t, %1, %2; max.NaN.f32 %0, t, %3; }" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // Square roots of a pair (a, b) of normal numbers: g = x y, g + (y/2) (x - g g) from y =
 // rsqrt(x), Newton's step with the residual exact in FP32 (Markstein's square root), in packed
 // FP32.  The value before the last rounding is within 2^-44 of the root: of all significands
@@ -230,12 +238,11 @@ __global__ void __launch_bounds__(32 * kTileWarps, 8)
                 float4 p;
                 if (t + (uint32_t)lane < re) {
                     p = __ldg(sorted + t + lane);
-                    // distance to the box: no larger than to any node, operation by operation
-                    const float dx = fmaxf(fmaxf(lox - p.x, p.x - hix), 0.0f), dy = fmaxf(fmaxf(loy - p.y, p.y - hiy), 0.0f),
-                                dz = fmaxf(fmaxf(loz - p.z, p.z - hiz), 0.0f);
-                    // (a NaN coordinate, which the maxima here and in add() pass over, is near no node)
-                    const float any = p.x + p.y + p.z;
-                    keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < h2 && any == any;
+                    // distance to the box: no larger than to any node, operation by operation; a NaN
+                    // coordinate, which add()'s maximum would pass over, stays one and is not near
+                    const float dx = max_nan(lox - p.x, p.x - hix, 0.0f), dy = max_nan(loy - p.y, p.y - hiy, 0.0f),
+                                dz = max_nan(loz - p.z, p.z - hiz, 0.0f);
+                    keep = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < h2;
                 }
                 const unsigned kept = __ballot_sync(0xffffffffu, keep);
                 if (keep) buf[cnt + __popc(kept & ((1u << lane) - 1u))] = p;
