@@ -377,7 +377,7 @@ __device__ __forceinline__ void emit_tet(const Cube &c, uint32_t above, int t, f
 // 16M cubes of the 1.2M scene: about 250 us; 640 us with a count a cube in memory (64 MB written,
 // scanned and read) and a crossed cube's thread writing all its triangles alone; 276 us as one
 // launch with look-back between the tiles, which it spent waiting.
-constexpr int kMeshThreads = 256, kMeshItems = 8, kMeshTile = kMeshThreads * kMeshItems;
+constexpr int kMeshThreads = 256;   // of a block, and cubes of a tile: ITEMS a thread
 // Division of n < 2^31 by d >= 1: n m >> (31 + l), l = ceil(log2 d), m = ceil(2^(31+l) / d).
 struct Divisor {
     uint32_t d, l;
@@ -410,12 +410,13 @@ __device__ __forceinline__ void mesh_counts(uint8_t *s_count)
 
 // Corner bits of this thread's cubes of a tile: base + t, base + t + 256, ...: a warp reads 33
 // consecutive values of each of four rows.
-__device__ __forceinline__ void mesh_corners(const MeshGrid &g, uint32_t tile, uint32_t (&above)[kMeshItems])
+template <int ITEMS>
+__device__ __forceinline__ void mesh_corners(const MeshGrid &g, uint32_t tile, uint32_t (&above)[ITEMS])
 {
     const int64_t dz = (int64_t)g.nx * g.ny;
 #pragma unroll
-    for (int q = 0; q < kMeshItems; ++q) {
-        const uint32_t cube = tile * kMeshTile + (uint32_t)(q * kMeshThreads) + threadIdx.x;
+    for (int q = 0; q < ITEMS; ++q) {
+        const uint32_t cube = tile * (uint32_t)(ITEMS * kMeshThreads) + (uint32_t)(q * kMeshThreads) + threadIdx.x;
         above[q] = 0u;
         if (cube < g.cubes) {
             const uint32_t row = g.by_x.quotient(cube), i = cube - row * g.by_x.d, k = g.by_y.quotient(row), j = row - k * g.by_y.d;
@@ -428,15 +429,16 @@ __device__ __forceinline__ void mesh_corners(const MeshGrid &g, uint32_t tile, u
     }
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kMeshThreads) k_mt_count(MeshGrid g, uint32_t *tile_count)
 {
     __shared__ uint8_t s_count[256];
     __shared__ uint32_t s_warp[kMeshThreads / 32];
     mesh_counts(s_count);
-    uint32_t above[kMeshItems], n = 0u;
+    uint32_t above[ITEMS], n = 0u;
     mesh_corners(g, blockIdx.x, above);
 #pragma unroll
-    for (int q = 0; q < kMeshItems; ++q) n += s_count[above[q]];
+    for (int q = 0; q < ITEMS; ++q) n += s_count[above[q]];
     n = __reduce_add_sync(0xffffffffu, n);
     if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = n;
     __syncthreads();
@@ -445,6 +447,12 @@ __global__ void __launch_bounds__(kMeshThreads) k_mt_count(MeshGrid g, uint32_t 
         tile_count[blockIdx.x] = n;
     }
 }
+
+// Cubes a thread.  Eight leave few blocks to a small grid, each writing a long list: a ball's surface
+// in 64^3 cubes takes 18.6 us with eight and 13.8 with one (55.8 with a thread a cube for
+// everything), a noisy one 153 and 75, in 100^3 cubes 31.2 and 27.9, 128^3 40.1 and 44.3, 252^3
+// 130 and 259 (the places of 62,500 tiles).  The line: five tiles of eight a SM.
+int mesh_items(int64_t cubes) { return cubes < (int64_t)5 * 152 * 8 * kMeshThreads ? 1 : 8; }
 
 // Exclusive sums of the tiles' counts in place, the total behind them (one block).
 __global__ void __launch_bounds__(1024) k_mt_places(uint32_t *tile_count, int32_t ntiles)
@@ -472,6 +480,7 @@ __global__ void __launch_bounds__(1024) k_mt_places(uint32_t *tile_count, int32_
     if (threadIdx.x == 0) tile_count[ntiles] = run;
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kMeshThreads)
     k_mt_emit(MeshGrid g, float ox, float oy, float oz, float sp, const uint32_t *__restrict__ place, float *tris, int64_t cap)
 {
@@ -479,20 +488,21 @@ __global__ void __launch_bounds__(kMeshThreads)
     const int64_t first = (int64_t)place[tile];
     if ((int64_t)place[tile + 1] == first || first >= cap) return;
     constexpr int kWarps = kMeshThreads / 32;
-    static_assert(kMeshItems * kWarps == 64, "one warp scans the sums of all items, two a lane");
+    constexpr int kSums = ITEMS * kWarps;
+    static_assert(kSums <= 64, "one warp scans the sums of all items, two a lane");
     __shared__ uint8_t s_count[256];                 // triangles by corner bits
-    __shared__ uint32_t s_list[kMeshTile];           // crossed cubes: index in the tile, corner bits
-    __shared__ uint16_t s_first[kMeshTile];          // their first triangle in the tile (at most 24,576)
-    __shared__ uint32_t s_sum[kMeshItems * kWarps];  // per item and warp, then their exclusive sums
+    __shared__ uint32_t s_list[ITEMS * kMeshThreads];           // crossed cubes: index in the tile, corner bits
+    __shared__ uint16_t s_first[ITEMS * kMeshThreads];          // their first triangle in the tile (at most 24,576)
+    __shared__ uint32_t s_sum[kSums];  // per item and warp, then their exclusive sums
     __shared__ uint32_t s_crossed;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     mesh_counts(s_count);
     // per item, places in cube order from sums over the warp of the triangles (low 16 bits)
     // and the crossed cubes (high 16 bits)
-    uint32_t above[kMeshItems], sum[kMeshItems];
+    uint32_t above[ITEMS], sum[ITEMS];
     mesh_corners(g, tile, above);
 #pragma unroll
-    for (int q = 0; q < kMeshItems; ++q) {
+    for (int q = 0; q < ITEMS; ++q) {
         const uint32_t n = s_count[above[q]], v = n | (n ? 0x10000u : 0u);
         uint32_t x = v;
         if (__any_sync(0xffffffffu, n != 0u)) {
@@ -507,7 +517,8 @@ __global__ void __launch_bounds__(kMeshThreads)
     }
     __syncthreads();
     if (warp == 0) {
-        const uint32_t a = s_sum[2 * lane], b = s_sum[2 * lane + 1];
+        const bool any = 2 * lane < kSums;
+        const uint32_t a = any ? s_sum[2 * lane] : 0u, b = any ? s_sum[2 * lane + 1] : 0u;
         uint32_t x = a + b;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -515,13 +526,15 @@ __global__ void __launch_bounds__(kMeshThreads)
             if (lane >= o) x += y;
         }
         if (lane == 31) s_crossed = x >> 16;
-        s_sum[2 * lane] = x - a - b;
-        s_sum[2 * lane + 1] = x - b;
+        if (any) {
+            s_sum[2 * lane] = x - a - b;
+            s_sum[2 * lane + 1] = x - b;
+        }
     }
     __syncthreads();
     const uint32_t crossed = s_crossed;
 #pragma unroll
-    for (int q = 0; q < kMeshItems; ++q) {
+    for (int q = 0; q < ITEMS; ++q) {
         if (s_count[above[q]] == 0u) continue;
         const uint32_t at = s_sum[q * kWarps + warp] + sum[q];
         s_list[at >> 16] = (uint32_t)(q * kMeshThreads + t) | (above[q] << 16);
@@ -536,7 +549,7 @@ __global__ void __launch_bounds__(kMeshThreads)
         int64_t o = first + s_first[c];
         for (int q = 0; q < tet; ++q) o += tet_count(a, q);
         if (o >= cap) continue;
-        const uint32_t cube = tile * kMeshTile + (e & 0xffffu), row = g.by_x.quotient(cube), k = g.by_y.quotient(row);
+        const uint32_t cube = tile * (uint32_t)(ITEMS * kMeshThreads) + (e & 0xffffu), row = g.by_x.quotient(cube), k = g.by_y.quotient(row);
         const Cube cb{g.f, g.nx, g.ny, (int32_t)(cube - row * g.by_x.d), (int32_t)(row - k * g.by_y.d), (int32_t)k, ox, oy, oz, sp};
         emit_tet(cb, a, tet, g.iso, o, tris, cap);
     }
@@ -658,15 +671,21 @@ extern "C" sph_status sph_surface_mesh(const float *field, const int32_t dims[3]
     const int64_t cubes = (int64_t)(dims[0] - 1) * (dims[1] - 1) * (dims[2] - 1);
     if ((int64_t)dims[0] * dims[1] * dims[2] > ((int64_t)1 << 31)) return SPH_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t ntiles = (cubes + kMeshTile - 1) / kMeshTile;
+    const int items = mesh_items(cubes);
+    const int64_t ntiles = (cubes + items * kMeshThreads - 1) / (items * kMeshThreads);
     uint32_t *place = nullptr, total = 0;
     cudaError_t e = cudaMallocAsync((void **)&place, sizeof(uint32_t) * (size_t)(ntiles + 1), s);
     if (e == cudaSuccess) {
         const MeshGrid g{field, dims[0], dims[1], Divisor((uint32_t)dims[0] - 1u), Divisor((uint32_t)dims[1] - 1u),
                          (uint32_t)cubes, iso};
-        k_mt_count<<<(unsigned)ntiles, kMeshThreads, 0, s>>>(g, place);
+        const unsigned blocks = (unsigned)ntiles;
+        if (items == 8) k_mt_count<8><<<blocks, kMeshThreads, 0, s>>>(g, place);
+        else k_mt_count<1><<<blocks, kMeshThreads, 0, s>>>(g, place);
         k_mt_places<<<1, 1024, 0, s>>>(place, (int32_t)ntiles);
-        if (cap > 0) k_mt_emit<<<(unsigned)ntiles, kMeshThreads, 0, s>>>(g, origin[0], origin[1], origin[2], spacing, place, tris, cap);
+        if (cap > 0) {
+            if (items == 8) k_mt_emit<8><<<blocks, kMeshThreads, 0, s>>>(g, origin[0], origin[1], origin[2], spacing, place, tris, cap);
+            else k_mt_emit<1><<<blocks, kMeshThreads, 0, s>>>(g, origin[0], origin[1], origin[2], spacing, place, tris, cap);
+        }
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&total, place + ntiles, sizeof total, cudaMemcpyDeviceToHost, s);
         cudaFreeAsync(place, s);
