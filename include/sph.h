@@ -201,7 +201,9 @@ sph_status sph_create_batch(const sph_scene_desc *scenes, int32_t n, const sph_a
 /* Enqueue one DFSPH step of every scene (Sec. 4.2 order; Sec. 3.3 Alg. general_algorithm,
  * Sec. 3.4.2 Alg. ppe_solver for both solves).  dt > 0: that step size for all scenes;
  * dt <= 0: each scene's CFL step (dt_max when cfl <= 0).  Returns without waiting;
- * errors of the step surface at the next synchronising call. */
+ * errors of the step surface at the next synchronising call.  A context of up to eight scenes
+ * whose sweeps fit the GPU at once runs each solve as one cooperative launch, which starts
+ * once all its blocks have room beside what runs on other streams. */
 sph_status sph_step(sph_ctx *ctx, float dt);
 
 /* Enqueue n steps (same dt rule). */
@@ -308,7 +310,9 @@ typedef struct sph_tuning {
 sph_status sph_get_tuning(sph_ctx *ctx, sph_tuning *out);
 
 /* Per-kernel timing collected in eager timing mode: up to cap entries of name (63
- * chars + NUL), launches and total milliseconds; returns the entry count in *n. */
+ * chars + NUL), launches and total milliseconds; returns the entry count in *n.  Where a
+ * solve is one launch (see sph_step) it appears as div_solve or dens_solve in place of its
+ * passes and checks, here and in the device trace. */
 typedef struct sph_kernel_time {
     char name[64];
     int64_t launches;
@@ -472,8 +476,9 @@ sph_status sph_grid_order_noalloc_status(void *stream);
  * (the SPH interpolant of Sec. 3.2 applied to 1: about 1 inside, 0 outside) at the grid
  * nodes origin + spacing (i, j, k), 0 <= i < dims[0] ..., for scene `scene` at its
  * current positions, rho_j the density of the last step (rho0 before the first step).
- * field: device float [dims[2]][dims[1]][dims[0]], caller-owned.  Enqueued on the
- * context's stream; returns after enqueueing.  The reconstruction of a surface is the
+ * field: device float [dims[2]][dims[1]][dims[0]], caller-owned.  A particle with a NaN
+ * coordinate adds nothing.  Enqueued on the context's stream, on which it uses the step's
+ * sort scratch; returns after enqueueing.  The reconstruction of a surface is the
  * iso-level 0.5 of this field (sph_surface_mesh).  SPH_EINVAL for a scene out of range,
  * NULL pointers, a spacing that is not positive and finite, dims < 1, a non-finite origin
  * or more than 2^31 nodes; SPH_ECUDA if scratch cannot be allocated. */

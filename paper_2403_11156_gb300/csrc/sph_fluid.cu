@@ -9,7 +9,8 @@
 // through that list, lane s taking entries s, s + T, ..., and combines the T partial sums
 // with warp shuffles.  The solvers' error sums are accumulated per block in FP64 by pass A,
 // folded by pass B and summed in a fixed order by a one-block check kernel, which also
-// decides the loop condition on the device (CUDA graph conditional node).
+// decides the loop condition on the device (CUDA graph conditional node); small contexts run a
+// whole solve as one cooperative launch (k_solve).
 #include <cuda_fp16.h>
 #include <math_constants.h>
 
@@ -125,7 +126,7 @@ __global__ void k_step_begin(Ptrs P)
 // 2^16, added to the bits of the half 1536, is that half plus the difference (a half's step is 1
 // from 1024 to 2048, which covers differences up to h; beyond, the value only has to stay
 // beyond), so no conversion is needed; one 32-bit addition serves both, its carry being one step
-// in the second.  The threshold lies above 1 by more than all rounding (SceneDev::qthr), so every
+// in the second.  The threshold lies above 1 by more than all rounding (sph_filter.h), so every
 // neighbour passes, with 2 to 4 % more.  Phase 2 walks the passed ones with the exact predicate,
 // drops those that fail from the list in place, and sums: list, counts and sums are those of
 // the exact test on every candidate, in the same order.

@@ -4,8 +4,9 @@
 //
 // with Q a degree-9 polynomial without constant term fitted to log2 erfc(t/sqrt 2) on
 // [0, 6] (minimax of the error times erfc, by iteratively reweighted least squares against
-// 40-digit values).  No branch and one ex2 in place of erff's two polynomial branches and its exp: 8
-// instructions an evaluation in the pairwise form below, about 28 before.  Error against
+// 40-digit values).  No branch and one ex2, two values at a time: the forward pass of 1.2M rows
+// takes 96 us with it (83 without the rounding ties below) where it took 205 with the library's erff.
+// Error against
 // 64-bit values over [-9, 9]: at most 2.4e-7 and 5.0e-8 rms, where 0.5 z (1 + erff(z/sqrt 2))
 // has 4.5e-7 and 6.4e-8.  Beyond |z| = 6 erfc is held at its value there (2e-9).  NaN stays
 // NaN, +inf gives +inf and -inf gives NaN, as the product form does.

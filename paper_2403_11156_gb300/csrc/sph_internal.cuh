@@ -284,7 +284,7 @@ struct Ptrs {
     int32_t scan_tiles;
     // implicit viscosity CG
     float4 *cg_r, *cg_p, *cg_ap;
-    double *cg_dots;                  // per-block partials [max(nfblk, ntblk)][2]
+    double *cg_dots;                  // per-block partials [max(nfblk, ntblk)]; [..][2] in the CG's start
     // network
     float *mlp_w;                     // device parameter block (float)
     int2 *mlp_rows;                   // [nlearned] gated (particle, scene) rows of the step

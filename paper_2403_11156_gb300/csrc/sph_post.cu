@@ -5,8 +5,9 @@
 //  * field: phi(g) = sum_j (m / rho_j) W(|g - x_j|), the SPH interpolant (Sec. 3.2) of the
 //    constant 1: about 1 inside the fluid, 0 outside.  The scene's particles are first
 //    sorted into its cell grid (counting sort, then a rank by index inside each cell, so
-//    the summation order and the result are reproducible); one thread per grid node then
-//    walks the node's stencil of cells.
+//    the summation order and the result are reproducible).  On fine grids a warp then takes a
+//    tile of nodes with the particles near it; on coarse ones a thread per node walks the
+//    node's stencil of cells.
 //  * mesh: each grid cube is split into the six tetrahedra around its diagonal from corner
 //    0 to corner 7 (corner index = dx + 2 dy + 4 dz); per tetrahedron the corners above the
 //    iso-level are cut off by one triangle (one or three corners above) or two (two
@@ -108,12 +109,16 @@ __global__ void k_pf_field(const float4 *__restrict__ sorted, const uint32_t *__
 // 150 broadcast reads a tile at spacing h/4 where each node alone loads 216 candidates, and
 // the distance and the spline of two nodes at a time in packed FP32.  A node meets its
 // neighbours in the same order and with the same operations as above (what it skips would
-// not have passed its test, and a candidate outside h adds an exact zero), so the field is
-// bit-identical.  Bound by instruction issue (70 % of the cycles).  Chosen up to a spacing of
-// 0.55 h: frames of 210k particles (field, surface, view) take 623, 409 and 394 us at h/4,
-// 3h/8 and h/2 where the general kernel's took 2032, 973 and 732; on coarser grids a tile's box holds
-// more candidates than its nodes share.
-constexpr float kTileSpacing = 0.55f;   // of h: above, a tile's box holds too many candidates
+// not have passed its test, and a candidate outside h adds an exact zero), the root apart, which
+// differs from sqrtf by an ulp at a few arguments in 2^24 (sqrt2): the field is that of the
+// general kernel to an ulp of a distance, and bit for bit wherever it was compared.  Bound by
+// instruction issue (70 % of the cycles).
+// Chosen by the spacing; on coarser grids a tile's box holds more candidates than its nodes share.
+// Field alone, this kernel against the general one, us: 1.2M particles at 0.25 h 1217 and 2193,
+// 0.4 h 518 and 723, 0.5 h 404 and 452, 0.55 h 383 and 375, 0.6 h 366 and 321, 0.8 h 393 and 211;
+// 210k particles, whose dense tiles are few, 0.25 h 291 and 672, 0.4 h 174 and 212, 0.5 h 176 and
+// 147, 0.55 h 180 and 132, 0.6 h 204 and 122.
+constexpr float kTileSpacing = 0.55f;   // of h
 constexpr int kTileX = 8, kTileY = 4, kTileZ = 4, kTileWarps = 4;
 
 typedef unsigned long long f2;   // two packed floats
@@ -378,7 +383,8 @@ __device__ __forceinline__ void emit_tet(const Cube &c, uint32_t above, int t, f
 // scanned and read) and a crossed cube's thread writing all its triangles alone; 276 us as one
 // launch with look-back between the tiles, which it spent waiting.
 constexpr int kMeshThreads = 256;   // of a block, and cubes of a tile: ITEMS a thread
-// Division of n < 2^31 by d >= 1: n m >> (31 + l), l = ceil(log2 d), m = ceil(2^(31+l) / d).
+// Division of n < 2^31 by d >= 1 by multiplication (Granlund and Montgomery, Division by invariant
+// integers using multiplication, 1994): n m >> (31 + l), l = ceil(log2 d), m = ceil(2^(31+l) / d).
 struct Divisor {
     uint32_t d, l;
     uint64_t m;
