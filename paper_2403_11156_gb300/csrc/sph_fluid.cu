@@ -131,8 +131,9 @@ __global__ void k_step_begin(Ptrs P)
 // drops those that fail from the list in place, and sums: list, counts and sums are those of
 // the exact test on every candidate, in the same order.
 //
-// A particle whose passed candidates exceed the list, or that has left the range the filter
-// holds for (SceneDev::qreach), takes the exact predicate over its rows instead.
+// A particle whose passed candidates exceed the list takes the exact predicate on what passes the
+// filter, from the first row on; one that has left the range the filter holds for
+// (SceneDev::qreach) takes it on every candidate.
 //
 // Between the phases a thread keeps its first kStage passed candidates in shared memory: written
 // straight to the list, whose entries the lanes of a warp reach at different times, each store
@@ -142,7 +143,12 @@ __global__ void k_step_begin(Ptrs P)
 // Bound by instruction issue and gather latency in turn: at 500k particles 146 us (167 with the
 // exact predicate on every candidate and boundary rows looked up by all, 154 without the stage),
 // 1.2M with bodies 343 us (396, 356).  24 staged candidates, which 28 neighbours overrun, take 153
-// and 355.  With two and four lanes the lists are built here and the lanes only sum: 100k particles
+// and 355.  Past the stage the list is read four entries ahead: particles twice as dense (60
+// neighbours, 500k) 611 -> 505 us a step; with the exact predicate on every candidate it was 472.
+// Where lists overrun (an error to the caller) or hold hundreds, the exact predicate alone was faster:
+// 110 neighbours in lists of 96 864 us, here 1200 (1540 before the second pass went by the filter),
+// 240 in lists of 512 351 (100k particles) and 505 (656 before).
+// With two and four lanes the lists are built here and the lanes only sum: 100k particles
 // 160 -> 59 us.
 __device__ __forceinline__ uint32_t query_pair(uint32_t word, uint32_t odd)
 {
@@ -156,26 +162,97 @@ struct Stencil {
     int32_t ny, nz, centre;  // rows a layer, layers, number of the particle's own row
 };
 
-// The exact predicate over the stencil: writes the list, returns the neighbour count.
-__device__ __noinline__ int exact_list(const Ptrs &P, const Stencil &st, int64_t i, float4 pi, float h2, int cap)
+// The filter's query: the particle's own coordinates and the threshold (a pair of halves each).
+struct Query {
+    uint32_t x, y, z, thr;
+    __device__ __forceinline__ Query(const Ptrs &P, const SceneDev &sc, uint32_t i) : thr(sc.qthr)
+    {
+        const uint4 own = P.qpos[i >> 1];
+        x = query_pair(own.x, i & 1u);
+        y = query_pair(own.y, i & 1u);
+        z = query_pair(own.z, i & 1u);
+    }
+};
+
+// Candidates c0, ... c0 + n - 1 (c0 even, n <= 32), eight at a time; a bit set: farther than h.
+__device__ __forceinline__ uint32_t far_bits(const uint4 *qpos, uint32_t c0, uint32_t n, const Query &c)
 {
+    const __half2 thr = as_half2(c.thr), unit = __float2half2_rn(1.0f / 512.0f), bias = __float2half2_rn(-3.0f);
+    uint32_t far = 0u;
+    const uint4 *w = qpos + (c0 >> 1);
+    for (uint32_t q = 0u; q < n; q += 8u, w += 4) {
+        uint4 p[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) p[u] = __ldg(w + u);
+        int bits = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const __half2 dx = __hfma2(as_half2(c.x + p[u].x), unit, bias);
+            const __half2 dy = __hfma2(as_half2(c.y + p[u].y), unit, bias);
+            const __half2 dz = __hfma2(as_half2(c.z + p[u].z), unit, bias);
+            const uint32_t f = __hgt2_mask(__hfma2(dx, dx, __hfma2(dy, dy, __hmul2(dz, dz))), thr);
+            // bytes 0 and 2 of the masks (-1 or 0) times -4^u and -2 4^u: bits 2u, 2u + 1
+            bits = __dp4a((int)f, (int)((uint32_t)(uint8_t)(-(1 << (2 * u))) | (uint32_t)(uint8_t)(-(2 << (2 * u))) << 16), bits);
+        }
+        far |= (uint32_t)bits << q;
+    }
+    return far;
+}
+
+// The exact predicate over the stencil, on the candidates that pass the filter or (out of its
+// reach) on all, loads four at a time: writes the list, returns the neighbour count.
+constexpr int kStage = 32;   // candidates a thread keeps in shared memory between the phases
+__device__ __noinline__ int exact_list(const Ptrs &P, const SceneDev &sc, const Stencil &st, int64_t i, float4 pi, bool filtered)
+{
+    const Query query(P, sc, (uint32_t)i);
+    const float h2 = sc.h2;
+    const int cap = sc.cap_f;
     int n = 0;
-    for (int32_t k = 0, y = 0, z = 0; k < st.ny * st.nz; ++k) {
-        const uint32_t row = st.row + (uint32_t)y * st.dx + (uint32_t)z * st.dxy;
-        if (++y == st.ny) { y = 0; ++z; }
-        const uint32_t je = P.cell_start[row + (uint32_t)st.x1 + 1u];
-        for (uint32_t j = P.cell_start[row + (uint32_t)st.x0]; j < je; ++j) {
-            float dx, dy, dz;
-            if (j != (uint32_t)i && pred_d2(pi, __ldg(P.pos_s + j), dx, dy, dz) < h2) {
-                if (n < cap) P.nbr[(int64_t)n * P.NF + i] = (int32_t)j;
-                ++n;
+    auto test = [&](uint32_t j, float4 p) {
+        float dx, dy, dz;
+        if (j == (uint32_t)i || !(pred_d2(pi, p, dx, dy, dz) < h2)) return;
+        if (n < cap) P.nbr[(int64_t)n * P.NF + i] = (int32_t)j;
+        ++n;
+    };
+    for (int32_t k = 0; k < st.ny * st.nz; ++k) {
+        const uint32_t row = st.row + (uint32_t)(k % st.ny) * st.dx + (uint32_t)(k / st.ny) * st.dxy;
+        const uint32_t jb = P.cell_start[row + (uint32_t)st.x0], je = P.cell_start[row + (uint32_t)st.x1 + 1u];
+        if (!filtered) {
+            uint32_t j = jb;
+            for (; j + 3u < je; j += 4u) {
+                float4 p[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) p[u] = __ldg(P.pos_s + j + u);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) test(j + (uint32_t)u, p[u]);
+            }
+            for (; j < je; ++j) test(j, __ldg(P.pos_s + j));
+            continue;
+        }
+        for (uint32_t c0 = jb & ~1u; c0 < je; c0 += 32u) {
+            const uint32_t m = min(je - c0, 32u);
+            uint32_t near = ~far_bits(P.qpos, c0, m, query) & (0xffffffffu >> (32u - m));
+            if (c0 < jb) near &= ~1u;
+            while (near != 0u) {
+                uint32_t j[4];
+                float4 p[4];
+                bool is[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    is[u] = near != 0u;
+                    j[u] = is[u] ? c0 + (uint32_t)__ffs((int)near) - 1u : j[0];
+                    near &= near - 1u;
+                    p[u] = __ldg(P.pos_s + j[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (is[u]) test(j[u], p[u]);
             }
         }
     }
     return n;
 }
 
-constexpr int kStage = 32;   // candidates a thread keeps in shared memory between the phases
 template <bool SUM>
 __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ Ptrs P)
 {
@@ -211,44 +288,27 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
         }
         const uint32_t self = (uint32_t)i;
         int passed = 0;
+        const float away = fmaxf(fmaxf(fabsf(pi.x - sc.origin[0]), fabsf(pi.y - sc.origin[1])), fabsf(pi.z - sc.origin[2]));
         {
-            const uint4 own = P.qpos[self >> 1];
-            const uint32_t qx = query_pair(own.x, self & 1u), qy = query_pair(own.y, self & 1u),
-                           qz = query_pair(own.z, self & 1u);
-            const __half2 thr = as_half2(sc.qthr), unit = __float2half2_rn(1.0f / 512.0f), bias = __float2half2_rn(-3.0f);
-            const int32_t rows = st.ny * st.nz;
+            const Query query(P, sc, self);
+            const int32_t rows = away <= sc.qreach ? st.ny * st.nz : 0;
             uint32_t row = st.row;
             for (int32_t k = 0, y = 0; k < rows; ++k) {
                 const uint32_t jb = P.cell_start[row + (uint32_t)st.x0], je = P.cell_start[row + (uint32_t)st.x1 + 1u];
                 row += st.dx;
                 if (++y == st.ny) { y = 0; row += st.dxy - (uint32_t)st.ny * st.dx; }
-                // 32 candidates from an even index on, eight at a time; a bit set: farther than h
-                for (uint32_t c0 = jb & ~1u; c0 < je; c0 += 32u) {
+                for (uint32_t c0 = jb & ~1u; c0 < je; c0 += 32u) {   // from an even index on
                     const uint32_t n = min(je - c0, 32u);
-                    uint32_t far = 0u;
-                    const uint4 *w = P.qpos + (c0 >> 1);
-                    for (uint32_t q = 0u; q < n; q += 8u, w += 4) {
-                        uint4 p[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) p[u] = __ldg(w + u);
-                        int bits = 0;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const __half2 dx = __hfma2(as_half2(qx + p[u].x), unit, bias);
-                            const __half2 dy = __hfma2(as_half2(qy + p[u].y), unit, bias);
-                            const __half2 dz = __hfma2(as_half2(qz + p[u].z), unit, bias);
-                            const uint32_t f = __hgt2_mask(__hfma2(dx, dx, __hfma2(dy, dy, __hmul2(dz, dz))), thr);
-                            // bytes 0 and 2 of the masks (-1 or 0) times -4^u and -2 4^u: bits 2u, 2u + 1
-                            bits = __dp4a((int)f, (int)((uint32_t)(uint8_t)(-(1 << (2 * u))) | (uint32_t)(uint8_t)(-(2 << (2 * u))) << 16), bits);
-                        }
-                        far |= (uint32_t)bits << q;
-                    }
+                    const uint32_t far = far_bits(P.qpos, c0, n, query);
                     uint32_t near = ~far & (0xffffffffu >> (32u - n));
                     if (c0 < jb) near &= ~1u;
                     if (k == st.centre && self - c0 < 32u) near &= ~(1u << (self - c0));
                     int q = passed;
                     passed += __popc(near);
-                    if (passed > cap_f) near = 0u;   // the exact predicate builds the list instead
+                    if (passed > cap_f) {   // the exact predicate builds the list instead
+                        k = rows;
+                        break;
+                    }
                     for (; near != 0u; near &= near - 1u, ++q) {
                         const int32_t j = (int32_t)(c0 + (uint32_t)__ffs((int)near) - 1u);
                         if (q < kStage) s_list[q][threadIdx.x] = j;
@@ -273,19 +333,17 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
             }
         }
         int total = -1;   // exact count, where the list was built by the exact predicate
-        const float away = fmaxf(fmaxf(fabsf(pi.x - sc.origin[0]), fabsf(pi.y - sc.origin[1])), fabsf(pi.z - sc.origin[2]));
         if (passed > cap_f || !(away <= sc.qreach)) {
-            total = exact_list(P, st, i, pi, h2, cap_f);
+            total = exact_list(P, sc, st, i, pi, away <= sc.qreach);
             passed = min(total, cap_f);
         }
         // phase 2: the exact predicate, density, alpha and the warm-start gate
         const float4 vi = P.vel_s[i];
         const Spline sp(sc);
         float w_sum = 0.0f, s1x = 0.0f, s1y = 0.0f, s1z = 0.0f, s2 = 0.0f, div_l = 0.0f;
-        // the passed candidates are in shared memory (the rest, and a list built by the exact
-        // predicate, in the list itself, which is read ahead of where it is written)
-        const int staged = total < 0 ? kStage : 0;
-        auto candidate = [&](int k) { return k < staged ? s_list[k][threadIdx.x] : P.nbr[(int64_t)k * NF + i]; };
+        // the first passed candidates are in shared memory, the rest, and a list built by the exact
+        // predicate, in the list itself
+        const int staged = total < 0 ? min(passed, kStage) : 0;
         auto visit = [&](int32_t j, float4 pj) {
             float dx, dy2, dz2;
             const float d2 = pred_d2(pi, pj, dx, dy2, dz2);
@@ -304,15 +362,36 @@ __global__ void __launch_bounds__(kBlock, 9) k_density(const __grid_constant__ P
             }
         };
         int k = 0;
-        for (; k + 2 <= passed; k += 2) {
-            const int32_t j0 = candidate(k), j1 = candidate(k + 1);
+        for (; k + 2 <= staged; k += 2) {
+            const int32_t j0 = s_list[k][threadIdx.x], j1 = s_list[k + 1][threadIdx.x];
             const float4 p0 = __ldg(P.pos_s + j0), p1 = __ldg(P.pos_s + j1);
             visit(j0, p0);
             visit(j1, p1);
         }
-        if (k < passed) {
-            const int32_t j0 = candidate(k);
+        if (k < staged) {
+            const int32_t j0 = s_list[k][threadIdx.x];
             visit(j0, __ldg(P.pos_s + j0));
+        }
+        // (read four ahead of where the list is written; past its end the last entry again)
+        if (staged < passed) {
+            const int32_t *list = P.nbr + i;
+            int32_t j[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) j[u] = list[(int64_t)min(staged + u, passed - 1) * NF];
+            for (k = staged; k < passed; k += 4) {
+                int32_t next[4];
+                float4 p[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    p[u] = __ldg(P.pos_s + j[u]);
+                    next[u] = list[(int64_t)min(k + 4 + u, passed - 1) * NF];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (k + u < passed) visit(j[u], p[u]);
+                    j[u] = next[u];
+                }
+            }
         }
         const int nb = min(nn_b, cap_b);
         P.nnf[i] = nn_f;
